@@ -13,8 +13,7 @@
 #include <algorithm>
 #include <cstring>
 
-#include "bk_common.cuh"
-#include "bk_kernels.h"
+#include "blas_common.cuh"
 
 SysPart make_part(int nsys, const int* Ls) {
     SysPart p;
@@ -39,48 +38,8 @@ SysPart single_part(int L) { return make_part(1, &L); }
 
 namespace {
 
-// system owning column pair q (columns 2q, 2q + 1)
-__device__ __forceinline__ int sys_of_pair(const SysPart& p, int q) {
-    int lo = 0, hi = p.nsys - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (2 * q >= p.col0[mid]) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
-}
-
-// Runs of whole active systems, at most TILE_MAXP pairs each (a system has
-// at most 64 pairs): the unit a thread block of the Gram and update kernels
-// takes, so that every column it combines is in its own shared memory.
+// pairs of a tile of the any-size update kernel
 constexpr int TILE_MAXP = 64;
-struct PTiles {
-    int n;
-    int p0[BK_MAX_SYS];
-    int np[BK_MAX_SYS];
-};
-
-PTiles make_ptiles(const SysPart& p, int maxp = TILE_MAXP) {
-    PTiles t;
-    t.n = 0;
-    bool open = false;
-    for (int s = 0; s < p.nsys; ++s) {
-        const int q0 = p.col0[s] / 2, nq = (p.col0[s + 1] - p.col0[s]) / 2;
-        if (!((p.active >> s) & 1ull) || nq == 0) {
-            open = false;
-            continue;
-        }
-        if (open && t.np[t.n - 1] + nq <= maxp) {
-            t.np[t.n - 1] += nq;
-        } else {
-            t.p0[t.n] = q0;
-            t.np[t.n] = nq;
-            t.n++;
-            open = true;
-        }
-    }
-    return t;
-}
 
 // Site chunks of the reductions and updates: grid.y, independent of the
 // tiles so that per-chunk partial sums have a fixed row count for a lattice.
@@ -100,11 +59,6 @@ __device__ __forceinline__ void store_elem(const Field& f, int n, int k, int p, 
         ((float4*)f.data)[((size_t)n * 12 + k) * f.np + p] = make_float4(re.x, re.y, im.x, im.y);
     }
 }
-
-template <typename R2>
-struct CxPair {  // one spinor component of a column pair, arithmetic type
-    R2 re, im;
-};
 
 // ---------------------------------------------------------------- warp tiles
 //
@@ -146,158 +100,8 @@ __device__ __forceinline__ WLane wlane(const SysPart& p, int tp0, int tnp, int l
     return w;
 }
 
-template <typename R2>
-__device__ __forceinline__ CxPair<R2> shfl_pair(const CxPair<R2>& v, int src) {
-    CxPair<R2> o;
-    o.re.x = __shfl_sync(0xffffffffu, v.re.x, src);
-    o.re.y = __shfl_sync(0xffffffffu, v.re.y, src);
-    o.im.x = __shfl_sync(0xffffffffu, v.im.x, src);
-    o.im.y = __shfl_sync(0xffffffffu, v.im.y, src);
-    return o;
-}
-
-// Element (n, k, p) through the read-only data path, FP16 scale applied.
-// Only for operands that no thread of the kernel writes, or that the reading
-// thread alone writes after its one read.
-template <int P>
-__device__ __forceinline__ CxPair<typename Prec<P>::pair> ldg_elem(const Field& f, int n, int k, int p,
-                                                                    typename Prec<P>::pair sc) {
-    CxPair<typename Prec<P>::pair> v;
-    const size_t e = ((size_t)n * 12 + k) * f.np + p;
-    if constexpr (P == BK_FP64) {
-        const double2* q = (const double2*)f.data + 2 * e;
-        v.re = __ldg(q);
-        v.im = __ldg(q + 1);
-    } else if constexpr (P == BK_FP32) {
-        const float4 q = __ldg((const float4*)f.data + e);
-        v.re = make_float2(q.x, q.y);
-        v.im = make_float2(q.z, q.w);
-    } else {
-        const uint2 q = __ldg((const uint2*)f.data + e);
-        v.re = pmul(__half22float2(*reinterpret_cast<const __half2*>(&q.x)), sc);
-        v.im = pmul(__half22float2(*reinterpret_cast<const __half2*>(&q.y)), sc);
-    }
-    return v;
-}
-
-__device__ __forceinline__ float2 bcast(float v) { return make_float2(v, v); }
-__device__ __forceinline__ double2 bcast(double v) { return make_double2(v, v); }
-
-// ---------------------------------------------------------------- Gram, small systems
-//
-// G_s = A_s^H B_s (and G2_s = A_s^H B2_s with NB = 2) for systems of at most
-// MAXL columns over warp tiles; grid: (warp tiles, site chunks), GW_WARPS
-// warps per block on different sites.  A lane adds conj(A_i) B_j for its two
-// columns i and every column j of its system, the pairs of B shuffled in
-// from their lanes.  FP32 / FP16 products are summed in FP32 registers
-// (packed pairs over j) and moved every GS_FLUSH sites into the lane's own
-// FP64 accumulators in shared memory; the warps' accumulators are added at
-// the end and the site chunks in FP64 by the finishing kernel (fixed order).
-
-constexpr int GS_FLUSH = 8;
+constexpr int GS_FLUSH = 8;  // sites per FP32 sum
 constexpr int GW_WARPS = 8;
-
-template <int P, int NB, int MAXL>
-__global__ void __launch_bounds__(GW_WARPS * 32) k_gram_w(Field A, Field B0, Field B1, SysPart p, PTiles wt,
-                                                          double2* __restrict__ partial, int V, int nchunk) {
-    using R = typename Prec<P>::real;
-    using R2 = typename Prec<P>::pair;
-    constexpr int FL = P == BK_FP64 ? (1 << 30) : GS_FLUSH;
-    constexpr int NACC = NB * 2 * MAXL;
-    // [warp][entry][lane]: every lane its own entries, no two threads share one
-    extern __shared__ double2 gw_acc[];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int chunk = blockIdx.y;
-    const WLane L = wlane(p, wt.p0[blockIdx.x], wt.np[blockIdx.x], lane);
-    double2* my = gw_acc + (size_t)w * NACC * 32 + lane;
-#pragma unroll
-    for (int e = 0; e < NACC; ++e) my[e * 32] = make_double2(0.0, 0.0);
-    CxPair<R2> acc[NB][2][MAXL / 2];
-#pragma unroll
-    for (int b = 0; b < NB; ++b)
-#pragma unroll
-        for (int ii = 0; ii < 2; ++ii)
-#pragma unroll
-            for (int jp = 0; jp < MAXL / 2; ++jp) acc[b][ii][jp].re = acc[b][ii][jp].im = pzero<R2>();
-    const int iters = (V + GW_WARPS * nchunk - 1) / (GW_WARPS * nchunk);
-    for (int it = 0; it < iters; ++it) {
-        const int n = (it * nchunk + chunk) * GW_WARPS + w;
-        if (n < V) {  // the same for the whole warp
-            R2 sa = pzero<R2>(), sb[NB];
-            if (L.live) sa = pair_scale<P>(A, n, L.q);
-#pragma unroll
-            for (int b = 0; b < NB; ++b) sb[b] = L.live ? pair_scale<P>(b == 0 ? B0 : B1, n, L.q) : pzero<R2>();
-#pragma unroll 2
-            for (int k = 0; k < 12; ++k) {
-                CxPair<R2> a, bv[NB];
-                a.re = a.im = pzero<R2>();
-#pragma unroll
-                for (int b = 0; b < NB; ++b) bv[b].re = bv[b].im = pzero<R2>();
-                if (L.live) {
-                    a = ldg_elem<P>(A, n, k, L.q, sa);
-#pragma unroll
-                    for (int b = 0; b < NB; ++b) bv[b] = ldg_elem<P>(b == 0 ? B0 : B1, n, k, L.q, sb[b]);
-                }
-#pragma unroll
-                for (int b = 0; b < NB; ++b)
-#pragma unroll
-                    for (int jp = 0; jp < MAXL / 2; ++jp) {
-                        const CxPair<R2> bp = shfl_pair(bv[b], L.base + min(jp, L.nps - 1));
-                        if (jp < L.nps) {
-#pragma unroll
-                            for (int ii = 0; ii < 2; ++ii) {
-                                const R2 ar = bcast(ii ? a.re.y : a.re.x);
-                                const R2 ai = bcast(ii ? a.im.y : a.im.x);
-                                const R2 nai = bcast(ii ? -a.im.y : -a.im.x);
-                                CxPair<R2>& c = acc[b][ii][jp];
-                                c.re = pfma(ar, bp.re, c.re);
-                                c.re = pfma(ai, bp.im, c.re);
-                                c.im = pfma(ar, bp.im, c.im);
-                                c.im = pfma(nai, bp.re, c.im);
-                            }
-                        }
-                    }
-            }
-        }
-        if ((it % FL) == FL - 1 || it == iters - 1) {
-#pragma unroll
-            for (int b = 0; b < NB; ++b)
-#pragma unroll
-                for (int ii = 0; ii < 2; ++ii)
-#pragma unroll
-                    for (int jp = 0; jp < MAXL / 2; ++jp)
-#pragma unroll
-                        for (int jj = 0; jj < 2; ++jj) {
-                            double2& v = my[((b * 2 + ii) * MAXL + 2 * jp + jj) * 32];
-                            CxPair<R2>& c = acc[b][ii][jp];
-                            v.x += (double)(jj ? c.re.y : c.re.x);
-                            v.y += (double)(jj ? c.im.y : c.im.x);
-                        }
-#pragma unroll
-            for (int b = 0; b < NB; ++b)
-#pragma unroll
-                for (int ii = 0; ii < 2; ++ii)
-#pragma unroll
-                    for (int jp = 0; jp < MAXL / 2; ++jp) acc[b][ii][jp].re = acc[b][ii][jp].im = pzero<R2>();
-        }
-    }
-    __syncthreads();
-    if (w != 0 || !L.live) return;
-    const int ne = p.coef_off[p.nsys];
-    for (int b = 0; b < NB; ++b)
-        for (int ii = 0; ii < 2; ++ii) {
-            if (L.i0 + ii >= L.Ls) continue;
-            for (int j = 0; j < L.Ls; ++j) {
-                double2 v = make_double2(0.0, 0.0);
-                for (int ww = 0; ww < GW_WARPS; ++ww) {
-                    const double2 a = gw_acc[((size_t)ww * NACC + (b * 2 + ii) * MAXL + j) * 32 + lane];
-                    v.x += a.x;
-                    v.y += a.y;
-                }
-                partial[(size_t)(b * nchunk + chunk) * ne + p.coef_off[L.s] + (L.i0 + ii) * L.Ls + j] = v;
-            }
-        }
-}
 
 // ---------------------------------------------------------------- Gram, any system size
 //
@@ -414,120 +218,161 @@ __global__ void __launch_bounds__(256) k_gram_big(Field A, Field B, SysPart p, B
         }
 }
 
-// G[e] (and G2) = sum over chunks of the partial sums, for the entries of the
-// active systems (one thread per entry, fixed order: reproducible).
-__global__ void k_gram_finish(const double2* __restrict__ partial, int nchunk, int NB, SysPart p,
-                              double2* __restrict__ G, double2* __restrict__ G2) {
-    const int ne = p.coef_off[p.nsys];
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= NB * ne) return;
-    const int b = e / ne, el = e - b * ne;
-    int s = 0;
-    while (s + 1 < p.nsys && el >= p.coef_off[s + 1]) ++s;
-    if (!((p.active >> s) & 1ull)) return;
+// Sums over the chunks' partial rows: 32 entries x FIN_ROWS row slices per
+// block (a thread adds every FIN_ROWS-th row), combined in shared memory in a
+// fixed order.  One thread per entry over all rows took 75 us for 304 rows.
+constexpr int FIN_ROWS = 16;
+
+template <typename F>
+__device__ __forceinline__ double2 sum_rows(int nrows, bool on, F row) {
+    __shared__ double2 red[FIN_ROWS][32];
     double2 v = make_double2(0.0, 0.0);
-    for (int c = 0; c < nchunk; ++c) {
-        const double2 x = partial[(size_t)(b * nchunk + c) * ne + el];
-        v.x += x.x;
-        v.y += x.y;
+    if (on) {
+#pragma unroll 4
+        for (int c = threadIdx.y; c < nrows; c += FIN_ROWS) {
+            const double2 x = row(c);
+            v.x += x.x;
+            v.y += x.y;
+        }
     }
-    (b == 0 ? G : G2)[el] = v;
+    red[threadIdx.y][threadIdx.x] = v;
+    __syncthreads();
+    v = make_double2(0.0, 0.0);
+    if (threadIdx.y == 0)
+        for (int y = 0; y < FIN_ROWS; ++y) {
+            v.x += red[y][threadIdx.x].x;
+            v.y += red[y][threadIdx.x].y;
+        }
+    return v;  // valid in the threads of row 0
+}
+
+// G[e] (and G2) = sum over chunks of the partial sums, for the entries of the
+// active systems.
+__global__ void __launch_bounds__(32 * FIN_ROWS) k_gram_finish(const double2* __restrict__ partial, int nchunk, int NB,
+                                                              SysPart p, double2* __restrict__ G,
+                                                              double2* __restrict__ G2) {
+    const int ne = p.coef_off[p.nsys];
+    const int e = blockIdx.x * 32 + threadIdx.x;
+    const int b = e / ne, el = e - b * ne;
+    bool on = e < NB * ne;
+    if (on) {
+        int lo = 0, hi = p.nsys - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (el >= p.coef_off[mid]) lo = mid;
+            else hi = mid - 1;
+        }
+        on = (p.active >> lo) & 1ull;
+    }
+    const double2 v =
+        sum_rows(nchunk, on, [&](int c) { return __ldg(partial + (size_t)(b * nchunk + c) * ne + el); });
+    if (on && threadIdx.y == 0) (b == 0 ? G : G2)[el] = v;
 }
 
 // ---------------------------------------------------------------- column dots
 //
-// out[k][j] = (A_k)_j^H (B_k)_j over pairs [q0, q0 + nq).  Thread block: 32
-// pair slots x 8 site rows (a warp reads one contiguous row); grid: (pair
-// groups, site chunks).  Sums as in the Gram kernels; the 8 site rows are
-// combined in shared memory.
+// Over pairs [q0, q0 + nq), column by column: MODE 0: out[0] = A^H B, 1:
+// out[0] = |A|^2, 2: out[0] = A^H B and out[1] = |A|^2 (one read of A).
+// Thread block: TX pair slots x 256 / TX rows (site, component); grid: (pair
+// groups, row chunks).  Rows, not sites: 12 times the parallelism, which the
+// small lattices need.  UR rows per thread are loaded before any is used.
+// Sums as in the Gram kernels.
 
-template <int P, int NPAIR, int TX>
-__global__ void __launch_bounds__(256) k_coldot(Field A0, Field B0, Field A1, Field B1, int q0, int nq,
-                                                double2* __restrict__ partial, int V, int nchunk) {
+template <int P, int MODE, int TX>
+__global__ void __launch_bounds__(256) k_coldot(Field A, Field B, int q0, int nq, double2* __restrict__ partial,
+                                                unsigned rows, int nchunk) {
     using R = typename Prec<P>::real;
     using R2 = typename Prec<P>::pair;
-    constexpr int TY = 256 / TX;  // site rows: narrow column ranges get more sites per block
-    constexpr int FL = P == BK_FP64 ? (1 << 30) : GS_FLUSH;
-    __shared__ double2 red[TY][TX][NPAIR * 2];
+    constexpr int TY = 256 / TX;  // rows: narrow column ranges get more of them per block
+    constexpr int NOUT = MODE == 2 ? 2 : 1;
+    constexpr int UR = P == BK_FP64 ? 2 : 4;
+    __shared__ double2 red[TY][TX][NOUT * 2];
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ql = blockIdx.x * TX + tx, q = q0 + ql;
     const bool on = ql < nq;
-    const int chunk = blockIdx.y;
-    cx<R> acc[NPAIR][2];
-    double2 acc64[NPAIR][2];
+    const int chunk = blockIdx.y, np = A.np;
+    R2 dr = pzero<R2>(), di = dr, nn = dr;
+    double2 d0 = make_double2(0.0, 0.0), d1 = d0, n01 = d0;
+    auto flush = [&]() {
+        d0 = make_double2(d0.x + (double)dr.x, d0.y + (double)di.x);
+        d1 = make_double2(d1.x + (double)dr.y, d1.y + (double)di.y);
+        n01 = make_double2(n01.x + (double)nn.x, n01.y + (double)nn.y);
+        dr = di = nn = pzero<R2>();
+    };
+    int since = 0;
+    const unsigned step = (unsigned)nchunk * TY;
+    for (unsigned r0 = (unsigned)chunk * TY + ty; r0 < rows; r0 += step * UR) {
+        CxPair<R2> a[UR], b[UR];
 #pragma unroll
-    for (int kk = 0; kk < NPAIR; ++kk)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            acc[kk][h] = mk(R(0), R(0));
-            acc64[kk][h] = make_double2(0.0, 0.0);
-        }
-    const int iters = (V + TY * nchunk - 1) / (TY * nchunk);
-    for (int it = 0; it < iters; ++it) {
-        const int n = (it * nchunk + chunk) * TY + ty;
-        if (on && n < V) {
-#pragma unroll
-            for (int kk = 0; kk < NPAIR; ++kk) {
-                R2 ar[12], ai[12], br[12], bi[12];
-                load_pair<P>(kk == 0 ? A0 : A1, n, q, ar, ai);
-                load_pair<P>(kk == 0 ? B0 : B1, n, q, br, bi);
-#pragma unroll
-                for (int k = 0; k < 12; ++k) {
-                    acc[kk][0].r = fma(ar[k].x, br[k].x, acc[kk][0].r);
-                    acc[kk][0].r = fma(ai[k].x, bi[k].x, acc[kk][0].r);
-                    acc[kk][0].i = fma(ar[k].x, bi[k].x, acc[kk][0].i);
-                    acc[kk][0].i = fma(-ai[k].x, br[k].x, acc[kk][0].i);
-                    acc[kk][1].r = fma(ar[k].y, br[k].y, acc[kk][1].r);
-                    acc[kk][1].r = fma(ai[k].y, bi[k].y, acc[kk][1].r);
-                    acc[kk][1].i = fma(ar[k].y, bi[k].y, acc[kk][1].i);
-                    acc[kk][1].i = fma(-ai[k].y, br[k].y, acc[kk][1].i);
+        for (int x = 0; x < UR; ++x) {
+            const unsigned r = r0 + x * step;
+            a[x] = b[x] = cp_zero<R2>();
+            if (on && r < rows) {
+                R2 sa = pzero<R2>(), sb = sa;
+                if constexpr (P == BK_FP16) {
+                    sa = pair_scale<P>(A, r / 12, q);
+                    if (MODE != 1) sb = pair_scale<P>(B, r / 12, q);
                 }
+                a[x] = ldg_at<P>(A, (size_t)r * np + q, sa);
+                if (MODE != 1) b[x] = ldg_at<P>(B, (size_t)r * np + q, sb);
             }
         }
-        if ((it % FL) == FL - 1 || it == iters - 1) {
 #pragma unroll
-            for (int kk = 0; kk < NPAIR; ++kk)
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    acc64[kk][h].x += (double)acc[kk][h].r;
-                    acc64[kk][h].y += (double)acc[kk][h].i;
-                    acc[kk][h] = mk(R(0), R(0));
-                }
+        for (int x = 0; x < UR; ++x) {
+            if (MODE != 1) {
+                dr = pfma(a[x].re, b[x].re, dr);
+                dr = pfma(a[x].im, b[x].im, dr);
+                di = pfma(a[x].re, b[x].im, di);
+                R2 nai;
+                nai.x = -a[x].im.x;
+                nai.y = -a[x].im.y;
+                di = pfma(nai, b[x].re, di);
+            }
+            if (MODE != 0) {
+                nn = pfma(a[x].re, a[x].re, nn);
+                nn = pfma(a[x].im, a[x].im, nn);
+            }
+        }
+        if constexpr (P != BK_FP64) {
+            since += UR;
+            if (since >= ROW_FLUSH) {
+                flush();
+                since = 0;
+            }
         }
     }
-#pragma unroll
-    for (int kk = 0; kk < NPAIR; ++kk)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) red[ty][tx][kk * 2 + h] = acc64[kk][h];
+    flush();
+    if (MODE != 1) {
+        red[ty][tx][0] = d0;
+        red[ty][tx][1] = d1;
+    }
+    if (MODE != 0) {
+        red[ty][tx][NOUT * 2 - 2] = make_double2(n01.x, 0.0);
+        red[ty][tx][NOUT * 2 - 1] = make_double2(n01.y, 0.0);
+    }
     __syncthreads();
-    if (ty == 0 && on) {
-#pragma unroll
-        for (int kk = 0; kk < NPAIR; ++kk)
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                double2 v = make_double2(0.0, 0.0);
-                for (int y = 0; y < TY; ++y) {
-                    v.x += red[y][tx][kk * 2 + h].x;
-                    v.y += red[y][tx][kk * 2 + h].y;
-                }
-                partial[((size_t)chunk * NPAIR + kk) * (2 * nq) + 2 * ql + h] = v;
-            }
+    for (int t = ty * TX + tx; t < TX * NOUT * 2; t += 256) {
+        const int c = t % (NOUT * 2), x = t / (NOUT * 2), qx = blockIdx.x * TX + x;
+        if (qx >= nq) continue;
+        double2 v = make_double2(0.0, 0.0);
+        for (int y = 0; y < TY; ++y) {
+            v.x += red[y][x][c].x;
+            v.y += red[y][x][c].y;
+        }
+        partial[((size_t)chunk * NOUT + (c >> 1)) * (2 * nq) + 2 * qx + (c & 1)] = v;
     }
 }
 
 // out[kk * ldo + j] = sum over chunks, columns j < n
-__global__ void k_coldot_finish(const double2* __restrict__ partial, int nchunk, int npair, int nq, int n,
-                                double2* __restrict__ out, int ldo) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= npair * n) return;
+__global__ void __launch_bounds__(32 * FIN_ROWS) k_coldot_finish(const double2* __restrict__ partial, int nchunk,
+                                                                int npair, int nq, int n, double2* __restrict__ out,
+                                                                int ldo) {
+    const int e = blockIdx.x * 32 + threadIdx.x;
+    const bool on = e < npair * n;
     const int kk = e / n, j = e - kk * n;
-    double2 v = make_double2(0.0, 0.0);
-    for (int c = 0; c < nchunk; ++c) {
-        const double2 x = partial[((size_t)c * npair + kk) * (2 * nq) + j];
-        v.x += x.x;
-        v.y += x.y;
-    }
-    out[(size_t)kk * ldo + j] = v;
+    const double2 v = sum_rows(
+        nchunk, on, [&](int c) { return __ldg(partial + ((size_t)c * npair + kk) * (2 * nq) + j); });
+    if (on && threadIdx.y == 0) out[(size_t)kk * ldo + j] = v;
 }
 
 // ---------------------------------------------------------------- fused block update
@@ -545,29 +390,6 @@ __global__ void k_coldot_finish(const double2* __restrict__ partial, int nchunk,
 // path, then writes its pair of Y and X.  Optionally the squared norms of
 // the Y columns are summed per chunk (the residual norms of the stopping
 // rule come with the R update).
-
-template <int P>
-__device__ __forceinline__ cx<typename Prec<P>::real> coef(const double* ptr, double mult, int s) {
-    using R = typename Prec<P>::real;
-    if (ptr) return mk((R)(mult * ptr[2 * s]), (R)(mult * ptr[2 * s + 1]));
-    return mk((R)mult, R(0));
-}
-
-// acc (pair) += c (complex scalar) * v (pair)
-template <typename R, typename R2>
-__device__ __forceinline__ void cpair_mac(CxPair<R2>& acc, cx<R> c, const CxPair<R2>& v) {
-    R2 cr, ci, nci;
-    cr.x = c.r;
-    cr.y = c.r;
-    ci.x = c.i;
-    ci.y = c.i;
-    nci.x = -c.i;
-    nci.y = -c.i;
-    acc.re = pfma(cr, v.re, acc.re);
-    acc.re = pfma(nci, v.im, acc.re);
-    acc.im = pfma(cr, v.im, acc.im);
-    acc.im = pfma(ci, v.re, acc.im);
-}
 
 // FP16 elements come with a per-(site, pair) scale: load_scaled applies it.
 template <int P>
@@ -755,69 +577,15 @@ __global__ void __launch_bounds__(256) k_genop(const __grid_constant__ GenOp g, 
 // NE and HX fix the operand counts of the hot updates at compile time (-1:
 // taken from the GenOp); every operand has the layout's pair count np, so
 // one element offset serves them all.
-template <int P>
-__device__ __forceinline__ CxPair<typename Prec<P>::pair> ldg_at(const Field& f, size_t e,
-                                                                  typename Prec<P>::pair sc) {
-    CxPair<typename Prec<P>::pair> v;
-    if constexpr (P == BK_FP64) {
-        const double2* q = (const double2*)f.data + 2 * e;
-        v.re = __ldg(q);
-        v.im = __ldg(q + 1);
-    } else if constexpr (P == BK_FP32) {
-        const float4 q = __ldg((const float4*)f.data + e);
-        v.re = make_float2(q.x, q.y);
-        v.im = make_float2(q.z, q.w);
-    } else {
-        const uint2 q = __ldg((const uint2*)f.data + e);
-        v.re = pmul(__half22float2(*reinterpret_cast<const __half2*>(&q.x)), sc);
-        v.im = pmul(__half22float2(*reinterpret_cast<const __half2*>(&q.y)), sc);
-    }
-    return v;
-}
-
-template <int P>
-__device__ __forceinline__ CxPair<typename Prec<P>::pair> load_at(const Field& f, size_t e) {
-    CxPair<typename Prec<P>::pair> v;
-    if constexpr (P == BK_FP64) {
-        const double2* q = (const double2*)f.data + 2 * e;
-        v.re = q[0];
-        v.im = q[1];
-    } else {
-        static_assert(P == BK_FP32, "accumulators are FP32 or FP64");
-        const float4 q = ((const float4*)f.data)[e];
-        v.re = make_float2(q.x, q.y);
-        v.im = make_float2(q.z, q.w);
-    }
-    return v;
-}
-
-template <int P>
-__device__ __forceinline__ void store_at(const Field& f, size_t e, typename Prec<P>::pair re,
-                                         typename Prec<P>::pair im) {
-    if constexpr (P == BK_FP64) {
-        double2* q = (double2*)f.data + 2 * e;
-        q[0] = re;
-        q[1] = im;
-    } else {
-        static_assert(P == BK_FP32, "element stores are for FP32 / FP64 blocks");
-        ((float4*)f.data)[e] = make_float4(re.x, re.y, im.x, im.y);
-    }
-}
-
-template <int P, int MAXL, int UK, int MINB, int NMI, int NE, int HX>
-__global__ void __launch_bounds__(GW_WARPS * 32, MINB) k_genop_w(const __grid_constant__ GenOp g, PTiles wt, int V,
-                                                                 int nchunk, int ncols, int np) {
-    using R = typename Prec<P>::real;
-    using R2 = typename Prec<P>::pair;
-    constexpr int XP = P == BK_FP64 ? BK_FP64 : BK_FP32;
-    using XR = typename Prec<XP>::real;
-    using X2 = typename Prec<XP>::pair;
-    static_assert(12 % UK == 0, "components per step divide 12");
-    constexpr int MMI = NMI >= 0 ? NMI : GENOP_MAXMI;
-    constexpr int ME = NE >= 0 ? NE : GENOP_MAXE;
-    const int nmi = NMI >= 0 ? NMI : g.nmi;
-    const int ne = NE >= 0 ? NE : g.ne;
-    const bool hx = HX >= 0 ? HX != 0 : g.hasX != 0;
+template <int MAXL>
+__global__ void __launch_bounds__(GW_WARPS * 32) k_genop_w(const __grid_constant__ GenOp g, PTiles wt, int V,
+                                                          int nchunk, int ncols, int np) {
+    constexpr int P = BK_FP16, XP = BK_FP32;
+    using R = float;
+    using R2 = float2;
+    constexpr int MMI = GENOP_MAXMI, ME = GENOP_MAXE;
+    const int nmi = g.nmi, ne = g.ne;
+    const bool hx = g.hasX != 0;
     __shared__ double2 ynred[GW_WARPS][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int chunk = blockIdx.y;
@@ -825,7 +593,7 @@ __global__ void __launch_bounds__(GW_WARPS * 32, MINB) k_genop_w(const __grid_co
     const bool act = L.live && !(g.skip && g.skip[L.s]);
     const int s = L.s;
     const bool mat = nmi > 0 && g.M != nullptr && ((g.hasY && g.ym != 0.0) || (hx && g.xm != 0.0));
-    cx<R> ea[ME > 0 ? ME : 1], ma[MMI > 0 ? MMI : 1], xa = mk(R(0), R(0));
+    cx<R> ea[ME], ma[MMI], xa = mk(R(0), R(0));
 #pragma unroll
     for (int e = 0; e < ME; ++e) ea[e] = e < ne ? coef<P>(g.ea[e], g.ea_mult[e], s) : mk(R(0), R(0));
 #pragma unroll
@@ -850,114 +618,80 @@ __global__ void __launch_bounds__(GW_WARPS * 32, MINB) k_genop_w(const __grid_co
         }
     }
     const R2 ym2 = bcast((R)g.ym);
-    const X2 xm2 = bcast((XR)g.xm);
-    const cx<XR> xax = mk((XR)xa.r, (XR)xa.i);
+    const R2 xm2 = bcast((R)g.xm);
     double yn0 = 0.0, yn1 = 0.0;
     const int iters = (V + GW_WARPS * nchunk - 1) / (GW_WARPS * nchunk);
     for (int it = 0; it < iters; ++it) {
         const int n = (it * nchunk + chunk) * GW_WARPS + w;
         if (n >= V) break;  // the same for the whole warp
-        R2 msc[MMI > 0 ? MMI : 1], esc[ME > 0 ? ME : 1], xsc = pzero<R2>();
+        R2 msc[MMI], esc[ME], xsc = pzero<R2>();
 #pragma unroll
         for (int u = 0; u < MMI; ++u) msc[u] = act && u < nmi ? pair_scale<P>(g.Mi[u], n, L.q) : pzero<R2>();
 #pragma unroll
         for (int e = 0; e < ME; ++e) esc[e] = act && e < ne ? pair_scale<P>(g.E[e], n, L.q) : pzero<R2>();
         if (act && hx) xsc = pair_scale<P>(g.Xin, n, L.q);
-        R2 yr[P == BK_FP16 ? 12 : 1], yi[P == BK_FP16 ? 12 : 1];
+        R2 yr[12], yi[12];
         R sa = R(0), sb = R(0);
         const size_t e0 = (size_t)n * 12 * np + L.q;
-        // FP16 keeps the site's 12 components in registers for the scaled store
-        constexpr int K0U = P == BK_FP16 ? 12 / UK : 1;
-#pragma unroll K0U
-        for (int k0 = 0; k0 < 12; k0 += UK) {
-            CxPair<R2> vm[UK][MMI > 0 ? MMI : 1], ve[UK][ME > 0 ? ME : 1], vx[UK];
-            CxPair<X2> xo[UK];
+        // the site's 12 components stay in registers for the scaled store
 #pragma unroll
-            for (int uk = 0; uk < UK; ++uk) {
-                const size_t e = e0 + (size_t)(k0 + uk) * np;
+        for (int k = 0; k < 12; ++k) {
+            const size_t e = e0 + (size_t)k * np;
+            CxPair<R2> vm[MMI], ve[ME], vx = cp_zero<R2>(), x = cp_zero<R2>();
+#pragma unroll
+            for (int u = 0; u < MMI; ++u)
+                vm[u] = act && mat && u < nmi ? ldg_at<P>(g.Mi[u], e, msc[u]) : cp_zero<R2>();
+#pragma unroll
+            for (int t = 0; t < ME; ++t) ve[t] = act && g.hasY && t < ne ? ldg_at<P>(g.E[t], e, esc[t]) : cp_zero<R2>();
+            if (act && hx) {
+                vx = ldg_at<P>(g.Xin, e, xsc);
+                x = load_at<XP>(g.X, e);
+            }
+            CxPair<R2> mp = cp_zero<R2>();
+            if (mat) {
+                CxPair<R2> c = cp_zero<R2>();
 #pragma unroll
                 for (int u = 0; u < MMI; ++u)
-                    vm[uk][u] = act && mat && u < nmi ? ldg_at<P>(g.Mi[u], e, msc[u])
-                                                      : CxPair<R2>{pzero<R2>(), pzero<R2>()};
+                    if (u < nmi) cpair_mac<R, R2>(c, ma[u], vm[u]);
 #pragma unroll
-                for (int t = 0; t < ME; ++t)
-                    ve[uk][t] = act && g.hasY && t < ne ? ldg_at<P>(g.E[t], e, esc[t])
-                                                        : CxPair<R2>{pzero<R2>(), pzero<R2>()};
-                vx[uk].re = vx[uk].im = pzero<R2>();
-                xo[uk].re = xo[uk].im = pzero<X2>();
-                if (act && hx) {
-                    vx[uk] = ldg_at<P>(g.Xin, e, xsc);
-                    xo[uk] = load_at<XP>(g.X, e);
-                }
-            }
+                for (int ip = 0; ip < MAXL / 2; ++ip) {
+                    const CxPair<R2> cp = shfl_pair(c, L.base + min(ip, L.nps - 1));
+                    if (ip < L.nps) {
 #pragma unroll
-            for (int uk = 0; uk < UK; ++uk) {
-                const int k = k0 + uk;
-                const size_t e = e0 + (size_t)k * np;
-                CxPair<R2> mp;
-                mp.re = mp.im = pzero<R2>();
-                if (mat) {
-                    CxPair<R2> c;
-                    c.re = c.im = pzero<R2>();
-#pragma unroll
-                    for (int u = 0; u < MMI; ++u)
-                        if (u < nmi) cpair_mac<R, R2>(c, ma[u], vm[uk][u]);
-#pragma unroll
-                    for (int ip = 0; ip < MAXL / 2; ++ip) {
-                        const CxPair<R2> cp = shfl_pair(c, L.base + min(ip, L.nps - 1));
-                        if (ip < L.nps) {
-#pragma unroll
-                            for (int h = 0; h < 2; ++h) {
-                                const R2 cr = bcast(h ? cp.re.y : cp.re.x), ci = bcast(h ? cp.im.y : cp.im.x);
-                                const R2 nci = bcast(h ? -cp.im.y : -cp.im.x);
-                                mp.re = pfma(cr, Mr[2 * ip + h], mp.re);
-                                mp.re = pfma(nci, Mi[2 * ip + h], mp.re);
-                                mp.im = pfma(cr, Mi[2 * ip + h], mp.im);
-                                mp.im = pfma(ci, Mr[2 * ip + h], mp.im);
-                            }
+                        for (int h = 0; h < 2; ++h) {
+                            const R2 cr = bcast(h ? cp.re.y : cp.re.x), ci = bcast(h ? cp.im.y : cp.im.x);
+                            const R2 nci = bcast(h ? -cp.im.y : -cp.im.x);
+                            mp.re = pfma(cr, Mr[2 * ip + h], mp.re);
+                            mp.re = pfma(nci, Mi[2 * ip + h], mp.re);
+                            mp.im = pfma(cr, Mi[2 * ip + h], mp.im);
+                            mp.im = pfma(ci, Mr[2 * ip + h], mp.im);
                         }
                     }
                 }
-                if (!act) continue;
-                if (g.hasY) {
-                    CxPair<R2> y;
-                    y.re = pmul(ym2, mp.re);
-                    y.im = pmul(ym2, mp.im);
+            }
+            if (!act) continue;
+            if (g.hasY) {
+                CxPair<R2> y;
+                y.re = pmul(ym2, mp.re);
+                y.im = pmul(ym2, mp.im);
 #pragma unroll
-                    for (int t = 0; t < ME; ++t)
-                        if (t < ne) cpair_mac<R, R2>(y, ea[t], ve[uk][t]);
-                    if (g.ynorm) {
-                        sa = fma(y.re.x, y.re.x, sa);
-                        sa = fma(y.im.x, y.im.x, sa);
-                        sb = fma(y.re.y, y.re.y, sb);
-                        sb = fma(y.im.y, y.im.y, sb);
-                    }
-                    if constexpr (P == BK_FP16) {
-                        yr[k] = y.re;
-                        yi[k] = y.im;
-                    } else {
-                        store_at<P>(g.Y, e, y.re, y.im);
-                    }
+                for (int t = 0; t < ME; ++t)
+                    if (t < ne) cpair_mac<R, R2>(y, ea[t], ve[t]);
+                if (g.ynorm) {
+                    sa = fma(y.re.x, y.re.x, sa);
+                    sa = fma(y.im.x, y.im.x, sa);
+                    sb = fma(y.re.y, y.re.y, sb);
+                    sb = fma(y.im.y, y.im.y, sb);
                 }
-                if (hx) {
-                    CxPair<X2> x = xo[uk], v;
-                    v.re.x = vx[uk].re.x;
-                    v.re.y = vx[uk].re.y;
-                    v.im.x = vx[uk].im.x;
-                    v.im.y = vx[uk].im.y;
-                    cpair_mac<XR, X2>(x, xax, v);
-                    X2 mr, mi;
-                    mr.x = mp.re.x;
-                    mr.y = mp.re.y;
-                    mi.x = mp.im.x;
-                    mi.y = mp.im.y;
-                    store_at<XP>(g.X, e, pfma(xm2, mr, x.re), pfma(xm2, mi, x.im));
-                }
+                yr[k] = y.re;
+                yi[k] = y.im;
+            }
+            if (hx) {
+                cpair_mac<R, R2>(x, xa, vx);
+                store_at<XP>(g.X, e, pfma(xm2, mp.re, x.re), pfma(xm2, mp.im, x.im));
             }
         }
-        if constexpr (P == BK_FP16) {
-            if (act && g.hasY) store_pair<P>(g.Y, n, L.q, yr, yi);
-        }
+        if (act && g.hasY) store_pair<P>(g.Y, n, L.q, yr, yi);
         yn0 += (double)sa;
         yn1 += (double)sb;
     }
@@ -976,14 +710,16 @@ __global__ void __launch_bounds__(GW_WARPS * 32, MINB) k_genop_w(const __grid_co
     }
 }
 
-__global__ void k_norm_finish(const double* __restrict__ part, int nrows, int ncols, int c0, int n,
-                              double* __restrict__ out) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    double v = 0.0;
-    for (int b = 0; b < nrows; ++b) v += part[(size_t)b * ncols + c0 + j];
-    out[2 * (c0 + j)] = v;
-    out[2 * (c0 + j) + 1] = 0.0;
+__global__ void __launch_bounds__(32 * FIN_ROWS) k_norm_finish(const double* __restrict__ part, int nrows, int ncols,
+                                                              int c0, int n, double* __restrict__ out) {
+    const int j = blockIdx.x * 32 + threadIdx.x;
+    const bool on = j < n;
+    const double2 v = sum_rows(
+        nrows, on, [&](int c) { return make_double2(__ldg(part + (size_t)c * ncols + c0 + j), 0.0); });
+    if (on && threadIdx.y == 0) {
+        out[2 * (c0 + j)] = v.x;
+        out[2 * (c0 + j) + 1] = 0.0;
+    }
 }
 
 // X64 += Xlo; Xlo = 0 over pairs [p0, p0 + np)
@@ -1334,29 +1070,9 @@ __global__ void __launch_bounds__(256) k_chol_inv(const double2* __restrict__ S,
 
 namespace {
 
-constexpr int GS_MAXL = 12;   // largest system of the small-system Gram kernel
-constexpr int GS2_MAXL = 6;   // ... of its fused two-output form
-
-int max_active_L(const SysPart& p) {
-    int m = 0;
-    for (int s = 0; s < p.nsys; ++s)
-        if ((p.active >> s) & 1ull) m = std::max(m, p.L[s]);
-    return m;
-}
-
 template <int P>
 size_t pair_smem(int rows, int np) {
     return (size_t)rows * 12 * np * sizeof(CxPair<typename Prec<P>::pair>);
-}
-
-template <int P, int NB, int MAXL>
-bk_status run_gram_w(Field A, Field B0, Field B1, const SysPart& p, const PTiles& wt, double2* part, int nchunk,
-                     int V, cudaStream_t st) {
-    const size_t smem = (size_t)GW_WARPS * NB * 2 * MAXL * 32 * sizeof(double2);
-    BK_CUDA_TRY(cudaFuncSetAttribute(k_gram_w<P, NB, MAXL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_gram_w<P, NB, MAXL><<<dim3(wt.n, nchunk), GW_WARPS * 32, smem, st>>>(A, B0, B1, p, wt, part, V, nchunk);
-    BK_CUDA_TRY(cudaGetLastError());
-    return BK_OK;
 }
 
 template <int P>
@@ -1366,18 +1082,8 @@ bk_status gram_impl(Field A, Field B, Field B2, int NB, const SysPart& p, double
     const int maxL = max_active_L(p);
     if (maxL == 0) return BK_OK;
     const int ne = p.coef_off[p.nsys];
-    if (maxL <= GS_MAXL) {
-        const PTiles wt = make_ptiles(p, WT_PAIRS);
-        if (NB == 2 && maxL <= GS2_MAXL) {
-            BK_TRY((run_gram_w<P, 2, GS2_MAXL>(A, B, B2, p, wt, part, nchunk, V, st)));
-        } else {
-            for (int b = 0; b < NB; ++b) {
-                Field Bb = b == 0 ? B : B2;
-                double2* pb = part + (size_t)b * nchunk * ne;
-                if (maxL <= 6) BK_TRY((run_gram_w<P, 1, 6>(A, Bb, Bb, p, wt, pb, nchunk, V, st)));
-                else BK_TRY((run_gram_w<P, 1, GS_MAXL>(A, Bb, Bb, p, wt, pb, nchunk, V, st)));
-            }
-        }
+    if (maxL <= ROWS_MAXL) {
+        BK_TRY(rows_gram(P, A, B, B2, NB, p, part, nchunk, V, st));
     } else {
         BigWork w;
         w.n = 0;
@@ -1410,7 +1116,7 @@ bk_status gram_impl(Field A, Field B, Field B2, int NB, const SysPart& p, double
             BK_CUDA_TRY(cudaGetLastError());
         }
     }
-    k_gram_finish<<<(NB * ne + 127) / 128, 128, 0, st>>>(part, nchunk, NB, p, (double2*)G, (double2*)G2);
+    k_gram_finish<<<(NB * ne + 31) / 32, dim3(32, FIN_ROWS), 0, st>>>(part, nchunk, NB, p, (double2*)G, (double2*)G2);
     BK_CUDA_TRY(cudaGetLastError());
     return BK_OK;
 }
@@ -1427,18 +1133,24 @@ bk_status gram_dispatch(int prec, Field A, Field B, Field B2, int NB, const SysP
 
 }  // namespace
 
+// partial-sum rows of a Gram matrix over the active systems
+static int gram_chunks(const SysPart& p, int V) {
+    return max_active_L(p) <= ROWS_MAXL ? gram_row_chunks(V, row_tiles(p).n) : site_chunks(V);
+}
+
 size_t gram_partial_bytes(const SysPart& p, int V) {
-    return (size_t)2 * site_chunks(V) * std::max(1, p.coef_off[p.nsys]) * sizeof(double2);
+    return (size_t)2 * std::max(site_chunks(V), gram_row_chunks_max(V)) * std::max(1, p.coef_off[p.nsys]) *
+           sizeof(double2);
 }
 
 bk_status launch_gram(int prec, Field A, Field B, const SysPart& p, double* G, double* partial, int V,
                       cudaStream_t st) {
-    return gram_dispatch(prec, A, B, B, 1, p, G, nullptr, partial, site_chunks(V), V, st);
+    return gram_dispatch(prec, A, B, B, 1, p, G, nullptr, partial, gram_chunks(p, V), V, st);
 }
 
 bk_status launch_gram2(int prec, Field A, Field B, Field B2, const SysPart& p, double* G, double* G2,
                        double* partial, int V, cudaStream_t st) {
-    return gram_dispatch(prec, A, B, B2, 2, p, G, G2, partial, site_chunks(V), V, st);
+    return gram_dispatch(prec, A, B, B2, 2, p, G, G2, partial, gram_chunks(p, V), V, st);
 }
 
 bk_status launch_gram_slots(int prec, Field A, Field B, const SysPart& p, double* G, double* partial,
@@ -1448,12 +1160,12 @@ bk_status launch_gram_slots(int prec, Field A, Field B, const SysPart& p, double
         bk_set_error("Gram partial sums need %lld slots per site chunk, %lld available", ne, slots);
         return BK_ERR_INVALID_ARG;
     }
-    const int nchunk = (int)std::min<long long>(site_chunks(V), slots / ne);
+    const int nchunk = (int)std::min<long long>(gram_chunks(p, V), slots / ne);
     return gram_dispatch(prec, A, B, B, 1, p, G, nullptr, partial, nchunk, V, st);
 }
 
 size_t coldot_partial_bytes(int L, int npair, int V) {
-    return (size_t)site_chunks(V) * npair * (2 * npairs(L) + 2) * sizeof(double2);
+    return (size_t)MAX_CHUNKS * npair * (2 * npairs(L) + 2) * sizeof(double2);
 }
 
 bk_status launch_coldot(int prec, int npair, const Field* A, const Field* B, int c0, int n, double* out, int ldo,
@@ -1463,52 +1175,57 @@ bk_status launch_coldot(int prec, int npair, const Field* A, const Field* B, int
         bk_set_error("column dots start on an even column");
         return BK_ERR_INVALID_ARG;
     }
+    // npair 1: A[0]^H B[0]; 2: A[0]^H B[0] and |A[0]|^2 (the only pairs the methods need)
+    const bool self = A[0].data == B[0].data;
+    if (npair < 1 || npair > 2 || (npair == 2 && (A[1].data != A[0].data || B[1].data != A[0].data))) {
+        bk_set_error("unsupported column dots");
+        return BK_ERR_INVALID_ARG;
+    }
+    const int mode = npair == 2 ? 2 : (self ? 1 : 0);
     const int q0 = c0 / 2, nq = (n + 1) / 2;
-    const int nchunk = site_chunks(V);
     double2* part = (double2*)partial;
-    const Field A1 = npair > 1 ? A[1] : A[0], B1 = npair > 1 ? B[1] : B[0];
     // pair slots per block: the smallest of 4, 8, 16, 32 that covers the range
     const int tx = nq <= 4 ? 4 : (nq <= 8 ? 8 : (nq <= 16 ? 16 : 32));
-    dim3 grid((nq + tx - 1) / tx, nchunk);
-#define BK_CD1(PP, NP, TX) k_coldot<PP, NP, TX><<<grid, dim3(TX, 256 / TX), 0, st>>>(A[0], B[0], A1, B1, q0, nq, part, V, nchunk)
-#define BK_CD(PP, NP)                       \
-    if (tx == 4) BK_CD1(PP, NP, 4);         \
-    else if (tx == 8) BK_CD1(PP, NP, 8);    \
-    else if (tx == 16) BK_CD1(PP, NP, 16);  \
-    else BK_CD1(PP, NP, 32);
-    if (npair == 1) {
-        switch (prec) {
-            case BK_FP64: BK_CD(BK_FP64, 1); break;
-            case BK_FP32: BK_CD(BK_FP32, 1); break;
-            case BK_FP16: BK_CD(BK_FP16, 1); break;
-            default: return BK_ERR_INVALID_ARG;
-        }
-    } else {
-        switch (prec) {
-            case BK_FP64: BK_CD(BK_FP64, 2); break;
-            case BK_FP32: BK_CD(BK_FP32, 2); break;
-            case BK_FP16: BK_CD(BK_FP16, 2); break;
-            default: return BK_ERR_INVALID_ARG;
-        }
+    const unsigned rows = 12u * (unsigned)V;
+    // at least 4 rows a thread, at most 2 blocks an SM in all
+    const int ngrp = (nq + tx - 1) / tx;
+    const int nchunk = (int)std::max(1u, std::min(rows / (256u / tx * 4u), (unsigned)std::max(1, MAX_CHUNKS / ngrp)));
+    dim3 grid(ngrp, nchunk);
+#define BK_CD1(PP, MD, TX) k_coldot<PP, MD, TX><<<grid, dim3(TX, 256 / TX), 0, st>>>(A[0], B[0], q0, nq, part, rows, nchunk)
+#define BK_CD(PP, MD)                       \
+    if (tx == 4) BK_CD1(PP, MD, 4);         \
+    else if (tx == 8) BK_CD1(PP, MD, 8);    \
+    else if (tx == 16) BK_CD1(PP, MD, 16);  \
+    else BK_CD1(PP, MD, 32);
+#define BK_CDM(PP)                          \
+    if (mode == 0) { BK_CD(PP, 0) }         \
+    else if (mode == 1) { BK_CD(PP, 1) }    \
+    else { BK_CD(PP, 2) }
+    switch (prec) {
+        case BK_FP64: BK_CDM(BK_FP64) break;
+        case BK_FP32: BK_CDM(BK_FP32) break;
+        case BK_FP16: BK_CDM(BK_FP16) break;
+        default: return BK_ERR_INVALID_ARG;
     }
+#undef BK_CDM
 #undef BK_CD
 #undef BK_CD1
     BK_CUDA_TRY(cudaGetLastError());
-    k_coldot_finish<<<(npair * n + 127) / 128, 128, 0, st>>>(part, nchunk, npair, nq, n,
-                                                             (double2*)out + c0, ldo);
+    k_coldot_finish<<<(npair * n + 31) / 32, dim3(32, FIN_ROWS), 0, st>>>(part, nchunk, npair, nq, n,
+                                                                         (double2*)out + c0, ldo);
     BK_CUDA_TRY(cudaGetLastError());
     return BK_OK;
 }
 
-int genop_norm_rows(int V) { return site_chunks(V); }
+// grid rows of the updates (a function of the lattice alone: the fused norms
+// of a system whose update was skipped stay those of its last residual)
+int genop_norm_rows(int V) { return std::max(1, std::min(MAX_CHUNKS, (12 * V) / 16)); }
 
 bk_status launch_genop(int prec, const GenOp& g, int V, cudaStream_t st, bool* ynorm_done) {
     if (ynorm_done) *ynorm_done = false;
-    const int nchunk = site_chunks(V);
+    const int nchunk = genop_norm_rows(V);
     const int ncols = g.p.col0[g.p.nsys];
-    int maxL = 0;
-    for (int s = 0; s < g.p.nsys; ++s)
-        if ((g.p.active >> s) & 1ull) maxL = std::max(maxL, g.p.L[s]);
+    const int maxL = max_active_L(g.p);
     if (maxL == 0) return BK_OK;
     // every operand in the layout's pair count (the fast kernels use one offset)
     const int np = g.Y.np;
@@ -1516,43 +1233,15 @@ bk_status launch_genop(int prec, const GenOp& g, int V, cudaStream_t st, bool* y
     for (int u = 0; u < g.nmi; ++u) same_np &= g.Mi[u].np == np;
     for (int e = 0; e < g.ne; ++e) same_np &= g.E[e].np == np;
     if (g.hasX) same_np &= g.X.np == np && g.Xin.np == np;
-    if (maxL <= 12 && g.hasY && same_np) {
+    if (maxL <= ROWS_MAXL && g.hasY && same_np && prec != BK_FP16) {
+        BK_TRY(rows_update(prec, g, V, genop_norm_rows(V), np, st));
+    } else if (maxL <= ROWS_MAXL && g.hasY && same_np) {
         const PTiles wt = make_ptiles(g.p, WT_PAIRS);
         const dim3 grid(wt.n, nchunk);
-        const bool h = g.hasX != 0;
-#define BK_GW(PP, ML, UK, MB, NM, NE, HX) \
-    k_genop_w<PP, ML, UK, MB, NM, NE, HX><<<grid, GW_WARPS * 32, 0, st>>>(g, wt, V, nchunk, ncols, np)
-        // the FP32 updates of the two methods, then any other combination
-#define BK_GW32(ML)                                                                     \
-    if (g.nmi == 1 && g.ne == 0 && !h) BK_GW(BK_FP32, ML, 2, 2, 1, 0, 0);               \
-    else if (g.nmi == 1 && g.ne == 1 && !h) BK_GW(BK_FP32, ML, 2, 2, 1, 1, 0);          \
-    else if (g.nmi == 1 && g.ne == 2 && h) BK_GW(BK_FP32, ML, 2, 2, 1, 2, 1);           \
-    else if (g.nmi == 2 && g.ne == 1 && !h) BK_GW(BK_FP32, ML, 2, 2, 2, 1, 0);          \
-    else if (g.nmi == 2 && g.ne == 0 && h) BK_GW(BK_FP32, ML, 2, 2, 2, 0, 1);           \
-    else if (g.nmi == 0 && g.ne == 3 && !h) BK_GW(BK_FP32, ML, 2, 2, 0, 3, 0);          \
-    else BK_GW(BK_FP32, ML, 1, 2, -1, -1, -1);
-        switch (prec) {
-            case BK_FP64:
-                if (maxL <= 6) BK_GW(BK_FP64, 6, 1, 1, -1, -1, -1);
-                else BK_GW(BK_FP64, 12, 1, 1, -1, -1, -1);
-                break;
-            case BK_FP32:
-                if (maxL <= 6) {
-                    BK_GW32(6)
-                } else {
-                    BK_GW32(12)
-                }
-                break;
-            case BK_FP16:
-                if (maxL <= 6) BK_GW(BK_FP16, 6, 1, 1, -1, -1, -1);
-                else BK_GW(BK_FP16, 12, 1, 1, -1, -1, -1);
-                break;
-            default: return BK_ERR_INVALID_ARG;
-        }
-#undef BK_GW32
-#undef BK_GW
+        if (maxL <= 6) k_genop_w<6><<<grid, GW_WARPS * 32, 0, st>>>(g, wt, V, nchunk, ncols, np);
+        else k_genop_w<12><<<grid, GW_WARPS * 32, 0, st>>>(g, wt, V, nchunk, ncols, np);
     } else {
-        const PTiles tl = make_ptiles(g.p);
+        const PTiles tl = make_ptiles(g.p, TILE_MAXP);
         constexpr int SR = 4;
         const dim3 grid(tl.n, nchunk), block(TILE_MAXP, SR);
         switch (prec) {
@@ -1569,7 +1258,7 @@ bk_status launch_genop(int prec, const GenOp& g, int V, cudaStream_t st, bool* y
 
 bk_status launch_norm_finish(const double* ynorm, int ncols, int c0, int n, double* out, int V, cudaStream_t st) {
     if (n <= 0) return BK_OK;
-    k_norm_finish<<<(n + 127) / 128, 128, 0, st>>>(ynorm, genop_norm_rows(V), ncols, c0, n, out);
+    k_norm_finish<<<(n + 31) / 32, dim3(32, FIN_ROWS), 0, st>>>(ynorm, genop_norm_rows(V), ncols, c0, n, out);
     BK_CUDA_TRY(cudaGetLastError());
     return BK_OK;
 }

@@ -1,0 +1,170 @@
+// Shared by the block-algebra translation units: the column partition as the
+// kernels see it, runs of whole systems (tiles), element access in the
+// RHS-interleaved pair layout and packed complex arithmetic on column pairs.
+#pragma once
+
+#include <algorithm>
+
+#include "bk_common.cuh"
+#include "bk_kernels.h"
+
+// system owning column pair q (columns 2q, 2q + 1)
+__device__ __forceinline__ int sys_of_pair(const SysPart& p, int q) {
+    int lo = 0, hi = p.nsys - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (2 * q >= p.col0[mid]) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
+}
+
+// Runs of whole active systems, at most maxp pairs each (one system may be
+// larger): the unit a block or warp takes, so that every column it combines
+// is its own.
+struct PTiles {
+    int n;
+    int p0[BK_MAX_SYS];
+    int np[BK_MAX_SYS];
+};
+
+inline PTiles make_ptiles(const SysPart& p, int maxp) {
+    PTiles t;
+    t.n = 0;
+    bool open = false;
+    for (int s = 0; s < p.nsys; ++s) {
+        const int q0 = p.col0[s] / 2, nq = (p.col0[s + 1] - p.col0[s]) / 2;
+        if (!((p.active >> s) & 1ull) || nq == 0) {
+            open = false;
+            continue;
+        }
+        if (open && t.np[t.n - 1] + nq <= maxp) {
+            t.np[t.n - 1] += nq;
+        } else {
+            t.p0[t.n] = q0;
+            t.np[t.n] = nq;
+            t.n++;
+            open = true;
+        }
+    }
+    return t;
+}
+
+inline int max_active_L(const SysPart& p) {
+    int m = 0;
+    for (int s = 0; s < p.nsys; ++s)
+        if ((p.active >> s) & 1ull) m = std::max(m, p.L[s]);
+    return m;
+}
+
+template <typename R2>
+struct CxPair {  // one spinor component of a column pair, arithmetic type
+    R2 re, im;
+};
+
+template <typename R2>
+__device__ __forceinline__ CxPair<R2> cp_zero() {
+    CxPair<R2> v;
+    v.re = v.im = pzero<R2>();
+    return v;
+}
+
+template <typename R2>
+__device__ __forceinline__ CxPair<R2> shfl_pair(const CxPair<R2>& v, int src) {
+    CxPair<R2> o;
+    o.re.x = __shfl_sync(0xffffffffu, v.re.x, src);
+    o.re.y = __shfl_sync(0xffffffffu, v.re.y, src);
+    o.im.x = __shfl_sync(0xffffffffu, v.im.x, src);
+    o.im.y = __shfl_sync(0xffffffffu, v.im.y, src);
+    return o;
+}
+
+__device__ __forceinline__ float2 bcast(float v) { return make_float2(v, v); }
+__device__ __forceinline__ double2 bcast(double v) { return make_double2(v, v); }
+
+// acc (pair) += c (complex scalar) * v (pair)
+template <typename R, typename R2>
+__device__ __forceinline__ void cpair_mac(CxPair<R2>& acc, cx<R> c, const CxPair<R2>& v) {
+    const R2 cr = bcast(c.r), ci = bcast(c.i), nci = bcast(-c.i);
+    acc.re = pfma(cr, v.re, acc.re);
+    acc.re = pfma(nci, v.im, acc.re);
+    acc.im = pfma(cr, v.im, acc.im);
+    acc.im = pfma(ci, v.re, acc.im);
+}
+
+// Element e (row * np + pair) through the read-only data path, FP16 scale
+// applied.  Only for operands that no thread of the kernel writes, or that
+// the reading thread alone writes after its one read.
+template <int P>
+__device__ __forceinline__ CxPair<typename Prec<P>::pair> ldg_at(const Field& f, size_t e,
+                                                                  typename Prec<P>::pair sc) {
+    CxPair<typename Prec<P>::pair> v;
+    if constexpr (P == BK_FP64) {
+        const double2* q = (const double2*)f.data + 2 * e;
+        v.re = __ldg(q);
+        v.im = __ldg(q + 1);
+    } else if constexpr (P == BK_FP32) {
+        const float4 q = __ldg((const float4*)f.data + e);
+        v.re = make_float2(q.x, q.y);
+        v.im = make_float2(q.z, q.w);
+    } else {
+        const uint2 q = __ldg((const uint2*)f.data + e);
+        v.re = pmul(__half22float2(*reinterpret_cast<const __half2*>(&q.x)), sc);
+        v.im = pmul(__half22float2(*reinterpret_cast<const __half2*>(&q.y)), sc);
+    }
+    return v;
+}
+
+template <int P>
+__device__ __forceinline__ CxPair<typename Prec<P>::pair> load_at(const Field& f, size_t e) {
+    CxPair<typename Prec<P>::pair> v;
+    if constexpr (P == BK_FP64) {
+        const double2* q = (const double2*)f.data + 2 * e;
+        v.re = q[0];
+        v.im = q[1];
+    } else {
+        static_assert(P == BK_FP32, "accumulators are FP32 or FP64");
+        const float4 q = ((const float4*)f.data)[e];
+        v.re = make_float2(q.x, q.y);
+        v.im = make_float2(q.z, q.w);
+    }
+    return v;
+}
+
+template <int P>
+__device__ __forceinline__ void store_at(const Field& f, size_t e, typename Prec<P>::pair re,
+                                         typename Prec<P>::pair im) {
+    if constexpr (P == BK_FP64) {
+        double2* q = (double2*)f.data + 2 * e;
+        q[0] = re;
+        q[1] = im;
+    } else {
+        static_assert(P == BK_FP32, "element stores are for FP32 / FP64 blocks");
+        ((float4*)f.data)[e] = make_float4(re.x, re.y, im.x, im.y);
+    }
+}
+
+// complex coefficient mult * (ptr ? ptr[s] : 1)
+template <int P>
+__device__ __forceinline__ cx<typename Prec<P>::real> coef(const double* ptr, double mult, int s) {
+    using R = typename Prec<P>::real;
+    if (ptr) return mk((R)(mult * ptr[2 * s]), (R)(mult * ptr[2 * s + 1]));
+    return mk((R)mult, R(0));
+}
+
+// FP32 products are summed in FP32 over at most this many (site, component)
+// rows per lane, then moved to FP64
+constexpr int ROW_FLUSH = 96;
+
+// rows.cu: systems of at most ROWS_MAXL columns
+constexpr int ROWS_MAXL = 12;
+// site chunks (partial-sum rows) of the row Gram kernel over nt tiles
+inline int gram_row_chunks(int V, int nt) {
+    const int most = std::max(1, std::min((12 * V) / 16, 608));
+    return std::max(std::min(most, 76), most / std::max(1, nt));
+}
+inline int gram_row_chunks_max(int V) { return gram_row_chunks(V, 1); }
+bk_status rows_gram(int prec, Field A, Field B, Field B2, int NB, const SysPart& p, double2* partial, int nchunk,
+                    int V, cudaStream_t st);
+PTiles row_tiles(const SysPart& p);
+bk_status rows_update(int prec, const GenOp& g, int V, int nchunk, int np, cudaStream_t st);
