@@ -281,9 +281,7 @@ extern "C" bk_status bk_unpack(bk_ctx* c, const void* Xd, double* X, int L, bk_p
 // computes the same result.
 static bk_status tune_shape(bk_ctx* c, int prec, DslashOp op, cudaStream_t st, bk_ctx::Shape& best) {
     std::vector<bk_ctx::Shape> cands;
-    if (wide(prec)) {
-        for (int t : {64, 128}) cands.push_back({t, 0, 0, 0});
-    } else {
+    {
         // register caps 255 (variant 1), 170 (2), 128 (3); pair groups of 16
         // pairs or all pairs at once; no prefetch, prefetch into L2 or L1, or
         // the looped form with L1 prefetch one hop ahead
@@ -360,11 +358,8 @@ static bk_status dslash_fields(bk_ctx* c, int prec, const double* kappa, Field x
         op.variant = c->force_variant;
         op.group = 8;
         op.prefetch = c->force_prefetch;
-    } else if (c->autotune && ncol <= BK_MAX_COLS) {
-        // FP64-class launches are bound by the FP64 pipe whatever their width:
-        // one shape per mode, tuned at first use
-        const long long key =
-            ((long long)prec << 40) | ((long long)(residual != 0) << 36) | (wide(prec) ? 0 : ncol);
+    } else if (c->autotune && ncol <= BK_MAX_COLS && !wide(prec)) {
+        const long long key = ((long long)prec << 40) | ((long long)(residual != 0) << 36) | ncol;
         auto it = c->shapes.find(key);
         if (it == c->shapes.end()) {
             bk_ctx::Shape sh;
@@ -916,14 +911,66 @@ struct Solve {
         for (const auto& cr : col_runs(part.active)) BK_TRY(coldot(P, npair, A, B, out, cr.first, cr.second));
         return BK_OK;
     }
-    // L x L solves in two steps: factor G once, substitute for each right-hand side
-    bk_status factor(const double* G, int* info) {
-        launches += 1;
-        return launch_lu_factor(G, LU, piv, info, part, st);
+    // the systems are small enough for the one-launch L x L steps (small.cu)
+    bool small_systems() const {
+        for (int s = 0; s < nsys; ++s)
+            if (part.L[s] > SMALL_MAXL) return false;
+        return true;
     }
-    bk_status substitute(const double* H, const double* scale_dev, const double* scale_host, double* X, int* info) {
+    SmallStep small_step() const {
+        SmallStep a;
+        memset(&a, 0, sizeof(a));
+        a.p = part;
+        a.LU = LU;
+        a.piv = piv;
+        return a;
+    }
+    void with_zeta(SmallStep& a) const {
+        a.dots = dots;
+        a.Lt = Lt;
+        a.zeta = zeta;
+        a.mzeta = mzeta;
+        a.izeta = izeta;
+        a.zbad = zbad;
+    }
+    // Factor G and solve X = G^-1 (scale H); zeta_too: also the scalars zeta from dots
+    bk_status factor_solve(const double* G, const double* H, const double* scale_dev, double* X, int* info,
+                           bool zeta_too) {
+        if (small_systems()) {
+            SmallStep a = small_step();
+            a.G = G;
+            a.H = H;
+            a.hs_dev = scale_dev;
+            a.X = X;
+            a.info = info;
+            if (zeta_too) with_zeta(a);
+            launches += 1;
+            return launch_small_step(a, st);
+        }
+        if (zeta_too) BK_TRY(scalars());
+        launches += 2;
+        BK_TRY(launch_lu_factor(G, LU, piv, info, part, st));
+        return launch_lu_solve(LU, piv, H, scale_dev, nullptr, X, info, part, st);
+    }
+    // X = -G^-1 H with the factors of the last factor_solve (its status in
+    // info_in), and the scalars zeta from dots
+    bk_status resolve_neg_zeta(const double* H, double* X, const int* info_in, int* info) {
+        if (small_systems()) {
+            SmallStep a = small_step();
+            a.H = H;
+            a.hs_neg = 1;
+            a.X = X;
+            a.info_in = info_in;
+            a.info = info;
+            with_zeta(a);
+            launches += 1;
+            return launch_small_step(a, st);
+        }
+        BK_TRY(scalars());
         launches += 1;
-        return launch_lu_solve(LU, piv, H, scale_dev, scale_host, X, info, part, st);
+        BK_CUDA_TRY(cudaMemcpyAsync(info, info_in, sizeof(int) * nsys, cudaMemcpyDeviceToDevice, st));
+        const double hs[2] = {-1.0, 0.0};
+        return launch_lu_solve(LU, piv, H, nullptr, hs, X, info, part, st);
     }
     bk_status scalars() {
         launches += 1;
@@ -1514,7 +1561,7 @@ struct Solve {
     bk_status cholesky_basis() {
         BK_TRY(gram(Pb, Pb, G_Z));
         launches += 1;
-        BK_TRY(launch_chol_inv(G_Z, gam, part, st));
+        BK_TRY(small_systems() ? launch_small_chol(G_Z, gam, part, st) : launch_chol_inv(G_Z, gam, part, st));
         GenOp g = genop0();
         g.nmi = 1;
         g.Mi[0] = Pb;
@@ -1547,11 +1594,9 @@ struct Solve {
                 BK_TRY(gram(Rt, Vb, G_V));
                 Field a[2] = {Wb, Wb}, b[2] = {R, Wb};
                 BK_TRY(coldot_active(2, a, b, dots));
-                BK_TRY(scalars());
             }
-            // alpha: (R~^H V) alpha = R~^H R
-            BK_TRY(factor(G_V, info_a));
-            BK_TRY(substitute(G_RR, nullptr, nullptr, alpha, info_a));
+            // alpha: (R~^H V) alpha = R~^H R; zeta
+            BK_TRY(factor_solve(G_V, G_RR, nullptr, alpha, info_a, true));
             {   // U = (P - zeta V) alpha;  X += zeta R + U
                 GenOp g = genop0();
                 g.nmi = 2;
@@ -1598,8 +1643,7 @@ struct Solve {
             BK_TRY(gram(Rt, R, G_RRn));          // R~^H R_{k+1}
             BK_TRY(dslash_active(R, Wb, R));  // W = A R
             // gamma: (R~^H R_k) gamma = R~^H R_{k+1} / zeta
-            BK_TRY(factor(G_RR, info_g));
-            BK_TRY(substitute(G_RRn, izeta, nullptr, gam, info_g));
+            BK_TRY(factor_solve(G_RR, G_RRn, izeta, gam, info_g, false));
             {   // P = R + U gamma
                 GenOp g = genop0();
                 g.ne = 1;
@@ -1633,8 +1677,7 @@ struct Solve {
             if (orth) BK_TRY(cholesky_basis());  // before V = A P
             BK_TRY(dslash_active(Pb, Vb, Pb));  // V = A P
             BK_TRY(gram2(Rt, Vb, R, G_V, G_RR));  // R~^H V, R~^H R
-            BK_TRY(factor(G_V, info_a));  // R~^H V, used for alpha and beta
-            BK_TRY(substitute(G_RR, nullptr, nullptr, alpha, info_a));
+            BK_TRY(factor_solve(G_V, G_RR, nullptr, alpha, info_a, false));  // R~^H V, used for alpha and beta
             {   // T = R - V alpha
                 GenOp g = genop0();
                 g.ne = 1;
@@ -1654,15 +1697,10 @@ struct Solve {
             {
                 Field a[2] = {Zb, Zb}, b[2] = {Tb, Zb};
                 BK_TRY(coldot_active(2, a, b, dots));  // Tr(Z^H T), Tr(Z^H Z)
-                BK_TRY(scalars());
                 BK_TRY(gram(Rt, Zb, G_Z));
             }
-            // beta: (R~^H V) beta = -R~^H Z, with the factors of alpha's matrix
-            {
-                const double m1[2] = {-1.0, 0.0};
-                BK_CUDA_TRY(cudaMemcpyAsync(info_g, info_a, sizeof(int) * nsys, cudaMemcpyDeviceToDevice, st));
-                BK_TRY(substitute(G_Z, nullptr, m1, gam, info_g));
-            }
+            // beta: (R~^H V) beta = -R~^H Z, with the factors of alpha's matrix; zeta
+            BK_TRY(resolve_neg_zeta(G_Z, gam, info_a, info_g));
             {   // X += P alpha + zeta T;  R = T - zeta Z
                 GenOp g = genop0();
                 g.ne = 2;

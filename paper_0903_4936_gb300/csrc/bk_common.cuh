@@ -156,6 +156,47 @@ __host__ inline Field field_pairs(Field f, int p0, int prec) {
     return g;
 }
 
+// ---------------------------------------------------------------- FP64 <-> FP32 without the FP64 pipe
+//
+// A conversion instruction between float and double occupies the FP64 pipe
+// like an FP64 operation (64 cycles of a scheduler per warp), which made the
+// casts and the coefficient loads of the FP32 kernels wait for it.  For zero
+// and normal numbers that stay normal the same bits come from a few integer
+// instructions; everything else takes the instruction.
+
+// round to nearest even, as (float)x
+__device__ __forceinline__ float d2f(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned ex = (hi >> 20) & 0x7ff;
+    if (ex - 897u < 253u) {  // 2^-126 <= |x| < 2^127: the result is normal
+        const unsigned m = (hi << 3) | (lo >> 29);  // exponent and mantissa bits of the float, unrounded
+        unsigned f = (m ^ 0x40000000u) & 0x7fffffffu;  // exponent less 896, modulo 256
+        const unsigned rest = lo << 3;  // the discarded 29 bits, left-aligned
+        f += (rest > 0x80000000u || (rest == 0x80000000u && (f & 1u))) ? 1u : 0u;
+        return __uint_as_float(f | (hi & 0x80000000u));
+    }
+    if (((hi << 1) | lo) == 0u) return __uint_as_float(hi);  // +-0
+    return __double2float_rn(x);
+}
+// exact, as (double)x
+__device__ __forceinline__ double f2d(float x) {
+    const unsigned b = __float_as_uint(x), ex = (b >> 23) & 0xff;
+    if (ex - 1u < 254u)
+        return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
+    if ((b << 1) == 0u) return __hiloint2double((int)b, 0);
+    return (double)x;
+}
+__device__ __forceinline__ double f2d(double x) { return x; }
+__device__ __forceinline__ float2 d2f(double2 v) { return make_float2(d2f(v.x), d2f(v.y)); }
+__device__ __forceinline__ double2 f2d(float2 v) { return make_double2(f2d(v.x), f2d(v.y)); }
+// to the arithmetic type R
+template <typename R>
+__device__ __forceinline__ R d2r(double x);
+template <>
+__device__ __forceinline__ float d2r<float>(double x) { return d2f(x); }
+template <>
+__device__ __forceinline__ double d2r<double>(double x) { return x; }
+
 // ---------------------------------------------------------------- packed pair arithmetic
 //
 // Pairs of reals (the same component of two columns) are combined with one

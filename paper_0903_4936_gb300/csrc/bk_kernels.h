@@ -152,6 +152,8 @@ struct GenOp {
     // optional: squared norms of the Y columns, as per-block partial sums
     // ynorm[b * ncols + col] (FP64), summed by launch_norm_finish
     double* ynorm;
+    // set by the launcher: which coefficients are 1 or -1 (else 0), and whether M is used
+    int ea_unit[GENOP_MAXE], ma_unit[GENOP_MAXMI], xa_unit, y_unit, x_unit, mat;
 };
 // *ynorm_done = whether the kernel filled g.ynorm
 bk_status launch_genop(int prec, const GenOp& g, int V, cudaStream_t st, bool* ynorm_done = nullptr);
@@ -190,3 +192,31 @@ bk_status launch_lu_solve(const double* LU, const int* piv, const double* H, con
 // system), Tinv_s = T^-1; identity if not numerically positive definite.
 // L <= 118 per system.
 bk_status launch_chol_inv(const double* S, double* Tinv, const SysPart& p, cudaStream_t st, double shift_rel = 0.0);
+
+// ---------------------------------------------------------------- small.cu
+// The L x L steps of an iteration for systems of at most SMALL_MAXL columns,
+// one launch: with G, factor G_s (LU, piv) and, with H, solve X_s = G_s^-1
+// (scale_s H_s); without G, solve with the factors of an earlier step (info_in:
+// its status).  scale: hs_dev (complex FP64 per system), or -1 (hs_neg) or 1.  With
+// dots (d0 at [j], real d1 at [Lt + j]): zeta_s = sum d0 / sum d1, -zeta,
+// 1 / zeta, zbad.  info[s]: 0, the failed pivot + 1, or L + 1 (X not finite).
+constexpr int SMALL_MAXL = 12;
+struct SmallStep {
+    SysPart p;
+    const double* G;
+    double* LU;
+    int* piv;
+    const double* H;
+    const double* hs_dev;
+    int hs_neg;
+    double* X;
+    const int* info_in;
+    int* info;
+    const double* dots;
+    int Lt;
+    double *zeta, *mzeta, *izeta;
+    int* zbad;
+};
+bk_status launch_small_step(const SmallStep& a, cudaStream_t st);
+// S_s = T^H T, Tinv_s = T^-1 (identity if not numerically positive definite)
+bk_status launch_small_chol(const double* S, double* Tinv, const SysPart& p, cudaStream_t st);

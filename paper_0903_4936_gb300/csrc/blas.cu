@@ -218,14 +218,17 @@ __global__ void __launch_bounds__(256) k_gram_big(Field A, Field B, SysPart p, B
         }
 }
 
-// Sums over the chunks' partial rows: 32 entries x FIN_ROWS row slices per
+// Sums over the chunks' partial rows: FIN_E entries x FIN_ROWS row slices per
 // block (a thread adds every FIN_ROWS-th row), combined in shared memory in a
-// fixed order.  One thread per entry over all rows took 75 us for 304 rows.
-constexpr int FIN_ROWS = 16;
+// fixed order.  Few entries a block, because the FP64 adds of one SM are the
+// bound (one thread per entry over all rows: 75 us for 360 entries of 304
+// rows; 32 entries a block: 18 us for 144 entries of 608).
+constexpr int FIN_E = 8;
+constexpr int FIN_ROWS = 32;
 
 template <typename F>
 __device__ __forceinline__ double2 sum_rows(int nrows, bool on, F row) {
-    __shared__ double2 red[FIN_ROWS][32];
+    __shared__ double2 red[FIN_ROWS][FIN_E];
     double2 v = make_double2(0.0, 0.0);
     if (on) {
 #pragma unroll 4
@@ -236,23 +239,26 @@ __device__ __forceinline__ double2 sum_rows(int nrows, bool on, F row) {
         }
     }
     red[threadIdx.y][threadIdx.x] = v;
-    __syncthreads();
-    v = make_double2(0.0, 0.0);
-    if (threadIdx.y == 0)
-        for (int y = 0; y < FIN_ROWS; ++y) {
-            v.x += red[y][threadIdx.x].x;
-            v.y += red[y][threadIdx.x].y;
+#pragma unroll
+    for (int o = FIN_ROWS / 2; o > 0; o >>= 1) {
+        __syncthreads();
+        if (threadIdx.y < o) {
+            const double2 b = red[threadIdx.y + o][threadIdx.x];
+            v.x += b.x;
+            v.y += b.y;
+            red[threadIdx.y][threadIdx.x] = v;
         }
+    }
     return v;  // valid in the threads of row 0
 }
 
 // G[e] (and G2) = sum over chunks of the partial sums, for the entries of the
 // active systems.
-__global__ void __launch_bounds__(32 * FIN_ROWS) k_gram_finish(const double2* __restrict__ partial, int nchunk, int NB,
+__global__ void __launch_bounds__(FIN_E * FIN_ROWS) k_gram_finish(const double2* __restrict__ partial, int nchunk, int NB,
                                                               SysPart p, double2* __restrict__ G,
                                                               double2* __restrict__ G2) {
     const int ne = p.coef_off[p.nsys];
-    const int e = blockIdx.x * 32 + threadIdx.x;
+    const int e = blockIdx.x * FIN_E + threadIdx.x;
     const int b = e / ne, el = e - b * ne;
     bool on = e < NB * ne;
     if (on) {
@@ -294,9 +300,11 @@ __global__ void __launch_bounds__(256) k_coldot(Field A, Field B, int q0, int nq
     R2 dr = pzero<R2>(), di = dr, nn = dr;
     double2 d0 = make_double2(0.0, 0.0), d1 = d0, n01 = d0;
     auto flush = [&]() {
-        d0 = make_double2(d0.x + (double)dr.x, d0.y + (double)di.x);
-        d1 = make_double2(d1.x + (double)dr.y, d1.y + (double)di.y);
-        n01 = make_double2(n01.x + (double)nn.x, n01.y + (double)nn.y);
+        if (MODE != 1) {
+            d0 = make_double2(d0.x + f2d(dr.x), d0.y + f2d(di.x));
+            d1 = make_double2(d1.x + f2d(dr.y), d1.y + f2d(di.y));
+        }
+        if (MODE != 0) n01 = make_double2(n01.x + f2d(nn.x), n01.y + f2d(nn.y));
         dr = di = nn = pzero<R2>();
     };
     int since = 0;
@@ -364,10 +372,10 @@ __global__ void __launch_bounds__(256) k_coldot(Field A, Field B, int q0, int nq
 }
 
 // out[kk * ldo + j] = sum over chunks, columns j < n
-__global__ void __launch_bounds__(32 * FIN_ROWS) k_coldot_finish(const double2* __restrict__ partial, int nchunk,
+__global__ void __launch_bounds__(FIN_E * FIN_ROWS) k_coldot_finish(const double2* __restrict__ partial, int nchunk,
                                                                 int npair, int nq, int n, double2* __restrict__ out,
                                                                 int ldo) {
-    const int e = blockIdx.x * 32 + threadIdx.x;
+    const int e = blockIdx.x * FIN_E + threadIdx.x;
     const bool on = e < npair * n;
     const int kk = e / n, j = e - kk * n;
     const double2 v = sum_rows(
@@ -430,10 +438,10 @@ __global__ void __launch_bounds__(256) k_genop(const __grid_constant__ GenOp g, 
     const bool mat = g.nmi > 0 && g.M != nullptr && ((g.hasY && g.ym != 0.0) || (g.hasX && g.xm != 0.0));
     cx<R> ea[GENOP_MAXE], ma[GENOP_MAXMI], xa = mk(R(0), R(0));
 #pragma unroll
-    for (int e = 0; e < GENOP_MAXE; ++e) ea[e] = e < g.ne ? coef<P>(g.ea[e], g.ea_mult[e], s) : mk(R(0), R(0));
+    for (int e = 0; e < GENOP_MAXE; ++e) ea[e] = e < g.ne ? coef<P>(g.ea[e], g.ea_mult[e], 0, s) : mk(R(0), R(0));
 #pragma unroll
-    for (int u = 0; u < GENOP_MAXMI; ++u) ma[u] = u < g.nmi ? coef<P>(g.ma[u], g.ma_mult[u], s) : mk(R(0), R(0));
-    if (g.hasX) xa = coef<P>(g.xa, g.xa_mult, s);
+    for (int u = 0; u < GENOP_MAXMI; ++u) ma[u] = u < g.nmi ? coef<P>(g.ma[u], g.ma_mult[u], 0, s) : mk(R(0), R(0));
+    if (g.hasX) xa = coef<P>(g.xa, g.xa_mult, 0, s);
     const double2* M = reinterpret_cast<const double2*>(g.M) + (on && mat ? g.p.coef_off[s] : 0);
     const bool j1ok = i0 + 1 < Ls;
     R2 ym2;
@@ -595,10 +603,10 @@ __global__ void __launch_bounds__(GW_WARPS * 32) k_genop_w(const __grid_constant
     const bool mat = nmi > 0 && g.M != nullptr && ((g.hasY && g.ym != 0.0) || (hx && g.xm != 0.0));
     cx<R> ea[ME], ma[MMI], xa = mk(R(0), R(0));
 #pragma unroll
-    for (int e = 0; e < ME; ++e) ea[e] = e < ne ? coef<P>(g.ea[e], g.ea_mult[e], s) : mk(R(0), R(0));
+    for (int e = 0; e < ME; ++e) ea[e] = e < ne ? coef<P>(g.ea[e], g.ea_mult[e], 0, s) : mk(R(0), R(0));
 #pragma unroll
-    for (int u = 0; u < MMI; ++u) ma[u] = u < nmi ? coef<P>(g.ma[u], g.ma_mult[u], s) : mk(R(0), R(0));
-    if (hx) xa = coef<P>(g.xa, g.xa_mult, s);
+    for (int u = 0; u < MMI; ++u) ma[u] = u < nmi ? coef<P>(g.ma[u], g.ma_mult[u], 0, s) : mk(R(0), R(0));
+    if (hx) xa = coef<P>(g.xa, g.xa_mult, 0, s);
     // the lane's two columns of M; rows and columns past the system's size are zero
     R2 Mr[MAXL], Mi[MAXL];
     {
@@ -710,9 +718,9 @@ __global__ void __launch_bounds__(GW_WARPS * 32) k_genop_w(const __grid_constant
     }
 }
 
-__global__ void __launch_bounds__(32 * FIN_ROWS) k_norm_finish(const double* __restrict__ part, int nrows, int ncols,
+__global__ void __launch_bounds__(FIN_E * FIN_ROWS) k_norm_finish(const double* __restrict__ part, int nrows, int ncols,
                                                               int c0, int n, double* __restrict__ out) {
-    const int j = blockIdx.x * 32 + threadIdx.x;
+    const int j = blockIdx.x * FIN_E + threadIdx.x;
     const bool on = j < n;
     const double2 v = sum_rows(
         nrows, on, [&](int c) { return make_double2(__ldg(part + (size_t)c * ncols + c0 + j), 0.0); });
@@ -723,8 +731,8 @@ __global__ void __launch_bounds__(32 * FIN_ROWS) k_norm_finish(const double* __r
 }
 
 // X64 += Xlo; Xlo = 0 over pairs [p0, p0 + np)
-// X64 += sign * Xlo over pairs [p0, p0 + np); zero_lo: then Xlo = 0
-__global__ void k_accum(Field x64, Field xlo, int p0, int np, double sign, int zero_lo) {
+// (sub: -=) over pairs [p0, p0 + np); zero_lo: then Xlo = 0
+__global__ void k_accum(Field x64, Field xlo, int p0, int np, int sub, int zero_lo) {
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= (long long)x64.V * np) return;
     const int n = (int)(g / np), q = p0 + (int)(g - (long long)(g / np) * np);
@@ -734,8 +742,9 @@ __global__ void k_accum(Field x64, Field xlo, int p0, int np, double sign, int z
     load_pair<BK_FP32>(xlo, n, q, lr, li);
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
-        xr[k] = make_double2(fma(sign, (double)lr[k].x, xr[k].x), fma(sign, (double)lr[k].y, xr[k].y));
-        xi[k] = make_double2(fma(sign, (double)li[k].x, xi[k].x), fma(sign, (double)li[k].y, xi[k].y));
+        const double2 r = f2d(lr[k]), i = f2d(li[k]);
+        xr[k] = sub ? psub(xr[k], r) : padd(xr[k], r);
+        xi[k] = sub ? psub(xi[k], i) : padd(xi[k], i);
         lr[k] = make_float2(0.f, 0.f);
         li[k] = make_float2(0.f, 0.f);
     }
@@ -1116,7 +1125,7 @@ bk_status gram_impl(Field A, Field B, Field B2, int NB, const SysPart& p, double
             BK_CUDA_TRY(cudaGetLastError());
         }
     }
-    k_gram_finish<<<(NB * ne + 31) / 32, dim3(32, FIN_ROWS), 0, st>>>(part, nchunk, NB, p, (double2*)G, (double2*)G2);
+    k_gram_finish<<<(NB * ne + FIN_E - 1) / FIN_E, dim3(FIN_E, FIN_ROWS), 0, st>>>(part, nchunk, NB, p, (double2*)G, (double2*)G2);
     BK_CUDA_TRY(cudaGetLastError());
     return BK_OK;
 }
@@ -1134,8 +1143,8 @@ bk_status gram_dispatch(int prec, Field A, Field B, Field B2, int NB, const SysP
 }  // namespace
 
 // partial-sum rows of a Gram matrix over the active systems
-static int gram_chunks(const SysPart& p, int V) {
-    return max_active_L(p) <= ROWS_MAXL ? gram_row_chunks(V, row_tiles(p).n) : site_chunks(V);
+static int gram_chunks(int prec, const SysPart& p, int V) {
+    return max_active_L(p) <= ROWS_MAXL ? gram_row_chunks(prec, V, row_tiles(p)) : site_chunks(V);
 }
 
 size_t gram_partial_bytes(const SysPart& p, int V) {
@@ -1145,12 +1154,12 @@ size_t gram_partial_bytes(const SysPart& p, int V) {
 
 bk_status launch_gram(int prec, Field A, Field B, const SysPart& p, double* G, double* partial, int V,
                       cudaStream_t st) {
-    return gram_dispatch(prec, A, B, B, 1, p, G, nullptr, partial, gram_chunks(p, V), V, st);
+    return gram_dispatch(prec, A, B, B, 1, p, G, nullptr, partial, gram_chunks(prec, p, V), V, st);
 }
 
 bk_status launch_gram2(int prec, Field A, Field B, Field B2, const SysPart& p, double* G, double* G2,
                        double* partial, int V, cudaStream_t st) {
-    return gram_dispatch(prec, A, B, B2, 2, p, G, G2, partial, gram_chunks(p, V), V, st);
+    return gram_dispatch(prec, A, B, B2, 2, p, G, G2, partial, gram_chunks(prec, p, V), V, st);
 }
 
 bk_status launch_gram_slots(int prec, Field A, Field B, const SysPart& p, double* G, double* partial,
@@ -1160,7 +1169,7 @@ bk_status launch_gram_slots(int prec, Field A, Field B, const SysPart& p, double
         bk_set_error("Gram partial sums need %lld slots per site chunk, %lld available", ne, slots);
         return BK_ERR_INVALID_ARG;
     }
-    const int nchunk = (int)std::min<long long>(gram_chunks(p, V), slots / ne);
+    const int nchunk = (int)std::min<long long>(gram_chunks(prec, p, V), slots / ne);
     return gram_dispatch(prec, A, B, B, 1, p, G, nullptr, partial, nchunk, V, st);
 }
 
@@ -1211,7 +1220,7 @@ bk_status launch_coldot(int prec, int npair, const Field* A, const Field* B, int
 #undef BK_CD
 #undef BK_CD1
     BK_CUDA_TRY(cudaGetLastError());
-    k_coldot_finish<<<(npair * n + 31) / 32, dim3(32, FIN_ROWS), 0, st>>>(part, nchunk, npair, nq, n,
+    k_coldot_finish<<<(npair * n + FIN_E - 1) / FIN_E, dim3(FIN_E, FIN_ROWS), 0, st>>>(part, nchunk, npair, nq, n,
                                                                          (double2*)out + c0, ldo);
     BK_CUDA_TRY(cudaGetLastError());
     return BK_OK;
@@ -1219,7 +1228,10 @@ bk_status launch_coldot(int prec, int npair, const Field* A, const Field* B, int
 
 // grid rows of the updates (a function of the lattice alone: the fused norms
 // of a system whose update was skipped stay those of its last residual)
-int genop_norm_rows(int V) { return std::max(1, std::min(MAX_CHUNKS, (12 * V) / 16)); }
+int genop_norm_rows(int V) {
+    const int c = std::max(1, (12 * V) / 16);  // 16 rows a block and more
+    return c >= 304 ? 304 : (c >= 152 ? 152 : c);  // whole waves of one or two blocks an SM
+}
 
 bk_status launch_genop(int prec, const GenOp& g, int V, cudaStream_t st, bool* ynorm_done) {
     if (ynorm_done) *ynorm_done = false;
@@ -1258,7 +1270,7 @@ bk_status launch_genop(int prec, const GenOp& g, int V, cudaStream_t st, bool* y
 
 bk_status launch_norm_finish(const double* ynorm, int ncols, int c0, int n, double* out, int V, cudaStream_t st) {
     if (n <= 0) return BK_OK;
-    k_norm_finish<<<(n + 31) / 32, dim3(32, FIN_ROWS), 0, st>>>(ynorm, genop_norm_rows(V), ncols, c0, n, out);
+    k_norm_finish<<<(n + FIN_E - 1) / FIN_E, dim3(FIN_E, FIN_ROWS), 0, st>>>(ynorm, genop_norm_rows(V), ncols, c0, n, out);
     BK_CUDA_TRY(cudaGetLastError());
     return BK_OK;
 }
@@ -1287,7 +1299,7 @@ bk_status launch_xmy(int prec, Field X, const double* M, const double* c_dev, Fi
 bk_status launch_accum(Field X64, Field Xlo, int p0, int np, cudaStream_t st) {
     if (np <= 0) return BK_OK;
     const long long items = (long long)X64.V * np;
-    k_accum<<<(unsigned)((items + 127) / 128), 128, 0, st>>>(X64, Xlo, p0, np, 1.0, 1);
+    k_accum<<<(unsigned)((items + 127) / 128), 128, 0, st>>>(X64, Xlo, p0, np, 0, 1);
     BK_CUDA_TRY(cudaGetLastError());
     return BK_OK;
 }
@@ -1295,7 +1307,7 @@ bk_status launch_accum(Field X64, Field Xlo, int p0, int np, cudaStream_t st) {
 bk_status launch_sub_lo(Field X64, Field Ylo, int p0, int np, cudaStream_t st) {
     if (np <= 0) return BK_OK;
     const long long items = (long long)X64.V * np;
-    k_accum<<<(unsigned)((items + 127) / 128), 128, 0, st>>>(X64, Ylo, p0, np, -1.0, 0);
+    k_accum<<<(unsigned)((items + 127) / 128), 128, 0, st>>>(X64, Ylo, p0, np, 1, 0);
     BK_CUDA_TRY(cudaGetLastError());
     return BK_OK;
 }

@@ -144,12 +144,17 @@ __device__ __forceinline__ void store_at(const Field& f, size_t e, typename Prec
     }
 }
 
-// complex coefficient mult * (ptr ? ptr[s] : 1)
+// complex coefficient mult * (ptr ? ptr[s] : 1); unit: 1 or -1 when mult is that
 template <int P>
-__device__ __forceinline__ cx<typename Prec<P>::real> coef(const double* ptr, double mult, int s) {
+__device__ __forceinline__ cx<typename Prec<P>::real> coef(const double* ptr, double mult, int unit, int s) {
     using R = typename Prec<P>::real;
-    if (ptr) return mk((R)(mult * ptr[2 * s]), (R)(mult * ptr[2 * s + 1]));
-    return mk((R)mult, R(0));
+    if (!ptr) return mk(d2r<R>(mult), R(0));
+    double re = __ldg(ptr + 2 * s), im = __ldg(ptr + 2 * s + 1);
+    if (unit == 0) {
+        re *= mult;
+        im *= mult;
+    }
+    return unit < 0 ? mk(d2r<R>(-re), d2r<R>(-im)) : mk(d2r<R>(re), d2r<R>(im));
 }
 
 // FP32 products are summed in FP32 over at most this many (site, component)
@@ -158,12 +163,20 @@ constexpr int ROW_FLUSH = 96;
 
 // rows.cu: systems of at most ROWS_MAXL columns
 constexpr int ROWS_MAXL = 12;
-// site chunks (partial-sum rows) of the row Gram kernel over nt tiles
-inline int gram_row_chunks(int V, int nt) {
-    const int most = std::max(1, std::min((12 * V) / 16, 608));
-    return std::max(std::min(most, 76), most / std::max(1, nt));
+// Row chunks (grid.y, partial-sum rows) of the row Gram kernel.  FP64: a chunk
+// per 4 warp steps, so that a small lattice still fills every SM's FP64 pipe
+// (4^4, 12 columns: 615 steps).  FP32 / FP16: a chunk per 64 steps, 8 a warp,
+// since there a block's fixed costs (FP64 conversions, the finishing sums)
+// outweigh a few more rows.  At most the blocks that are resident at once
+// (FP64: 1 an SM, else 2), over all tiles: a 153rd block would double the time.
+inline int gram_row_chunks(int prec, int V, const PTiles& t) {
+    int spw = 32;
+    for (int i = 0; i < t.n; ++i) spw = std::min(spw, 32 / std::max(1, t.np[i]));
+    const int steps = (12 * V) / std::max(1, spw);
+    const int most = std::max(76, (prec == BK_FP64 ? 152 : 304) / std::max(1, t.n));
+    return std::max(1, std::min(steps / (prec == BK_FP64 ? 4 : 64), most));
 }
-inline int gram_row_chunks_max(int V) { return gram_row_chunks(V, 1); }
+inline int gram_row_chunks_max(int V) { return std::max(1, std::min(12 * V / 4, 304)); }
 bk_status rows_gram(int prec, Field A, Field B, Field B2, int NB, const SysPart& p, double2* partial, int nchunk,
                     int V, cudaStream_t st);
 PTiles row_tiles(const SysPart& p);

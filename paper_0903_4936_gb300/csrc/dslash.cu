@@ -750,12 +750,37 @@ __device__ __forceinline__ void project(const cx<R> (&q)[12], cx<R> (&h)[6]) {
     }
 }
 
-template <int MU, int S, typename R>
+// FIRST: acc is taken as zero (the first hop sets it, 24 additions saved)
+template <int MU, int S, bool FIRST, typename R>
 __device__ __forceinline__ void reconstruct(const cx<R> (&w)[6], cx<R> (&acc)[12]) {
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         const cx<R> w0 = w[a], w1 = w[3 + a];
-        if constexpr (MU == 0) {
+        if constexpr (FIRST) {
+            static_assert(!FIRST || S < 0, "the first hop is a forward one");
+            const R two = R(2), zero = R(0);
+            if constexpr (MU == 0) {
+                acc[a] = w0;
+                acc[3 + a] = w1;
+                acc[6 + a] = mk(w1.i, -w1.r);
+                acc[9 + a] = mk(w0.i, -w0.r);
+            } else if constexpr (MU == 1) {
+                acc[a] = w0;
+                acc[3 + a] = w1;
+                acc[6 + a] = mk(-w1.r, -w1.i);
+                acc[9 + a] = w0;
+            } else if constexpr (MU == 2) {
+                acc[a] = w0;
+                acc[3 + a] = w1;
+                acc[6 + a] = mk(w0.i, -w0.r);
+                acc[9 + a] = mk(-w1.i, w1.r);
+            } else {
+                acc[a] = mk(zero, zero);
+                acc[3 + a] = mk(zero, zero);
+                acc[6 + a] = two * w0;
+                acc[9 + a] = two * w1;
+            }
+        } else if constexpr (MU == 0) {
             acc[a] = acc[a] + w0;
             acc[3 + a] = acc[3 + a] + w1;
             acc[6 + a] = S > 0 ? acc[6 + a] + ti(w1) : acc[6 + a] - ti(w1);
@@ -793,7 +818,7 @@ __device__ __forceinline__ void load_link(const L* __restrict__ U, int mu, int s
 }
 
 // HALF: the input x is a half-lattice (one parity) block, site n at index n >> 1
-template <int P, int MU, bool HALF = false, typename Args>
+template <int P, int MU, bool HALF, bool FIRST, typename Args>
 __device__ __forceinline__ void hop_dir_col(const Args& a, const int (&co)[4], int n, int c,
                                             cx<typename Prec<P>::real> (&acc)[12]) {
     using R = typename Prec<P>::real;
@@ -815,7 +840,7 @@ __device__ __forceinline__ void hop_dir_col(const Args& a, const int (&co)[4], i
                 cmac(t, u[3 * i + 2], h[3 * hh + 2]);
                 w[3 * hh + i] = t;
             }
-        reconstruct<MU, -1>(w, acc);
+        reconstruct<MU, -1, FIRST>(w, acc);
     }
     {   // backward: (1 + gamma_mu) U_mu(n - mu)^+ x(n - mu)
         cx<R> u[9], q[12], h[6], w[6];
@@ -832,7 +857,7 @@ __device__ __forceinline__ void hop_dir_col(const Args& a, const int (&co)[4], i
                 cjmac(t, u[6 + i], h[3 * hh + 2]);
                 w[3 * hh + i] = t;
             }
-        reconstruct<MU, +1>(w, acc);
+        reconstruct<MU, +1, false>(w, acc);
     }
 }
 
@@ -871,12 +896,10 @@ __global__ void __launch_bounds__(128) k_dslash_col(const __grid_constant__ DCol
         co[3] = r / a.L[2];
     }
     cx<R> acc[12];
-#pragma unroll
-    for (int k = 0; k < 12; ++k) acc[k] = mk(R(0), R(0));
-    hop_dir_col<P, 0>(a, co, n, c, acc);
-    hop_dir_col<P, 1>(a, co, n, c, acc);
-    hop_dir_col<P, 2>(a, co, n, c, acc);
-    hop_dir_col<P, 3>(a, co, n, c, acc);
+    hop_dir_col<P, 0, false, true>(a, co, n, c, acc);
+    hop_dir_col<P, 1, false, false>(a, co, n, c, acc);
+    hop_dir_col<P, 2, false, false>(a, co, n, c, acc);
+    hop_dir_col<P, 3, false, false>(a, co, n, c, acc);
     cx<R> q[12];
     load_col<P>(a.x, n, c, q);
     // clover: the chiral blocks act on a = u + l (block 0) and b = u - l (block 1)
@@ -910,6 +933,101 @@ __global__ void __launch_bounds__(128) k_dslash_col(const __grid_constant__ DCol
         for (int k = 0; k < 12; ++k) out[k] = bb[k] - out[k];
     }
     store_col<P>(a.y, n, c, out);
+}
+
+// Rows 3 H .. 3 H + 2 of chiral block BLK times v (Hermitian, packed as herm6).
+template <int BLK, int H>
+__device__ __forceinline__ void herm6_rows(const double2* __restrict__ C, int V, int n, const cx<double> (&v)[6],
+                                           cx<double> (&y)[3]) {
+    const double* c = reinterpret_cast<const double*>(C);
+    auto real_at = [&](int e) {  // packed real e of this block
+        const int q = 36 * BLK + e;
+        return __ldg(c + 2 * ((size_t)(q >> 1) * V + n) + (q & 1));
+    };
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        const int i = 3 * H + r;
+        y[r] = real_at(i) * v[i];
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+            if (j == i) continue;
+            const int hi = i > j ? i : j, lo = i > j ? j : i, e = 6 + 2 * (hi * (hi - 1) / 2 + lo);
+            const cx<double> A = mk(real_at(e), real_at(e + 1));
+            if (i > j) cmac(y[r], A, v[j]);
+            else cjmac(y[r], A, v[j]);
+        }
+    }
+}
+
+// FP64 operator for few site-columns: four warps share 32 of them, warp t
+// takes the two hops of direction t and three rows of one chiral block of the
+// clover term, and finishes spin t.  An SM's scheduler starts an FP64
+// instruction of a warp every 64 cycles, so one thread per site and column
+// (about 1000 of them) needs 33 us however few there are; a quarter of that
+// each, on four times the warps, is faster while they do not fill the chip's
+// 608 schedulers about twice (see dslash_col_impl).
+__global__ void __launch_bounds__(128) k_dslash_col4(const __grid_constant__ DColArgs<BK_FP64> a) {
+    __shared__ double hs[4][24][32], ys[4][6][32];
+    const int t = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long long g = (long long)blockIdx.x * 32 + lane;
+    const bool on = g < (long long)a.V * a.ncl;
+    const int n = on ? (int)(g / a.ncl) : 0;
+    const int cl = on ? (int)(g - (long long)n * a.ncl) : 0;
+    const int c = a.c0 + cl;
+    int co[4];
+    {
+        int r = n;
+        co[0] = r % a.L[0];
+        r /= a.L[0];
+        co[1] = r % a.L[1];
+        r /= a.L[1];
+        co[2] = r % a.L[2];
+        co[3] = r / a.L[2];
+    }
+    if (on) {
+        cx<double> acc[12];
+        if (t == 0) hop_dir_col<BK_FP64, 0, false, true>(a, co, n, c, acc);
+        else if (t == 1) hop_dir_col<BK_FP64, 1, false, true>(a, co, n, c, acc);
+        else if (t == 2) hop_dir_col<BK_FP64, 2, false, true>(a, co, n, c, acc);
+        else hop_dir_col<BK_FP64, 3, false, true>(a, co, n, c, acc);
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            hs[t][2 * k][lane] = acc[k].r;
+            hs[t][2 * k + 1][lane] = acc[k].i;
+        }
+        cx<double> q[12], v[6], y[3];
+        load_col<BK_FP64>(a.x, n, c, q);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) v[k] = t < 2 ? q[k] + q[k + 6] : q[k] - q[k + 6];
+        if (t == 0) herm6_rows<0, 0>(a.C, a.V, n, v, y);
+        else if (t == 1) herm6_rows<0, 1>(a.C, a.V, n, v, y);
+        else if (t == 2) herm6_rows<1, 0>(a.C, a.V, n, v, y);
+        else herm6_rows<1, 1>(a.C, a.V, n, v, y);
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            ys[t][2 * r][lane] = y[r].r;
+            ys[t][2 * r + 1][lane] = y[r].i;
+        }
+    }
+    __syncthreads();
+    if (!on) return;
+    const int h = t & 1;  // spin t = h + 2 (t >> 1): row h of u (t < 2) or of l
+    const size_t e0 = 4 * (((size_t)n * 12 + 3 * t) * a.x.np + (c >> 1)) + (c & 1), es = 4 * (size_t)a.x.np;
+    const double* xq = (const double*)a.x.data + e0;
+    const double* bq = (const double*)a.b.data + e0;
+    double* yq = (double*)a.y.data + e0;
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            const int k = 2 * (3 * t + r) + p;
+            double s = (hs[0][k][lane] + hs[1][k][lane]) + (hs[2][k][lane] + hs[3][k][lane]);
+            const double y0 = ys[h][2 * r + p][lane], y1 = ys[2 + h][2 * r + p][lane];
+            s += t < 2 ? y0 + y1 : y0 - y1;
+            double o = xq[r * es + 2 * p] - a.kappa[cl] * s;
+            if (a.residual) o = bq[r * es + 2 * p] - o;
+            yq[r * es + 2 * p] = o;
+        }
 }
 
 void geometry(const int dims[4], int (&L)[4], int (&st)[4]) {
@@ -987,6 +1105,12 @@ bk_status dslash_pair_impl(const DslashOp& op, cudaStream_t st) {
     return BK_OK;
 }
 
+// Threads per block of the one-column-per-thread kernels.  Their FP64 pipe
+// works at full rate with few warps, so what matters is that every scheduler
+// has the same number: single-warp blocks up to 16 warps a scheduler, two-warp
+// blocks above.
+int col_threads(long long items) { return items <= 608LL * 16 * 32 ? 32 : 64; }
+
 template <int P>
 bk_status dslash_col_impl(const DslashOp& op, cudaStream_t st) {
     for (int c0 = 0; c0 < op.ncol; c0 += BK_MAX_COLS) {
@@ -1003,8 +1127,15 @@ bk_status dslash_col_impl(const DslashOp& op, cudaStream_t st) {
         a.ncl = n;
         a.residual = op.residual;
         for (int j = 0; j < n; ++j) a.kappa[j] = op.kappa[c0 + j];
-        const int threads = op.threads > 0 ? std::min(op.threads, 128) : 128;
         const long long items = (long long)op.V * n;
+        if constexpr (P == BK_FP64) {
+            if (items <= 608LL * 2 * 32 && op.x.np == op.y.np && (!op.residual || op.b.np == op.x.np)) {
+                k_dslash_col4<<<(unsigned)((items + 31) / 32), 128, 0, st>>>(a);
+                BK_CUDA_TRY(cudaGetLastError());
+                continue;
+            }
+        }
+        const int threads = col_threads(items);
         k_dslash_col<P><<<(unsigned)((items + threads - 1) / threads), threads, 0, st>>>(a);
         BK_CUDA_TRY(cudaGetLastError());
     }
@@ -1120,10 +1251,16 @@ __global__ void k_cast(Field in, Field out, int np) {
     typename Prec<PO>::pair ro[12], io[12];
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
-        ro[k].x = r[k].x;
-        ro[k].y = r[k].y;
-        io[k].x = i[k].x;
-        io[k].y = i[k].y;
+        if constexpr (PI == BK_FP64 && PO != BK_FP64) {
+            ro[k] = d2f(r[k]);
+            io[k] = d2f(i[k]);
+        } else if constexpr (PI != BK_FP64 && PO == BK_FP64) {
+            ro[k] = f2d(r[k]);
+            io[k] = f2d(i[k]);
+        } else {
+            ro[k] = r[k];
+            io[k] = i[k];
+        }
     }
     store_pair<PO>(out, n, p, ro, io);
 }
@@ -1412,10 +1549,10 @@ __global__ void __launch_bounds__(128) k_eo_col(const __grid_constant__ EOColArg
 #pragma unroll
     for (int k = 0; k < 12; ++k) acc[k] = mk(R(0), R(0));
     if (a.hop) {
-        hop_dir_col<P, 0, true>(a, co, n, c, acc);
-        hop_dir_col<P, 1, true>(a, co, n, c, acc);
-        hop_dir_col<P, 2, true>(a, co, n, c, acc);
-        hop_dir_col<P, 3, true>(a, co, n, c, acc);
+        hop_dir_col<P, 0, true, true>(a, co, n, c, acc);
+        hop_dir_col<P, 1, true, false>(a, co, n, c, acc);
+        hop_dir_col<P, 2, true, false>(a, co, n, c, acc);
+        hop_dir_col<P, 3, true, false>(a, co, n, c, acc);
     }
     const R kap = (R)a.kappa[cl];
     cx<R> xs[12];
@@ -1582,7 +1719,8 @@ bk_status eo_col_impl(const EoOp& op, cudaStream_t st) {
             a.Ci[j] = (const typename Prec<P>::clov*)op.Ci[c0 + j];
         }
         const long long items = (long long)a.Vh * n;
-        k_eo_col<P><<<(unsigned)((items + 127) / 128), 128, 0, st>>>(a);
+        const int threads = col_threads(items);
+        k_eo_col<P><<<(unsigned)((items + threads - 1) / threads), threads, 0, st>>>(a);
         BK_CUDA_TRY(cudaGetLastError());
     }
     return BK_OK;

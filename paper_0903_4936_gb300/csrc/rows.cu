@@ -44,24 +44,32 @@ __device__ __forceinline__ RLane rlane(const SysPart& p, int tp0, int tnp, int l
 // ---------------------------------------------------------------- Gram
 //
 // G_s = A_s^H B_s (NB = 2: and A_s^H B1_s).  A lane adds conj(A_i) B_j for its
-// two columns i and every column j of its system.  FP32 / FP16 products are
-// summed in FP32 registers (packed pairs over j) and moved every ROW_FLUSH
-// rows into the lane's own FP64 accumulators in shared memory; the block adds
-// its lanes' accumulators at the end and writes one partial row per chunk.
-// UR row groups are loaded before the first is used.
+// two columns i and every column j of its system.  UR row groups are loaded
+// before the first is used.  The block adds its warps' sums at the end and
+// writes one partial row per chunk.
+//
+// FP32 / FP16 products are summed in FP32 registers (packed pairs over j).
+// Every ROW_FLUSH rows these go to FP64 accumulators in shared memory; with
+// several rows side by side (spw > 1) the lanes of one column pair are added
+// in FP32 first, so that the conversion and the FP64 add, 16 cycles of the
+// SM's FP64 pipe per warp instruction, are done once per entry by a full warp
+// instead of once per lane.
+// FP64 sums stay in registers and are added over the rows in the tail.
 
 template <int P, int NB, int MAXL, int UR>
-__global__ void __launch_bounds__(GW * 32, P == BK_FP64 ? 1 : 2) k_gram_r(Field A, Field B0, Field B1, SysPart p, PTiles wt,
-                                                    double2* __restrict__ partial, unsigned rows, int nchunk) {
+__global__ void __launch_bounds__(GW * 32, P == BK_FP64 ? 1 : 2) k_gram_r(Field A, Field B0, Field B1, SysPart p,
+                                                                         PTiles wt, double2* __restrict__ partial,
+                                                                         unsigned rows, int nchunk) {
     using R2 = typename Prec<P>::pair;
     constexpr int NACC = NB * 2 * MAXL;
-    extern __shared__ double2 gr_acc[];  // [warp][entry][lane]
+    extern __shared__ double2 gr_acc[];  // [warp][NACC * 32]
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int chunk = blockIdx.y;
     const int tp0 = wt.p0[blockIdx.x], tnp = wt.np[blockIdx.x];
     const int spw = 32 / tnp, np = A.np;
     const RLane L = rlane(p, tp0, tnp, lane);
-    double2* my = gr_acc + (size_t)w * NACC * 32 + lane;
+    double2* my = gr_acc + (size_t)w * NACC * 32;
+    float2* stage = reinterpret_cast<float2*>(my + NACC * 16);  // spw > 1: accumulators fill at most the first half
     CxPair<R2> acc[NB][2][MAXL / 2];
 #pragma unroll
     for (int b = 0; b < NB; ++b)
@@ -73,6 +81,7 @@ __global__ void __launch_bounds__(GW * 32, P == BK_FP64 ? 1 : 2) k_gram_r(Field 
     bool first = true;
     int since = 0;
     auto flush = [&]() {
+        const bool staged = P != BK_FP64 && spw > 1;
 #pragma unroll
         for (int b = 0; b < NB; ++b)
 #pragma unroll
@@ -82,13 +91,29 @@ __global__ void __launch_bounds__(GW * 32, P == BK_FP64 ? 1 : 2) k_gram_r(Field 
                     CxPair<R2>& c = acc[b][ii][jp];
 #pragma unroll
                     for (int jj = 0; jj < 2; ++jj) {
-                        double2& v = my[((b * 2 + ii) * MAXL + 2 * jp + jj) * 32];
-                        const double re = (double)(jj ? c.re.y : c.re.x), im = (double)(jj ? c.im.y : c.im.x);
-                        if (first) v = make_double2(re, im);
-                        else v = make_double2(v.x + re, v.y + im);
+                        const int e = (b * 2 + ii) * MAXL + 2 * jp + jj;
+                        const auto re = jj ? c.re.y : c.re.x, im = jj ? c.im.y : c.im.x;
+                        if (staged) {
+                            stage[e * 32 + lane] = make_float2((float)re, (float)im);
+                        } else {
+                            double2& v = my[e * 32 + lane];
+                            if (first) v = make_double2(f2d(re), f2d(im));
+                            else v = make_double2(v.x + f2d(re), v.y + f2d(im));
+                        }
                     }
                     c = cp_zero<R2>();
                 }
+        if (staged) {
+            __syncwarp();
+            for (int x = lane; x < NACC * tnp; x += 32) {
+                const int e = x / tnp, pr = x - e * tnp;
+                float2 v = stage[e * 32 + pr];
+                for (int sub = 1; sub < spw; ++sub) v = padd(v, stage[e * 32 + sub * tnp + pr]);
+                if (first) my[x] = make_double2(f2d(v.x), f2d(v.y));
+                else my[x] = make_double2(my[x].x + f2d(v.x), my[x].y + f2d(v.y));
+            }
+            __syncwarp();
+        }
         first = false;
         since = 0;
     };
@@ -142,19 +167,20 @@ __global__ void __launch_bounds__(GW * 32, P == BK_FP64 ? 1 : 2) k_gram_r(Field 
             if (since >= ROW_FLUSH) flush();
         }
     }
-    if (first || since > 0 || P == BK_FP64) flush();
+    if (wid < units && (first || since > 0)) flush();
     __syncthreads();
-    // the block's partial sums: one thread per (pair, operand, column of the pair, column)
+    // the block's partial sums: one thread per (operand, column of the pair, column, pair)
     const int ne = p.coef_off[p.nsys];
     const int nact = min(GW, (int)((units - min(units, (unsigned)chunk) + nchunk - 1) / nchunk));  // warps with rows
+    const int estr = P == BK_FP64 || spw == 1 ? 32 : tnp, nsub = P == BK_FP64 ? spw : 1;
     for (int x = threadIdx.x; x < tnp * NACC; x += GW * 32) {
-        const int j = x % MAXL, ii = (x / MAXL) & 1, b = (x / (2 * MAXL)) % NB, pr = x / NACC;
+        const int e = x / tnp, pr = x - e * tnp, j = e % MAXL, ii = (e / MAXL) & 1, b = e / (2 * MAXL);
         const int s = sys_of_pair(p, tp0 + pr), Ls = p.L[s], i = 2 * (tp0 + pr) - p.col0[s] + ii;
         if (i >= Ls || j >= Ls) continue;
         double2 v = make_double2(0.0, 0.0);
         for (int ww = 0; ww < nact; ++ww)
-            for (int sub = 0; sub < spw; ++sub) {
-                const double2 a = gr_acc[((size_t)ww * NACC + (b * 2 + ii) * MAXL + j) * 32 + sub * tnp + pr];
+            for (int sub = 0; sub < nsub; ++sub) {
+                const double2 a = gr_acc[(size_t)ww * NACC * 32 + e * estr + sub * tnp + pr];
                 v.x += a.x;
                 v.y += a.y;
             }
@@ -226,44 +252,48 @@ __global__ void __launch_bounds__(GW * 32, MINB) k_update_r(const __grid_constan
     const RLane L = rlane(g.p, tp0, tnp, lane);
     const bool act = L.live && !(g.skip && g.skip[L.s]);
     const int s = L.s;
-    const bool mat = nmi > 0 && g.M != nullptr && ((g.hasY && g.ym != 0.0) || (hx && g.xm != 0.0));
+    const bool mat = g.mat != 0;
     cx<R> ea[ME > 0 ? ME : 1], ma[MMI > 0 ? MMI : 1], xa = mk(R(0), R(0));
-    bool eunit[ME > 0 ? ME : 1];
+    int ekind[ME > 0 ? ME : 1];  // coefficient of E_t: 1, -1 (adds) or general
 #pragma unroll
     for (int e = 0; e < ME; ++e) {
-        ea[e] = e < ne ? coef<P>(g.ea[e], g.ea_mult[e], s) : mk(R(0), R(0));
-        eunit[e] = e < ne && g.ea[e] == nullptr && g.ea_mult[e] == 1.0;
+        ea[e] = e < ne ? coef<P>(g.ea[e], g.ea_mult[e], g.ea_unit[e], s) : mk(R(0), R(0));
+        ekind[e] = e < ne && g.ea[e] == nullptr ? g.ea_unit[e] : 0;
     }
 #pragma unroll
-    for (int u = 0; u < MMI; ++u) ma[u] = u < nmi ? coef<P>(g.ma[u], g.ma_mult[u], s) : mk(R(0), R(0));
-    const bool munit = nmi == 1 || (g.ma[0] == nullptr && g.ma_mult[0] == 1.0);
-    if (hx) xa = coef<P>(g.xa, g.xa_mult, s);
+    for (int u = 0; u < MMI; ++u) ma[u] = u < nmi ? coef<P>(g.ma[u], g.ma_mult[u], g.ma_unit[u], s) : mk(R(0), R(0));
+    const bool munit = nmi == 1 || (g.ma[0] == nullptr && g.ma_unit[0] == 1);
+    if (hx) xa = coef<P>(g.xa, g.xa_mult, g.xa_unit, s);
     // the lane's two columns of M; rows and columns past the system's size are zero
     R2 Mr[MAXL], Mi[MAXL];
     {
         const double2* M = reinterpret_cast<const double2*>(g.M) + (act && mat ? g.p.coef_off[s] : 0);
         const bool j1ok = L.i0 + 1 < L.Ls;
-        cx<double> f = mk(1.0, 0.0);
-        if (nmi == 1 && mat) f = coef<BK_FP64>(g.ma[0], g.ma_mult[0], s);
+        // one operand: its coefficient goes into M (a real one as a factor, +-1 without arithmetic)
+        const bool fold = nmi == 1 && mat, fcx = fold && g.ma[0] != nullptr;
+        const double fr = fold ? g.ma_mult[0] : 1.0;
+        const cx<double> f = fcx ? coef<BK_FP64>(g.ma[0], g.ma_mult[0], g.ma_unit[0], s) : mk(fr, 0.0);
+        auto times_f = [&](double2 a) {
+            if (fcx) return f * mk(a.x, a.y);
+            if (!fold || g.ma_unit[0] == 1) return mk(a.x, a.y);
+            if (g.ma_unit[0] == -1) return mk(-a.x, -a.y);
+            return mk(fr * a.x, fr * a.y);
+        };
 #pragma unroll
         for (int i = 0; i < MAXL; ++i) {
             cx<double> m0 = mk(0.0, 0.0), m1 = mk(0.0, 0.0);
             if (act && mat && i < L.Ls) {
-                const double2 a = M[i * L.Ls + L.i0];
-                m0 = f * mk(a.x, a.y);
-                if (j1ok) {
-                    const double2 b = M[i * L.Ls + L.i0 + 1];
-                    m1 = f * mk(b.x, b.y);
-                }
+                m0 = times_f(__ldg(M + i * L.Ls + L.i0));
+                if (j1ok) m1 = times_f(__ldg(M + i * L.Ls + L.i0 + 1));
             }
-            Mr[i].x = (R)m0.r;
-            Mr[i].y = (R)m1.r;
-            Mi[i].x = (R)m0.i;
-            Mi[i].y = (R)m1.i;
+            Mr[i].x = d2r<R>(m0.r);
+            Mr[i].y = d2r<R>(m1.r);
+            Mi[i].x = d2r<R>(m0.i);
+            Mi[i].y = d2r<R>(m1.i);
         }
     }
-    const bool yunit = g.ym == 1.0, xunit = g.xm == 1.0;
-    const R2 ym2 = bcast((R)g.ym), xm2 = bcast((R)g.xm);
+    const bool yunit = g.y_unit == 1, xunit = g.x_unit == 1;
+    const R2 ym2 = bcast(d2r<R>(g.ym)), xm2 = bcast(d2r<R>(g.xm));
     double yn0 = 0.0, yn1 = 0.0;
     R sa = R(0), sb = R(0);
     int since = 0;
@@ -331,9 +361,14 @@ __global__ void __launch_bounds__(GW * 32, MINB) k_update_r(const __grid_constan
 #pragma unroll
                 for (int t = 0; t < ME; ++t)
                     if (t < ne) {
-                        if (eunit[t]) {
+                        if (t == 0 && !mat && ekind[0] == 1) {
+                            y = ve[x][0];
+                        } else if (ekind[t] == 1) {
                             y.re = padd(y.re, ve[x][t].re);
                             y.im = padd(y.im, ve[x][t].im);
+                        } else if (ekind[t] == -1) {
+                            y.re = psub(y.re, ve[x][t].re);
+                            y.im = psub(y.im, ve[x][t].im);
                         } else {
                             cpair_mac<R, R2>(y, ea[t], ve[x][t]);
                         }
@@ -362,14 +397,14 @@ __global__ void __launch_bounds__(GW * 32, MINB) k_update_r(const __grid_constan
         // FP32 squares of at most 12 rows per FP32 sum, then FP64
         since += UR;
         if (g.ynorm && since >= 12) {
-            yn0 += (double)sa;
-            yn1 += (double)sb;
+            yn0 += f2d(sa);
+            yn1 += f2d(sb);
             sa = sb = R(0);
             since = 0;
         }
     }
     if (g.ynorm) {
-        ynred[w][lane] = make_double2(yn0 + (double)sa, yn1 + (double)sb);
+        ynred[w][lane] = make_double2(yn0 + f2d(sa), yn1 + f2d(sb));
         __syncthreads();
         if (act && threadIdx.x < tnp) {
             double2 v = make_double2(0.0, 0.0);
@@ -416,7 +451,16 @@ bk_status rows_gram(int prec, Field A, Field B, Field B2, int NB, const SysPart&
     return BK_ERR_INVALID_ARG;
 }
 
-bk_status rows_update(int prec, const GenOp& g, int V, int nchunk, int np, cudaStream_t st) {
+bk_status rows_update(int prec, const GenOp& g0, int V, int nchunk, int np, cudaStream_t st) {
+    // what the kernel would otherwise find out with FP64 comparisons
+    GenOp g = g0;
+    auto unit = [](double x) { return x == 1.0 ? 1 : (x == -1.0 ? -1 : 0); };
+    for (int e = 0; e < GENOP_MAXE; ++e) g.ea_unit[e] = unit(g.ea_mult[e]);
+    for (int u = 0; u < GENOP_MAXMI; ++u) g.ma_unit[u] = unit(g.ma_mult[u]);
+    g.xa_unit = unit(g.xa_mult);
+    g.y_unit = unit(g.ym);
+    g.x_unit = unit(g.xm);
+    g.mat = g.nmi > 0 && g.M != nullptr && ((g.hasY && g.ym != 0.0) || (g.hasX && g.xm != 0.0));
     const PTiles wt = row_tiles(g.p);
     const dim3 grid(wt.n, nchunk);
     const int ncols = g.p.col0[g.p.nsys];
