@@ -44,7 +44,6 @@ constexpr int TILE_MAXP = 64;
 // Site chunks of the reductions and updates: grid.y, independent of the
 // tiles so that per-chunk partial sums have a fixed row count for a lattice.
 constexpr int MAX_CHUNKS = 304;  // 2 per SM of 152
-inline int site_chunks(int V) { return std::max(1, std::min(MAX_CHUNKS, V / 64)); }
 
 // element store (FP32 / FP64 pair layouts)
 template <int P>
@@ -100,123 +99,9 @@ __device__ __forceinline__ WLane wlane(const SysPart& p, int tp0, int tnp, int l
     return w;
 }
 
-constexpr int GS_FLUSH = 8;  // sites per FP32 sum
 constexpr int GW_WARPS = 8;
 
-// ---------------------------------------------------------------- Gram, any system size
-//
-// One thread block per (system, range of 256 output tiles, site chunk); an
-// output tile is 4 x 4 columns (2 pairs of A x 2 pairs of B).  The block
-// stages the system's rows of A and B for SRB sites in shared memory, then
-// each thread adds its 16 products per site and component.
-
-struct BigWork {
-    int n;
-    int sys[256];
-    int t0[256];
-};
-
-template <int P>
-__global__ void __launch_bounds__(256) k_gram_big(Field A, Field B, SysPart p, BigWork w,
-                                                  double2* __restrict__ partial, int V, int nchunk, int SRB) {
-    using R = typename Prec<P>::real;
-    using R2 = typename Prec<P>::pair;
-    constexpr int FL = P == BK_FP64 ? (1 << 30) : GS_FLUSH;
-    extern __shared__ __align__(16) unsigned char gb_smem[];
-    const int s = w.sys[blockIdx.x];
-    const int chunk = blockIdx.y;
-    const int Ls = p.L[s], nps = (Ls + 1) / 2, side = (nps + 1) / 2;
-    const int qs = p.col0[s] / 2;
-    CxPair<R2>* As = reinterpret_cast<CxPair<R2>*>(gb_smem);  // [SRB][12][nps]
-    CxPair<R2>* Bs = As + (size_t)SRB * 12 * nps;
-    const int tile = w.t0[blockIdx.x] + threadIdx.x;
-    const bool on = tile < side * side;
-    const int ti = on ? tile / side : 0, tj = on ? tile % side : 0;
-    cx<R> acc[4][4];
-    double2 acc64[4][4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            acc[a][b] = mk(R(0), R(0));
-            acc64[a][b] = make_double2(0.0, 0.0);
-        }
-    const int iters = (V + SRB * nchunk - 1) / (SRB * nchunk);
-    for (int it = 0; it < iters; ++it) {
-        const int nbase = (it * nchunk + chunk) * SRB;
-        for (int e = threadIdx.x; e < SRB * nps; e += blockDim.x) {
-            const int rr = e / nps, qq = e % nps, n = nbase + rr;
-            if (n < V) {
-                R2 xr[12], xi[12];
-                load_pair<P>(A, n, qs + qq, xr, xi);
-#pragma unroll
-                for (int k = 0; k < 12; ++k) {
-                    CxPair<R2> v;
-                    v.re = xr[k];
-                    v.im = xi[k];
-                    As[(rr * 12 + k) * nps + qq] = v;
-                }
-                load_pair<P>(B, n, qs + qq, xr, xi);
-#pragma unroll
-                for (int k = 0; k < 12; ++k) {
-                    CxPair<R2> v;
-                    v.re = xr[k];
-                    v.im = xi[k];
-                    Bs[(rr * 12 + k) * nps + qq] = v;
-                }
-            }
-        }
-        __syncthreads();
-        if (on) {
-            for (int rr = 0; rr < SRB && nbase + rr < V; ++rr) {
-                for (int k = 0; k < 12; ++k) {
-                    CxPair<R2> a2[2], b2[2];
-#pragma unroll
-                    for (int u = 0; u < 2; ++u) {
-                        const int qa = 2 * ti + u, qb = 2 * tj + u;
-                        a2[u] = As[(rr * 12 + k) * nps + (qa < nps ? qa : 0)];
-                        b2[u] = Bs[(rr * 12 + k) * nps + (qb < nps ? qb : 0)];
-                    }
-#pragma unroll
-                    for (int ia = 0; ia < 4; ++ia) {
-                        const R xr = (ia & 1) ? a2[ia >> 1].re.y : a2[ia >> 1].re.x;
-                        const R xi = (ia & 1) ? a2[ia >> 1].im.y : a2[ia >> 1].im.x;
-#pragma unroll
-                        for (int ib = 0; ib < 4; ++ib) {
-                            const R yr = (ib & 1) ? b2[ib >> 1].re.y : b2[ib >> 1].re.x;
-                            const R yi = (ib & 1) ? b2[ib >> 1].im.y : b2[ib >> 1].im.x;
-                            cx<R>& c = acc[ia][ib];
-                            c.r = fma(xr, yr, c.r);
-                            c.r = fma(xi, yi, c.r);
-                            c.i = fma(xr, yi, c.i);
-                            c.i = fma(-xi, yr, c.i);
-                        }
-                    }
-                }
-            }
-        }
-        __syncthreads();
-        if ((it % FL) == FL - 1 || it == iters - 1) {
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    acc64[a][b].x += (double)acc[a][b].r;
-                    acc64[a][b].y += (double)acc[a][b].i;
-                    acc[a][b] = mk(R(0), R(0));
-                }
-        }
-    }
-    if (!on) return;
-    const int ne = p.coef_off[p.nsys];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            const int i = 4 * ti + a, j = 4 * tj + b;
-            if (i < Ls && j < Ls) partial[(size_t)chunk * ne + p.coef_off[s] + i * Ls + j] = acc64[a][b];
-        }
-}
+// ---------------------------------------------------------------- finishing sums
 
 // Sums over the chunks' partial rows: FIN_E entries x FIN_ROWS row slices per
 // block (a thread adds every FIN_ROWS-th row), combined in shared memory in a
@@ -421,7 +306,7 @@ __global__ void __launch_bounds__(256) k_genop(const __grid_constant__ GenOp g, 
     using XR = typename Prec<XP>::real;
     using X2 = typename Prec<XP>::pair;
     __shared__ double2 ynred[SR][TILE_MAXP];
-    const int t = threadIdx.x, r = threadIdx.y;
+    const int tx = threadIdx.x, t = tx + (int)blockIdx.z * TILE_MAXP, r = threadIdx.y;  // systems wider than a tile: grid.z
     const int tile = blockIdx.x, chunk = blockIdx.y;
     const int tp0 = tl.p0[tile], tnp = tl.np[tile];
     bool on = t < tnp;
@@ -561,13 +446,13 @@ __global__ void __launch_bounds__(256) k_genop(const __grid_constant__ GenOp g, 
         yn[1] += (double)sb;
     }
     if (g.ynorm) {
-        ynred[r][t] = make_double2(yn[0], yn[1]);
+        ynred[r][tx] = make_double2(yn[0], yn[1]);
         __syncthreads();
         if (on && r == 0) {
             double2 v = make_double2(0.0, 0.0);
             for (int rr = 0; rr < SR; ++rr) {
-                v.x += ynred[rr][t].x;
-                v.y += ynred[rr][t].y;
+                v.x += ynred[rr][tx].x;
+                v.y += ynred[rr][tx].y;
             }
             g.ynorm[(size_t)chunk * ncols + 2 * q] = v.x;
             g.ynorm[(size_t)chunk * ncols + 2 * q + 1] = v.y;
@@ -1080,11 +965,6 @@ __global__ void __launch_bounds__(256) k_chol_inv(const double2* __restrict__ S,
 namespace {
 
 template <int P>
-size_t pair_smem(int rows, int np) {
-    return (size_t)rows * 12 * np * sizeof(CxPair<typename Prec<P>::pair>);
-}
-
-template <int P>
 bk_status gram_impl(Field A, Field B, Field B2, int NB, const SysPart& p, double* G, double* G2, double* partial,
                     int nchunk, int V, cudaStream_t st) {
     double2* part = (double2*)partial;
@@ -1094,36 +974,8 @@ bk_status gram_impl(Field A, Field B, Field B2, int NB, const SysPart& p, double
     if (maxL <= ROWS_MAXL) {
         BK_TRY(rows_gram(P, A, B, B2, NB, p, part, nchunk, V, st));
     } else {
-        BigWork w;
-        w.n = 0;
-        int maxnp = 0;
-        for (int s = 0; s < p.nsys; ++s) {
-            if (!((p.active >> s) & 1ull)) continue;
-            const int nps = (p.L[s] + 1) / 2, side = (nps + 1) / 2;
-            maxnp = std::max(maxnp, nps);
-            for (int t0 = 0; t0 < side * side; t0 += 256) {
-                if (w.n >= 256) {
-                    bk_set_error("Gram of this partition needs more than 256 thread-block rows");
-                    return BK_ERR_INVALID_ARG;
-                }
-                w.sys[w.n] = s;
-                w.t0[w.n] = t0;
-                w.n++;
-            }
-        }
-        const size_t row = 2 * pair_smem<P>(1, maxnp);
-        if (row > (size_t)200 * 1024) {
-            bk_set_error("Gram supports systems of at most 512 columns");
-            return BK_ERR_INVALID_ARG;
-        }
-        const int SRB = (int)std::max<size_t>(1, std::min<size_t>(4, (size_t)96 * 1024 / row));
-        const size_t smem = row * SRB;
-        BK_CUDA_TRY(cudaFuncSetAttribute(k_gram_big<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        for (int b = 0; b < NB; ++b) {
-            k_gram_big<P><<<dim3(w.n, nchunk), 256, smem, st>>>(A, b == 0 ? B : B2, p, w,
-                                                                part + (size_t)b * nchunk * ne, V, nchunk, SRB);
-            BK_CUDA_TRY(cudaGetLastError());
-        }
+        for (int b = 0; b < NB; ++b)
+            BK_TRY(wide_gram(P, A, b == 0 ? B : B2, p, part + (size_t)b * nchunk * ne, nchunk, V, st));
     }
     k_gram_finish<<<(NB * ne + FIN_E - 1) / FIN_E, dim3(FIN_E, FIN_ROWS), 0, st>>>(part, nchunk, NB, p, (double2*)G, (double2*)G2);
     BK_CUDA_TRY(cudaGetLastError());
@@ -1144,12 +996,11 @@ bk_status gram_dispatch(int prec, Field A, Field B, Field B2, int NB, const SysP
 
 // partial-sum rows of a Gram matrix over the active systems
 static int gram_chunks(int prec, const SysPart& p, int V) {
-    return max_active_L(p) <= ROWS_MAXL ? gram_row_chunks(prec, V, row_tiles(p)) : site_chunks(V);
+    return max_active_L(p) <= ROWS_MAXL ? gram_row_chunks(prec, V, row_tiles(p)) : wide_gram_chunks(p, V);
 }
 
 size_t gram_partial_bytes(const SysPart& p, int V) {
-    return (size_t)2 * std::max(site_chunks(V), gram_row_chunks_max(V)) * std::max(1, p.coef_off[p.nsys]) *
-           sizeof(double2);
+    return (size_t)2 * gram_row_chunks_max(V) * std::max(1, p.coef_off[p.nsys]) * sizeof(double2);
 }
 
 bk_status launch_gram(int prec, Field A, Field B, const SysPart& p, double* G, double* partial, int V,
@@ -1239,15 +1090,20 @@ bk_status launch_genop(int prec, const GenOp& g, int V, cudaStream_t st, bool* y
     const int ncols = g.p.col0[g.p.nsys];
     const int maxL = max_active_L(g.p);
     if (maxL == 0) return BK_OK;
-    // every operand in the layout's pair count (the fast kernels use one offset)
+    // every operand has the layout's pair count (one element offset serves them all)
     const int np = g.Y.np;
-    bool same_np = true;
+    bool same_np = g.hasY != 0;
     for (int u = 0; u < g.nmi; ++u) same_np &= g.Mi[u].np == np;
     for (int e = 0; e < g.ne; ++e) same_np &= g.E[e].np == np;
     if (g.hasX) same_np &= g.X.np == np && g.Xin.np == np;
-    if (maxL <= ROWS_MAXL && g.hasY && same_np && prec != BK_FP16) {
-        BK_TRY(rows_update(prec, g, V, genop_norm_rows(V), np, st));
-    } else if (maxL <= ROWS_MAXL && g.hasY && same_np) {
+    if (!same_np) {
+        bk_set_error("block update: an output and operands of one layout expected");
+        return BK_ERR_INVALID_ARG;
+    }
+    if (prec != BK_FP16) {
+        BK_TRY(maxL <= ROWS_MAXL ? rows_update(prec, with_units(g), V, nchunk, np, st)
+                                 : wide_update(prec, with_units(g), V, nchunk, st));
+    } else if (maxL <= ROWS_MAXL) {
         const PTiles wt = make_ptiles(g.p, WT_PAIRS);
         const dim3 grid(wt.n, nchunk);
         if (maxL <= 6) k_genop_w<6><<<grid, GW_WARPS * 32, 0, st>>>(g, wt, V, nchunk, ncols, np);
@@ -1255,13 +1111,10 @@ bk_status launch_genop(int prec, const GenOp& g, int V, cudaStream_t st, bool* y
     } else {
         const PTiles tl = make_ptiles(g.p, TILE_MAXP);
         constexpr int SR = 4;
-        const dim3 grid(tl.n, nchunk), block(TILE_MAXP, SR);
-        switch (prec) {
-            case BK_FP64: k_genop<BK_FP64, SR><<<grid, block, 0, st>>>(g, tl, V, nchunk, ncols); break;
-            case BK_FP32: k_genop<BK_FP32, SR><<<grid, block, 0, st>>>(g, tl, V, nchunk, ncols); break;
-            case BK_FP16: k_genop<BK_FP16, SR><<<grid, block, 0, st>>>(g, tl, V, nchunk, ncols); break;
-            default: return BK_ERR_INVALID_ARG;
-        }
+        int widest = 1;
+        for (int i = 0; i < tl.n; ++i) widest = std::max(widest, tl.np[i]);
+        k_genop<BK_FP16, SR><<<dim3(tl.n, nchunk, (widest + TILE_MAXP - 1) / TILE_MAXP), dim3(TILE_MAXP, SR), 0, st>>>(
+            g, tl, V, nchunk, ncols);
     }
     BK_CUDA_TRY(cudaGetLastError());
     if (ynorm_done && g.ynorm && g.hasY) *ynorm_done = true;

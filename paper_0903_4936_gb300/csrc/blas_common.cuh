@@ -181,3 +181,19 @@ bk_status rows_gram(int prec, Field A, Field B, Field B2, int NB, const SysPart&
                     int V, cudaStream_t st);
 PTiles row_tiles(const SysPart& p);
 bk_status rows_update(int prec, const GenOp& g, int V, int nchunk, int np, cudaStream_t st);
+// GenOp's unit flags and whether it uses M
+inline GenOp with_units(GenOp g) {
+    auto unit = [](double x) { return x == 1.0 ? 1 : (x == -1.0 ? -1 : 0); };
+    for (int e = 0; e < GENOP_MAXE; ++e) g.ea_unit[e] = unit(g.ea_mult[e]);
+    for (int u = 0; u < GENOP_MAXMI; ++u) g.ma_unit[u] = unit(g.ma_mult[u]);
+    g.xa_unit = unit(g.xa_mult);
+    g.y_unit = unit(g.ym);
+    g.x_unit = unit(g.xm);
+    g.mat = g.nmi > 0 && g.M != nullptr && ((g.hasY && g.ym != 0.0) || (g.hasX && g.xm != 0.0));
+    return g;
+}
+// wide.cu: systems of any size
+int wide_gram_chunks(const SysPart& p, int V);
+bk_status wide_gram(int prec, Field A, Field B, const SysPart& p, double2* partial, int nchunk, int V,
+                    cudaStream_t st);
+bk_status wide_update(int prec, const GenOp& g, int V, int nchunk, cudaStream_t st);

@@ -451,16 +451,7 @@ bk_status rows_gram(int prec, Field A, Field B, Field B2, int NB, const SysPart&
     return BK_ERR_INVALID_ARG;
 }
 
-bk_status rows_update(int prec, const GenOp& g0, int V, int nchunk, int np, cudaStream_t st) {
-    // what the kernel would otherwise find out with FP64 comparisons
-    GenOp g = g0;
-    auto unit = [](double x) { return x == 1.0 ? 1 : (x == -1.0 ? -1 : 0); };
-    for (int e = 0; e < GENOP_MAXE; ++e) g.ea_unit[e] = unit(g.ea_mult[e]);
-    for (int u = 0; u < GENOP_MAXMI; ++u) g.ma_unit[u] = unit(g.ma_mult[u]);
-    g.xa_unit = unit(g.xa_mult);
-    g.y_unit = unit(g.ym);
-    g.x_unit = unit(g.xm);
-    g.mat = g.nmi > 0 && g.M != nullptr && ((g.hasY && g.ym != 0.0) || (g.hasX && g.xm != 0.0));
+bk_status rows_update(int prec, const GenOp& g, int V, int nchunk, int np, cudaStream_t st) {
     const PTiles wt = row_tiles(g.p);
     const dim3 grid(wt.n, nchunk);
     const int ncols = g.p.col0[g.p.nsys];

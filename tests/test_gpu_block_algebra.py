@@ -1,0 +1,78 @@
+"""Block algebra and L x L steps (C ABI) at the sizes where their kernels
+change: the row kernels up to 12 columns, the tiled ones above, odd column
+counts, lattices that fill no tile, and the FP64 operator on either side of
+its split over four warps."""
+import numpy as np
+import pytest
+
+import synth
+from oracle import dense, dirac
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+# sums of n products of unit-size terms: sqrt(n) roundings of the arithmetic, with a factor of ten to spare
+GRAM_TOL = {"fp64": 1e-13, "fp32": 1e-5, "fp16": 2e-3}
+XMY_TOL = {"fp64": 2e-14, "fp32": 2e-6, "fp16": 2e-3}
+
+
+def _rel(a, b):
+    return float(np.max(np.abs(a - b)) / np.max(np.abs(b)))
+
+
+def _lat(dims, seed=1):
+    import paper_0903_4936_gb300 as bk
+    lat = bk.Lattice(dims)
+    U = synth.random_su3_field(dims, 0.4, seed)
+    lat.upload_gauge(U)
+    lat.build_clover(1.0)
+    return lat, U
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "fp16"])
+@pytest.mark.parametrize("dims,L", [((3, 5, 4, 6), 1), ((3, 5, 4, 6), 5), ((2, 2, 2, 2), 6), ((3, 5, 4, 6), 7),
+                                    ((3, 5, 4, 6), 12), ((3, 5, 4, 6), 13), ((2, 2, 2, 2), 27), ((4, 4, 4, 6), 48),
+                                    ((3, 5, 4, 6), 63), ((3, 5, 2, 6), 97), ((2, 3, 4, 6), 130), ((2, 3, 4, 6), 259)])
+def test_gram_and_xmy(prec, dims, L):
+    """G = A^H B and Y = Z + c X M against numpy in FP64."""
+    lat, _ = _lat(dims)
+    A = synth.gaussian_sources(dims, L, 21)
+    B = synth.gaussian_sources(dims, L, 22)
+    Fa, Fb = lat.pack(torch.from_numpy(A).cuda(), prec), lat.pack(torch.from_numpy(B).cuda(), prec)
+    G = lat.gram(Fa, Fb, L, prec).cpu().numpy()
+    a, b = A.reshape(L, -1), B.reshape(L, -1)
+    assert _rel(G, a.conj() @ b.T) < GRAM_TOL[prec]
+    rng = np.random.default_rng(5)
+    M = (rng.standard_normal((L, L)) + 1j * rng.standard_normal((L, L))) / np.sqrt(2 * L)
+    for c, Z in ((1.0, None), (0.3 - 0.7j, Fb)):
+        Y = lat.unpack(lat.xmy(Fa, torch.from_numpy(M).cuda(), L, c=c, Z=Z, prec=prec), L, prec).cpu().numpy()
+        ref = c * (M.T @ a) + (b if Z is not None else 0.0)
+        assert _rel(Y.reshape(L, -1), ref) < XMY_TOL[prec]
+
+
+@pytest.mark.parametrize("method", ["bicggr", "bicgstab"])
+@pytest.mark.parametrize("Ls", [(1,), (2, 5), (7,), (11, 3), (12, 6), (13,)])
+def test_fp64_solves_by_system_size(method, Ls):
+    """FP64 solves whose systems are on either side of 6 and 12 columns against dense LU."""
+    dims = (4, 4, 4, 4)
+    lat, U = _lat(dims, 7)
+    B = synth.z4_noise(dims, sum(Ls), 31)
+    X, infos = lat.block_solve_batched(torch.from_numpy(B).cuda(), [0.12] * len(Ls), list(Ls), method=method,
+                                       prec="fp64", tol=1e-11, maxiter=500)
+    D = dense.dense_matrix(U, 0.12, 1.0)
+    ref = np.linalg.solve(D, dense.to_columns(B))
+    got = dense.to_columns(X.cpu().numpy())
+    assert all(i["converged"] == 1 for i in infos)
+    # ||x - x*|| <= ||D^-1|| ||r||, ||D^-1|| < 20 at this kappa
+    assert np.max(np.linalg.norm(got - ref, axis=0) / np.linalg.norm(B.reshape(sum(Ls), -1).T, axis=0)) < 2e-10
+
+
+@pytest.mark.parametrize("dims,L", [((2, 2, 2, 2), 1), ((3, 5, 4, 6), 3), ((8, 8, 8, 8), 9), ((8, 8, 8, 8), 10)])
+def test_fp64_operator_split_over_warps(dims, L):
+    """Site-columns below (38912 of them) and above the limit of the four-warp form, with a residual solve's path."""
+    lat, U = _lat(dims, 9)
+    X = synth.gaussian_sources(dims, L, 3)
+    kap = np.linspace(0.11, 0.13, L)
+    Y = lat.dslash(torch.from_numpy(X).cuda(), list(kap), "fp64").cpu().numpy()
+    assert _rel(Y, dirac.apply_dirac(U, X, kap, 1.0)) < 1e-13
