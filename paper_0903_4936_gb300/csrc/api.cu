@@ -110,16 +110,7 @@ struct bk_ctx {
     DevBuf B64, X64, R64, Xlo, blk[8], small, spart, stage, colmap, fscratch, ynorm;
     HostBuf rb_host;
     std::vector<cudaEvent_t> events;
-    // operator launch shapes chosen by the autotuner, keyed by (prec, residual, ncol)
-    struct Shape {
-        int threads, variant, group, prefetch;
-    };
-    std::map<long long, Shape> shapes;
-    bool autotune = true;
-    bool verbose = false;  // BK_VERBOSE=1: one line per solve and per tuning decision on stderr
-    int force_variant = 0;  // BK_DSLASH_VARIANT=1..5: FP32/FP16 operator variant (4, 5: FP32 staged form),
-                            // 128 threads, pair groups of 8, no tuning (tests the variants the tuner may pick)
-    int force_prefetch = 0; // BK_DSLASH_PREFETCH=0..3: its prefetch mode (with BK_DSLASH_VARIANT)
+    bool verbose = false;  // BK_VERBOSE=1: one line per solve on stderr
     // even-odd form: A^-1 = (1 - kappa C)^-1 per kappa (FP64 and FP32 tables), built
     // on first use and dropped when the gauge field or the clover term changes
     struct CInv {
@@ -175,21 +166,15 @@ extern "C" bk_status bk_create(const int dims[4], int device, bk_ctx** out) {
     for (int mu = 0; mu < 4; ++mu) c->dims[mu] = dims[mu];
     c->V = (int)V;
     {
-        const char* e = getenv("BK_AUTOTUNE");
-        c->autotune = !(e && e[0] == '0');
         const char* v = getenv("BK_VERBOSE");
         c->verbose = v && v[0] == '1';
-        const char* fv = getenv("BK_DSLASH_VARIANT");
-        if (fv && fv[0] >= '1' && fv[0] <= '5') c->force_variant = fv[0] - '0';
-        const char* fp = getenv("BK_DSLASH_PREFETCH");
-        if (fp && fp[0] >= '0' && fp[0] <= '3') c->force_prefetch = fp[0] - '0';
     }
     c->device = device;
     bk_status s;
     if ((s = c->U64.ensure((size_t)36 * V * sizeof(double2))) != BK_OK ||
-        (s = c->U32.ensure((size_t)4 * V * BK_LINK32_F4 * sizeof(float4))) != BK_OK ||
+        (s = c->U32.ensure((size_t)4 * V * BK_LINKC * sizeof(float))) != BK_OK ||
         (s = c->C64.ensure((size_t)36 * V * sizeof(double2))) != BK_OK ||
-        (s = c->C32.ensure((size_t)V * BK_CLOV32_F4 * sizeof(float4))) != BK_OK) {
+        (s = c->C32.ensure((size_t)V * BK_CLOVC * sizeof(float))) != BK_OK) {
         bk_destroy(c);
         return s;
     }
@@ -227,7 +212,7 @@ extern "C" bk_status bk_upload_gauge(bk_ctx* c, const double* U, int on_device, 
         BK_CUDA_TRY(cudaMemcpyAsync(c->Utmp.p, U, (size_t)36 * c->V * sizeof(double2), cudaMemcpyHostToDevice, st));
         src = c->Utmp.as<double>();
     }
-    BK_TRY(launch_gauge_convert(src, c->U64.as<double2>(), c->U32.as<float4>(), c->V, st));
+    BK_TRY(launch_gauge_convert(src, c->U64.as<double2>(), c->U32.as<float>(), c->V, st));
     if (!on_device) BK_CUDA_TRY(cudaStreamSynchronize(st));
     c->has_gauge = true;
     c->has_clover = false;
@@ -242,7 +227,7 @@ extern "C" bk_status bk_build_clover(bk_ctx* c, double csw, void* stream) {
         return BK_ERR_NO_GAUGE;
     }
     BK_CUDA_TRY(cudaSetDevice(c->device));
-    BK_TRY(launch_clover_build(c->U64.as<double2>(), c->C64.as<double2>(), c->C32.as<float4>(), c->dims, csw,
+    BK_TRY(launch_clover_build(c->U64.as<double2>(), c->C64.as<double2>(), c->C32.as<float>(), c->dims, csw,
                                (cudaStream_t)stream));
     c->csw = csw;
     c->has_clover = true;
@@ -274,67 +259,6 @@ extern "C" bk_status bk_unpack(bk_ctx* c, const void* Xd, double* X, int L, bk_p
     return launch_unpack(prec, make_field((void*)Xd, L, c->V, prec), nullptr, 0, X, L, (cudaStream_t)stream);
 }
 
-// Pick the operator's launch shape (threads per block and, for FP32 / FP16,
-// the register cap) for this context: on first use of a (precision, mode,
-// column count) every candidate runs on the caller's data and the fastest
-// (CUDA events, 2 timed launches after 1 warm-up) is kept.  Every candidate
-// computes the same result.
-static bk_status tune_shape(bk_ctx* c, int prec, DslashOp op, cudaStream_t st, bk_ctx::Shape& best) {
-    std::vector<bk_ctx::Shape> cands;
-    {
-        // register caps 255 (variant 1), 170 (2), 128 (3); pair groups of 16
-        // pairs or all pairs at once; no prefetch, prefetch into L2 or L1, or
-        // the looped form with L1 prefetch one hop ahead
-        const int npl = (op.ncol + 1) / 2;
-        for (int pf : {0, 1, 2, 3})
-            for (int grp : {16, 0}) {
-                if (grp > 0 && grp >= npl) continue;
-                cands.push_back({128, 1, grp, pf});
-                cands.push_back({128, 2, grp, pf});
-                cands.push_back({128, 3, grp, pf});
-            }
-        // FP32: the staged form (rows through a shared-memory ring of 2 or 3 slots)
-        if (prec == BK_FP32)
-            for (int grp : {16, 0}) {
-                if (grp > 0 && grp >= npl) continue;
-                cands.push_back({128, 4, grp, 0});
-                cands.push_back({128, 5, grp, 0});
-            }
-    }
-    // events released on every return path
-    struct EventPair {
-        cudaEvent_t a = nullptr, b = nullptr;
-        ~EventPair() {
-            if (a) cudaEventDestroy(a);
-            if (b) cudaEventDestroy(b);
-        }
-    } ev;
-    BK_CUDA_TRY(cudaEventCreate(&ev.a));
-    BK_CUDA_TRY(cudaEventCreate(&ev.b));
-    cudaEvent_t e0 = ev.a, e1 = ev.b;
-    float best_ms = 1e30f;
-    best = cands[0];
-    for (const auto& cd : cands) {
-        op.threads = cd.threads;
-        op.variant = cd.variant;
-        op.group = cd.group;
-        op.prefetch = cd.prefetch;
-        BK_TRY(launch_dslash(prec, op, st));
-        BK_CUDA_TRY(cudaEventRecord(e0, st));
-        BK_TRY(launch_dslash(prec, op, st));
-        BK_TRY(launch_dslash(prec, op, st));
-        BK_CUDA_TRY(cudaEventRecord(e1, st));
-        BK_CUDA_TRY(cudaEventSynchronize(e1));
-        float ms = 0.f;
-        BK_CUDA_TRY(cudaEventElapsedTime(&ms, e0, e1));
-        if (ms < best_ms) {
-            best_ms = ms;
-            best = cd;
-        }
-    }
-    return BK_OK;
-}
-
 static bk_status dslash_fields(bk_ctx* c, int prec, const double* kappa, Field x, Field y, Field b, int col0,
                                int ncol, int residual, cudaStream_t st) {
     DslashOp op;
@@ -349,33 +273,6 @@ static bk_status dslash_fields(bk_ctx* c, int prec, const double* kappa, Field x
     op.ncol = ncol;
     op.residual = residual;
     op.kappa = kappa;
-    op.threads = 0;
-    op.variant = 0;
-    op.group = 0;
-    op.prefetch = 0;
-    if (c->force_variant && !wide(prec)) {
-        op.threads = 128;
-        op.variant = c->force_variant;
-        op.group = 8;
-        op.prefetch = c->force_prefetch;
-    } else if (c->autotune && ncol <= BK_MAX_COLS && !wide(prec)) {
-        const long long key = ((long long)prec << 40) | ((long long)(residual != 0) << 36) | ncol;
-        auto it = c->shapes.find(key);
-        if (it == c->shapes.end()) {
-            bk_ctx::Shape sh;
-            BK_TRY(tune_shape(c, prec, op, st, sh));
-            it = c->shapes.emplace(key, sh).first;
-            if (c->verbose)
-                fprintf(stderr,
-                        "[bkrylov] tuned operator prec=%d residual=%d ncol=%d: threads=%d variant=%d group=%d "
-                        "prefetch=%d\n",
-                        prec, residual, ncol, sh.threads, sh.variant, sh.group, sh.prefetch);
-        }
-        op.threads = it->second.threads;
-        op.variant = it->second.variant;
-        op.group = it->second.group;
-        op.prefetch = it->second.prefetch;
-    }
     return launch_dslash(prec, op, st);
 }
 
@@ -390,10 +287,10 @@ static bk_status clover_inverse(bk_ctx* c, double kappa, cudaStream_t st, const 
     if (it == c->cinv.end()) {
         std::unique_ptr<bk_ctx::CInv> ci(new bk_ctx::CInv());
         BK_TRY(ci->c64.ensure((size_t)36 * c->V * sizeof(double2)));
-        BK_TRY(ci->c32.ensure((size_t)c->V * BK_CLOV32_F4 * sizeof(float4)));
+        BK_TRY(ci->c32.ensure((size_t)c->V * BK_CLOVC * sizeof(float)));
         BK_TRY(c->cinv_bound.ensure(2 * sizeof(unsigned long long)));
         BK_CUDA_TRY(cudaMemsetAsync(c->cinv_bound.p, 0, 2 * sizeof(unsigned long long), st));
-        BK_TRY(launch_clover_inverse(c->C64.as<double2>(), kappa, ci->c64.as<double2>(), ci->c32.as<float4>(), c->V,
+        BK_TRY(launch_clover_inverse(c->C64.as<double2>(), kappa, ci->c64.as<double2>(), ci->c32.as<float>(), c->V,
                                      c->cinv_bound.as<unsigned long long>(), st));
         unsigned long long hb[2];
         BK_CUDA_TRY(cudaMemcpyAsync(hb, c->cinv_bound.p, sizeof(hb), cudaMemcpyDeviceToHost, st));
@@ -409,55 +306,6 @@ static bk_status clover_inverse(bk_ctx* c, double kappa, cudaStream_t st, const 
         it = c->cinv.emplace(key, std::move(ci)).first;
     }
     *out = it->second.get();
-    return BK_OK;
-}
-
-// FP32 / FP16 even-odd launch shape, tuned once per (precision, column count)
-// on the caller's data (mode 1, the half of the Schur operator that writes
-// only the temporary): 256 or 128 threads, or (FP32) the staged form with 2
-// or 3 ring slots; pair groups of 16 or all pairs.
-static bk_status eo_shape(bk_ctx* c, int prec, EoOp op, cudaStream_t st) {
-    const long long key = (1LL << 44) | ((long long)prec << 40) | op.ncol;
-    auto it = c->shapes.find(key);
-    if (it == c->shapes.end()) {
-        bk_ctx::Shape best{0, 2, 0, 0};
-        if (c->autotune) {
-            cudaEvent_t e0, e1;
-            BK_CUDA_TRY(cudaEventCreate(&e0));
-            BK_CUDA_TRY(cudaEventCreate(&e1));
-            float best_ms = 1e30f;
-            const int npl = (op.ncol + 1) / 2;
-            for (int v : {1, 2, 4, 5})
-                for (int grp : {16, 0}) {
-                    if (grp > 0 && grp >= npl) continue;
-                    if (v >= 4 && prec != BK_FP32) continue;  // staged forms: FP32 only
-                    op.variant = v;
-                    op.group = grp;
-                    bk_status r = launch_eo(prec, op, st);
-                    if (r == BK_OK) r = (cudaEventRecord(e0, st) == cudaSuccess) ? BK_OK : BK_ERR_CUDA;
-                    if (r == BK_OK) r = launch_eo(prec, op, st);
-                    if (r == BK_OK) r = launch_eo(prec, op, st);
-                    if (r == BK_OK) r = (cudaEventRecord(e1, st) == cudaSuccess) ? BK_OK : BK_ERR_CUDA;
-                    float ms = 0.f;
-                    if (r == BK_OK && cudaEventSynchronize(e1) == cudaSuccess &&
-                        cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess && ms < best_ms) {
-                        best_ms = ms;
-                        best = {0, v, grp, 0};
-                    }
-                    if (r != BK_OK) {
-                        cudaEventDestroy(e0);
-                        cudaEventDestroy(e1);
-                        return r;
-                    }
-                }
-            cudaEventDestroy(e0);
-            cudaEventDestroy(e1);
-            if (c->verbose)
-                fprintf(stderr, "[bkrylov] tuned even-odd operator prec=%d ncol=%d: variant=%d group=%d\n", prec,
-                        op.ncol, best.variant, best.group);
-        }
-        it = c->shapes.emplace(key, best).first;
-    }
     return BK_OK;
 }
 
@@ -483,16 +331,6 @@ static bk_status schur_fields(bk_ctx* c, int prec, const double* kappa, const vo
     op.b = t;
     op.par = 1;
     op.mode = 1;
-    op.variant = 2;
-    if (!wide(prec) && c->force_variant) {  // BK_DSLASH_VARIANT: 1, 2 (3 -> 2), 4, 5 (FP32); groups of 8
-        op.variant = c->force_variant == 3 ? 2 : c->force_variant;
-        op.group = 8;
-    } else if (!wide(prec)) {
-        BK_TRY(eo_shape(c, prec, op, st));
-        const long long key = (1LL << 44) | ((long long)prec << 40) | ncol;
-        op.variant = c->shapes[key].variant;
-        op.group = c->shapes[key].group;
-    }
     BK_TRY(launch_eo(prec, op, st));
     // y_e = x_e - kappa^2 A_ee^-1 H_eo t_o   (or b_e minus that)
     op.x = t;

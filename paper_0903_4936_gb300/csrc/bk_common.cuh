@@ -367,8 +367,9 @@ void bk_set_error(const char* fmt, ...);
 
 // Maximum columns handled by one operator launch (kernel-argument kappa list).
 #define BK_MAX_COLS 256
-// FP32 packed-pair gauge link: float4 units per (mu, site); clover: per site.
-#define BK_LINK32_F4 14
-#define BK_CLOV32_F4 51
-// Maximum number of systems of a batched solve (one bit each in a 64-bit mask).
 #define BK_MAX_SYS 64
+// FP32 tables, in floats: a link (row-major {re, im}, padded to 80 bytes; the
+// four of a site together) and a site term (per chiral block 6 diagonal
+// entries, then 15 complex ones below it)
+#define BK_LINKC 20
+#define BK_CLOVC 72

@@ -7,33 +7,26 @@
 #include "bk_common.cuh"
 
 // ---------------------------------------------------------------- gauge.cu
-bk_status launch_gauge_convert(const double* Uin_dev, double2* U64, float4* U32, int V, cudaStream_t st);
-bk_status launch_clover_build(const double2* U64, double2* C64, float4* C32, const int dims[4], double csw,
+bk_status launch_gauge_convert(const double* Uin_dev, double2* U64, float* U32, int V, cudaStream_t st);
+bk_status launch_clover_build(const double2* U64, double2* C64, float* C32, const int dims[4], double csw,
                               cudaStream_t st);
 // Even-odd form: A(n)^-1 = (1 - kappa C(n))^-1 for one kappa, stored like the
-// clover (FP64 [36][V], FP32 packed pairs); bound[0] = the largest infinity
+// clover (FP64 [36][V], FP32 compact); bound[0] = the largest infinity
 // norm of A's chiral blocks (as double bits), bound[1] += singular blocks.
-bk_status launch_clover_inverse(const double2* C64, double kappa, double2* Ci64, float4* Ci32, int V,
+bk_status launch_clover_inverse(const double2* C64, double kappa, double2* Ci64, float* Ci32, int V,
                                 unsigned long long* bound, cudaStream_t st);
 
 // ---------------------------------------------------------------- dslash.cu
 struct DslashOp {
     Field x, y, b;         // y = D x, or y = b - D x when residual != 0
-    const void* U;         // FP64: [4][9][V] double2; FP32/FP16: packed-pair links (gauge.cu)
-    const void* clov;      // FP64: [36][V] double2; FP32/FP16: packed-pair clover (gauge.cu)
+    const void* U;         // FP64: [4][9][V] double2; FP32/FP16: compact links (bk_common.cuh)
+    const void* clov;      // FP64: [36][V] double2; FP32/FP16: compact clover
     int dims[4];
     int V;
     int col0, ncol;        // columns [col0, col0 + ncol) of x, y, b (FP32/FP16: col0 even,
                            // the launch covers whole pairs)
     int residual;
     const double* kappa;   // host array, ncol entries (kappa of column col0 + j)
-    int threads;           // launch shape: threads per block (0 = default)
-    int variant;           // FP32/FP16: register cap, 1 = 255, 2 = 170, 3 = 128 (0 = 2)
-    int group;             // FP32/FP16: column pairs per group, groups run one after the
-                           // other over all sites (0 = all pairs in one group)
-    int prefetch;          // FP32/FP16: prefetch every row of the eight hops at thread
-                           // start, 0 = no, 1 = into L2, 2 = into L1; 3 = the hops as
-                           // a loop, each prefetching the next hop's rows into L1
 };
 bk_status launch_dslash(int prec, const DslashOp& op, cudaStream_t st);
 
@@ -51,8 +44,6 @@ struct EoOp {
     int col0, ncol;
     int par, mode, hop, residual;
     const double* kappa;  // kappa of column col0 + j
-    int variant, group;   // FP32 / FP16: 1 = 256 threads (255 registers), 2 = 128 (170); FP32 4 / 5 =
-                          // staged, 2 / 3 ring slots; pair groups of `group` pairs (0: all)
 };
 bk_status launch_eo(int prec, const EoOp& op, cudaStream_t st);
 // FP64 full-lattice block <-> its even and odd half-lattice blocks (same columns)

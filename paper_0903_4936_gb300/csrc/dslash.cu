@@ -7,13 +7,23 @@
 // FP32 / FP16 storage (k_dslash_pair): one thread per site and column pair.
 // Blocks are RHS-interleaved (all columns of a site in one row), so the
 // lanes of a warp read one contiguous line per spinor component and share
-// every gauge link and clover entry of their site (one transaction for the
-// warp).  All arithmetic is on pairs {column 2p, column 2p + 1} with the
-// packed FP32x2 multiply-add of sm_100+, against links and clover entries
-// stored as duplicated pairs {u_r, u_r}, {u_i, u_i}, {-u_i, -u_i}, so that
-// a complex product costs four packed instructions for two columns.  The
-// clover term is applied first (out = x - kappa C x needs x(n) only once);
-// each of the eight hops then adds -kappa times its term directly.
+// every gauge link and clover entry of their site.  All arithmetic is on pairs
+// {column 2p, column 2p + 1} with the packed FP32x2 multiply-add of sm_100+;
+// a link or clover entry is loaded as {re, im} (8 bytes for the whole warp)
+// and its operands {u_r, u_r}, {u_i, u_i}, {-u_i, -u_i} are formed by moves,
+// for which the issue slots are free.  The clover term is applied first (out =
+// x - kappa C x needs x(n) only once); each of the eight hops then adds -kappa
+// times its term directly.
+//
+// What bounds it: the rows' eight-fold fetches from L2, 10 TB/s of L2-to-SM
+// traffic (16^3x32, 30 columns: 3.0 GB in 284 us).  Before, links and clover
+// were stored as the duplicated pairs (224 and 816 bytes) and took 216 loads a
+// thread, which with staging copies through shared memory kept the load/store
+// pipe 74 % busy: 404 us there (24^3x48, 96 columns 5080 us, now 4240; FP16
+// 12x10x14x18, 13 columns 51, now 34).  A form with the rows staged by bulk
+// copies (cp.async.bulk, a producer warp, 2x2x2 site tiles sharing their rows,
+// 5 fetches a site instead of 8) took 306 us: its producer and 128-register
+// workers, not L2, were the limit.
 //
 // FP64 / double-float (k_dslash_col): one thread per site and column, FP64
 // links and clover in [element][site] order (the FP64 pipe, not memory,
@@ -38,11 +48,10 @@ namespace {
 
 struct DPairArgs {
     Field x, y, b;
-    const float4* __restrict__ U;  // packed-pair links, BK_LINK32_F4 float4 per (mu, site)
-    const float4* __restrict__ C;  // packed-pair clover, BK_CLOV32_F4 float4 per site
+    const float* __restrict__ U;  // compact links, [site][mu] of BK_LINKC floats
+    const float* __restrict__ C;  // compact clover, BK_CLOVC floats per site
     int L[4], st[4];
     int V, p0, npl, residual;
-    int G;  // pairs per group: all sites of group g run before group g + 1 starts
     float2 nk[BK_MAX_COLS / 2];  // {-kappa_2p, -kappa_2p+1} of launch pair p - p0
 };
 
@@ -174,59 +183,129 @@ __device__ __forceinline__ void reconstruct_colour(int a, float2 w0r, float2 w0i
     }
 }
 
-template <int MU, int S>
-__device__ __forceinline__ void reconstruct_pair(const Hop& w, float2 nk, float2 pk, float2 (&ar)[12],
-                                                 float2 (&ai)[12]) {
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-        reconstruct_colour<MU, S>(a, w.r[a], w.i[a], w.r[3 + a], w.i[3 + a], nk, pk, ar, ai);
-}
+// Compact complex table entries (gauge.cu), in global or in shared memory.  All
+// lanes of a site read the same 8 bytes, and the pairs {u, u} of the packed
+// arithmetic are formed by moves: a 64-bit shared read takes two passes of the
+// load pipe and a 128-bit one four, whatever it broadcasts, so 72 bytes a link
+// cost a third of links stored as pairs (216 bytes).
+struct GTab {
+    const float2* p;
+    __device__ __forceinline__ float2 at(int e) const { return __ldg(p + e); }
+};
+struct STab {
+    unsigned a;
+    __device__ __forceinline__ float2 at(int e) const {
+        float2 v;
+        asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a + 8 * e));
+        return v;
+    }
+};
+__device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
 
-// w = U h (forward) or U^+ h (backward) for both half-spinor vectors.  Link
-// element e = 3 row + col: {u_r, u_r, u_i, u_i} at float4 e, {-u_i, -u_i} at
-// float2 18 + e.  One output row at a time: three link elements are live.
-template <bool DAG>
-__device__ __forceinline__ void link_mul(const float4* __restrict__ u4, const Hop& h, Hop& w) {
-    const float2* u2 = reinterpret_cast<const float2*>(u4);
+// Product with the link U (forward) or U^+ (backward) and reconstruction, fused
+// row by row: output colour i of both half-spinor vectors is formed and added
+// at once, so only one row of the link and one colour of w are live.
+template <int MU, int S, typename T>
+__device__ __forceinline__ void link_mul_add(T u, const Hop& h, float2 nk, float2 pk, float2 (&ar)[12],
+                                             float2 (&ai)[12]) {
+    constexpr bool DAG = S > 0;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        float2 ur[3], ui[3], un[3];
+        float2 e[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) e[j] = u.at(DAG ? 3 * j + i : 3 * i + j);
+        float2 wr[2], wi[2];
+#pragma unroll
+        for (int hh = 0; hh < 2; ++hh) wr[hh] = wi[hh] = make_float2(0.f, 0.f);
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-            const int e = DAG ? 3 * j + i : 3 * i + j;
-            const float4 q = __ldg(u4 + e);
-            ur[j] = make_float2(q.x, q.y);
-            ui[j] = make_float2(q.z, q.w);
-            un[j] = __ldg(u2 + 18 + e);
-        }
+            const float2 ur = dup(e[j].x), ui = dup(e[j].y), un = dup(-e[j].y);
 #pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-            float2 wr = make_float2(0.f, 0.f), wi = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int j = 0; j < 3; ++j) {
+            for (int hh = 0; hh < 2; ++hh) {
                 const float2 hr = h.r[3 * hh + j], hi = h.i[3 * hh + j];
-                if constexpr (!DAG) {  // U_ij h_j: (u_r h_r - u_i h_i, u_r h_i + u_i h_r)
-                    wr = pfma(ur[j], hr, wr);
-                    wr = pfma(un[j], hi, wr);
-                    wi = pfma(ur[j], hi, wi);
-                    wi = pfma(ui[j], hr, wi);
-                } else {  // conj(U_ji) h_j: (u_r h_r + u_i h_i, u_r h_i - u_i h_r)
-                    wr = pfma(ur[j], hr, wr);
-                    wr = pfma(ui[j], hi, wr);
-                    wi = pfma(ur[j], hi, wi);
-                    wi = pfma(un[j], hr, wi);
-                }
+                wr[hh] = pfma(ur, hr, wr[hh]);
+                wr[hh] = pfma(DAG ? ui : un, hi, wr[hh]);
+                wi[hh] = pfma(ur, hi, wi[hh]);
+                wi[hh] = pfma(DAG ? un : ui, hr, wi[hh]);
             }
-            w.r[3 * hh + i] = wr;
-            w.i[3 * hh + i] = wi;
+        }
+        reconstruct_colour<MU, S>(i, wr[0], wi[0], wr[1], wi[1], nk, pk, ar, ai);
+    }
+}
+
+// y = H_b v for chiral block b (6 diagonal entries, then 15 complex ones below
+// the diagonal) of a compact site term
+template <typename T>
+__device__ __forceinline__ void herm6_pair(T c, int b, const float2 (&vr)[6], const float2 (&vi)[6], float2 (&yr)[6],
+                                           float2 (&yi)[6]) {
+#pragma unroll
+    for (int i = 0; i < 6; i += 2) {
+        const float2 d = c.at(18 * b + i / 2);
+        yr[i] = pmul(dup(d.x), vr[i]);
+        yi[i] = pmul(dup(d.x), vi[i]);
+        yr[i + 1] = pmul(dup(d.y), vr[i + 1]);
+        yi[i + 1] = pmul(dup(d.y), vi[i + 1]);
+    }
+    int q = 0;
+#pragma unroll
+    for (int i = 1; i < 6; ++i)
+#pragma unroll
+        for (int j = 0; j < i; ++j, ++q) {
+            const float2 A = c.at(18 * b + 3 + q);
+            const float2 AR = dup(A.x), AI = dup(A.y), NAI = dup(-A.y);
+            // y_i += A v_j, y_j += conj(A) v_i
+            yr[i] = pfma(AR, vr[j], yr[i]);
+            yr[i] = pfma(NAI, vi[j], yr[i]);
+            yi[i] = pfma(AR, vi[j], yi[i]);
+            yi[i] = pfma(AI, vr[j], yi[i]);
+            yr[j] = pfma(AR, vr[i], yr[j]);
+            yr[j] = pfma(AI, vi[i], yr[j]);
+            yi[j] = pfma(AR, vi[i], yi[j]);
+            yi[j] = pfma(NAI, vr[i], yi[j]);
+        }
+}
+
+// The site term on (ar, ai) in place: CLOVER: out = q - kappa C q (nk =
+// {-kappa}); else out = A^-1 q.  The blocks act on u + l and u - l.
+template <bool CLOVER, typename T>
+__device__ __forceinline__ void site_term(T c, float2 nk, float2 (&ar)[12], float2 (&ai)[12]) {
+    float2 vr[2][6], vi[2][6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        vr[0][k] = padd(ar[k], ar[k + 6]);
+        vi[0][k] = padd(ai[k], ai[k + 6]);
+        vr[1][k] = psub(ar[k], ar[k + 6]);
+        vi[1][k] = psub(ai[k], ai[k + 6]);
+    }
+    const float2 pk = make_float2(-nk.x, -nk.y);
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+        float2 yr[6], yi[6];
+        herm6_pair(c, b, vr[b], vi[b], yr, yi);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            if (CLOVER) {  // upper half: -kappa y; lower: -kappa y (b = 0), +kappa y (b = 1)
+                ar[k] = pfma(nk, yr[k], ar[k]);
+                ai[k] = pfma(nk, yi[k], ai[k]);
+                ar[k + 6] = pfma(b == 0 ? nk : pk, yr[k], ar[k + 6]);
+                ai[k + 6] = pfma(b == 0 ? nk : pk, yi[k], ai[k + 6]);
+            } else if (b == 0) {  // u = y0 + y1, l = y0 - y1
+                ar[k] = ar[k + 6] = yr[k];
+                ai[k] = ai[k + 6] = yi[k];
+            } else {
+                ar[k] = padd(ar[k], yr[k]);
+                ai[k] = padd(ai[k], yi[k]);
+                ar[k + 6] = psub(ar[k + 6], yr[k]);
+                ai[k + 6] = psub(ai[k + 6], yi[k]);
+            }
         }
     }
 }
 
 template <int P, int MU, int S>
-__device__ __forceinline__ void hop_pair(const Field& x, int nb, int p, const float4* __restrict__ link,
+__device__ __forceinline__ void hop_pair(const Field& x, int nb, int p, const float* __restrict__ link,
                                          float2 nk, float2 pk, float2 (&ar)[12], float2 (&ai)[12]) {
-    Hop h, w;
+    Hop h;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {  // the four spin components of colour c
         float2 qr[12], qi[12];
@@ -251,8 +330,7 @@ __device__ __forceinline__ void hop_pair(const Field& x, int nb, int p, const fl
             h.i[k] = pmul(h.i[k], sc);
         }
     }
-    link_mul<(S > 0)>(link, h, w);
-    reconstruct_pair<MU, S>(w, nk, pk, ar, ai);
+    link_mul_add<MU, S>(GTab{reinterpret_cast<const float2*>(link)}, h, nk, pk, ar, ai);
 }
 
 template <int P, int MU>
@@ -262,186 +340,39 @@ __device__ __forceinline__ void hop_dir_pair(const DPairArgs& a, const int (&co)
     const int nf = co[MU] == Lm - 1 ? n - (Lm - 1) * sm : n + sm;
     const int nb = co[MU] == 0 ? n + (Lm - 1) * sm : n - sm;
     // forward: (1 - gamma_mu) U_mu(n) x(n + mu)
-    hop_pair<P, MU, -1>(a.x, nf, p, a.U + ((size_t)MU * a.V + n) * BK_LINK32_F4, nk, pk, ar, ai);
+    hop_pair<P, MU, -1>(a.x, nf, p, a.U + ((size_t)n * 4 + MU) * BK_LINKC, nk, pk, ar, ai);
     // backward: (1 + gamma_mu) U_mu(n - mu)^+ x(n - mu)
-    hop_pair<P, MU, +1>(a.x, nb, p, a.U + ((size_t)MU * a.V + nb) * BK_LINK32_F4, nk, pk, ar, ai);
+    hop_pair<P, MU, +1>(a.x, nb, p, a.U + ((size_t)nb * 4 + MU) * BK_LINKC, nk, pk, ar, ai);
 }
 
-// out = q - kappa C q for one chiral 6x6 Hermitian block pair (see gauge.cu
-// for the packed-pair clover order); the blocks act on u + l and u - l.
-__device__ __forceinline__ void clover_pair(const float4* __restrict__ c4, const float2 (&qr)[12],
-                                            const float2 (&qi)[12], float2 nk, float2 (&ar)[12], float2 (&ai)[12]) {
-    float2 yr[2][6], yi[2][6];
-#pragma unroll
-    for (int b = 0; b < 2; ++b) {
-        float2 vr[6], vi[6];
-#pragma unroll
-        for (int k = 0; k < 6; ++k) {
-            vr[k] = b == 0 ? padd(qr[k], qr[k + 6]) : psub(qr[k], qr[k + 6]);
-            vi[k] = b == 0 ? padd(qi[k], qi[k + 6]) : psub(qi[k], qi[k + 6]);
-        }
-        const float2* c2 = reinterpret_cast<const float2*>(c4);
-#pragma unroll
-        for (int i = 0; i < 6; ++i) {
-            const float2 d = __ldg(c2 + 90 + 6 * b + i);
-            yr[b][i] = pmul(d, vr[i]);
-            yi[b][i] = pmul(d, vi[i]);
-        }
-        int q = 0;
-#pragma unroll
-        for (int i = 1; i < 6; ++i)
-#pragma unroll
-            for (int j = 0; j < i; ++j, ++q) {
-                const float4 A = __ldg(c4 + 15 * b + q);
-                const float2 AR = make_float2(A.x, A.y), AI = make_float2(A.z, A.w);
-                const float2 NAI = __ldg(c2 + 60 + 15 * b + q);
-                // y_i += A v_j
-                yr[b][i] = pfma(AR, vr[j], yr[b][i]);
-                yr[b][i] = pfma(NAI, vi[j], yr[b][i]);
-                yi[b][i] = pfma(AR, vi[j], yi[b][i]);
-                yi[b][i] = pfma(AI, vr[j], yi[b][i]);
-                // y_j += conj(A) v_i
-                yr[b][j] = pfma(AR, vr[i], yr[b][j]);
-                yr[b][j] = pfma(AI, vi[i], yr[b][j]);
-                yi[b][j] = pfma(AR, vi[i], yi[b][j]);
-                yi[b][j] = pfma(NAI, vr[i], yi[b][j]);
-            }
-    }
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        ar[k] = pfma(nk, padd(yr[0][k], yr[1][k]), qr[k]);
-        ai[k] = pfma(nk, padd(yi[0][k], yi[1][k]), qi[k]);
-        ar[k + 6] = pfma(nk, psub(yr[0][k], yr[1][k]), qr[k + 6]);
-        ai[k + 6] = pfma(nk, psub(yi[0][k], yi[1][k]), qi[k + 6]);
-    }
-}
-
-// Prefetch (no register cost) of every row this thread will read: the eight
-// neighbours' spinor elements of its pair and the eight links, so that the
-// DRAM requests of all hops are in flight at once instead of one hop after
-// the other.  PF 1: into L2, PF 2: into L1.
-template <int PF>
-__device__ __forceinline__ void prefetch_row(const void* ptr) {
-    if constexpr (PF == 1) asm volatile("prefetch.global.L2 [%0];" ::"l"(ptr));
-    if constexpr (PF == 2) asm volatile("prefetch.global.L1 [%0];" ::"l"(ptr));
-}
-
-template <int P, int PF>
-__device__ __forceinline__ void prefetch_hops(const DPairArgs& a, const int (&co)[4], int n, int p) {
-    if constexpr (PF > 0) {
-        const int eb = Prec<P>::ebytes;
-#pragma unroll
-        for (int mu = 0; mu < 4; ++mu) {
-            const int Lm = a.L[mu], sm = a.st[mu];
-            const int nf = co[mu] == Lm - 1 ? n - (Lm - 1) * sm : n + sm;
-            const int nb = co[mu] == 0 ? n + (Lm - 1) * sm : n - sm;
-#pragma unroll
-            for (int k = 0; k < 12; ++k) {
-                prefetch_row<PF>((const char*)a.x.data + (((size_t)nf * 12 + k) * a.x.np + p) * eb);
-                prefetch_row<PF>((const char*)a.x.data + (((size_t)nb * 12 + k) * a.x.np + p) * eb);
-            }
-            const float4* lf = a.U + ((size_t)mu * a.V + n) * BK_LINK32_F4;
-            const float4* lb = a.U + ((size_t)mu * a.V + nb) * BK_LINK32_F4;
-            prefetch_row<PF>(lf);
-            prefetch_row<PF>(lf + 8);
-            prefetch_row<PF>(lb);
-            prefetch_row<PF>(lb + 8);
-        }
-    }
-}
-
-// Looped form (PF 3): the eight hops run as a loop the compiler does not
-// unroll, so only one hop's operands are live (fewer registers, more resident
-// warps); while hop h computes, the rows of hop h + 1 are prefetched into L1.
-template <int P>
-__device__ __forceinline__ void prefetch_hop_l1(const DPairArgs& a, int nbr, int mu, int link_site, int p) {
-    const int eb = Prec<P>::ebytes;
-#pragma unroll
-    for (int k = 0; k < 12; ++k)
-        asm volatile("prefetch.global.L1 [%0];" ::"l"((const char*)a.x.data + (((size_t)nbr * 12 + k) * a.x.np + p) * eb));
-    const float4* l = a.U + ((size_t)mu * a.V + link_site) * BK_LINK32_F4;
-    asm volatile("prefetch.global.L1 [%0];" ::"l"(l));
-    asm volatile("prefetch.global.L1 [%0];" ::"l"(l + 8));
-}
-
-template <int P>
-__device__ __forceinline__ void hops_looped(const DPairArgs& a, const int (&co)[4], int n, int p, float2 nk,
-                                            float2 pk, float2 (&ar)[12], float2 (&ai)[12]) {
-    int nbr[8];
-#pragma unroll
-    for (int mu = 0; mu < 4; ++mu) {
-        const int Lm = a.L[mu], sm = a.st[mu];
-        nbr[2 * mu] = co[mu] == Lm - 1 ? n - (Lm - 1) * sm : n + sm;
-        nbr[2 * mu + 1] = co[mu] == 0 ? n + (Lm - 1) * sm : n - sm;
-    }
-    prefetch_hop_l1<P>(a, nbr[0], 0, n, p);
-#pragma unroll 1
-    for (int h = 0; h < 8; ++h) {
-        const int mu = h >> 1;
-        const int nb = h == 0 ? nbr[0] : h == 1 ? nbr[1] : h == 2 ? nbr[2] : h == 3 ? nbr[3]
-                     : h == 4 ? nbr[4] : h == 5 ? nbr[5] : h == 6 ? nbr[6] : nbr[7];
-        if (h < 7) {
-            const int h1 = h + 1;
-            const int nb1 = h1 == 1 ? nbr[1] : h1 == 2 ? nbr[2] : h1 == 3 ? nbr[3] : h1 == 4 ? nbr[4]
-                          : h1 == 5 ? nbr[5] : h1 == 6 ? nbr[6] : nbr[7];
-            prefetch_hop_l1<P>(a, nb1, h1 >> 1, (h1 & 1) ? nb1 : n, p);
-        }
-        const float4* link = a.U + ((size_t)mu * a.V + ((h & 1) ? nb : n)) * BK_LINK32_F4;
-        switch (h) {
-            case 0: hop_pair<P, 0, -1>(a.x, nb, p, link, nk, pk, ar, ai); break;
-            case 1: hop_pair<P, 0, +1>(a.x, nb, p, link, nk, pk, ar, ai); break;
-            case 2: hop_pair<P, 1, -1>(a.x, nb, p, link, nk, pk, ar, ai); break;
-            case 3: hop_pair<P, 1, +1>(a.x, nb, p, link, nk, pk, ar, ai); break;
-            case 4: hop_pair<P, 2, -1>(a.x, nb, p, link, nk, pk, ar, ai); break;
-            case 5: hop_pair<P, 2, +1>(a.x, nb, p, link, nk, pk, ar, ai); break;
-            case 6: hop_pair<P, 3, -1>(a.x, nb, p, link, nk, pk, ar, ai); break;
-            default: hop_pair<P, 3, +1>(a.x, nb, p, link, nk, pk, ar, ai); break;
-        }
-    }
-}
-
-template <int P, int MAXT, int MINB, int PF>
-__global__ void __launch_bounds__(MAXT, MINB) k_dslash_pair(const __grid_constant__ DPairArgs a) {
-    // Thread order: pair groups of G pairs outermost, then sites, then the
-    // group's pairs.  The blocks run roughly in this order, so the neighbour
-    // rows a group needs one time slice later are still in L2 (the window is
-    // two time slices of G pairs, not of every column).
+// Blocks of 128 threads, MINB of them an SM (3: 168 registers, 4: 128).
+template <int P, int MINB>
+__global__ void __launch_bounds__(128, MINB) k_dslash_pair(const __grid_constant__ DPairArgs a) {
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= (long long)a.V * a.npl) return;
-    const long long per_group = (long long)a.V * a.G;
-    const int grp = (int)(g / per_group);
-    const long long r = g - (long long)grp * per_group;
-    const int gw = min(a.G, a.npl - grp * a.G);  // pairs in this group (the last may be short)
-    const int n = (int)(r / gw);
-    const int pl = grp * a.G + (int)(r - (long long)n * gw);
-    const int p = a.p0 + pl;
+    const int s = (int)(g / a.npl), pl = (int)(g - (long long)s * a.npl), p = a.p0 + pl;
     int co[4];
     {
-        int r = n;
-        co[0] = r % a.L[0];
-        r /= a.L[0];
-        co[1] = r % a.L[1];
-        r /= a.L[1];
-        co[2] = r % a.L[2];
-        co[3] = r / a.L[2];
+        int r = s;
+        co[3] = r / a.st[3];
+        r -= co[3] * a.st[3];
+        co[2] = r / a.st[2];
+        r -= co[2] * a.st[2];
+        co[1] = r / a.st[1];
+        co[0] = r - co[1] * a.st[1];
     }
-    prefetch_hops<P, PF>(a, co, n, p);
+    // (the site again from its coordinates: s itself would stay in a register
+    // throughout, and with it the kernel spills at 128)
+    const int n = co[0] + a.st[1] * co[1] + a.st[2] * co[2] + a.st[3] * co[3];
     const float2 nk = a.nk[pl];
     const float2 pk = make_float2(-nk.x, -nk.y);
     float2 ar[12], ai[12];
-    {   // out = x - kappa C x
-        float2 qr[12], qi[12];
-        load_pair<P>(a.x, n, p, qr, qi);
-        clover_pair(a.C + (size_t)n * BK_CLOV32_F4, qr, qi, nk, ar, ai);
-    }
-    if constexpr (PF == 3) {
-        hops_looped<P>(a, co, n, p, nk, pk, ar, ai);
-    } else {
-        hop_dir_pair<P, 0>(a, co, n, p, nk, pk, ar, ai);
-        hop_dir_pair<P, 1>(a, co, n, p, nk, pk, ar, ai);
-        hop_dir_pair<P, 2>(a, co, n, p, nk, pk, ar, ai);
-        hop_dir_pair<P, 3>(a, co, n, p, nk, pk, ar, ai);
-    }
+    load_pair<P>(a.x, n, p, ar, ai);  // out = x - kappa C x
+    site_term<true>(GTab{reinterpret_cast<const float2*>(a.C + (size_t)n * BK_CLOVC)}, nk, ar, ai);
+    hop_dir_pair<P, 0>(a, co, n, p, nk, pk, ar, ai);
+    hop_dir_pair<P, 1>(a, co, n, p, nk, pk, ar, ai);
+    hop_dir_pair<P, 2>(a, co, n, p, nk, pk, ar, ai);
+    hop_dir_pair<P, 3>(a, co, n, p, nk, pk, ar, ai);
     if (a.residual) {  // b - D x
         float2 br[12], bi[12];
         load_pair<P>(a.b, n, p, br, bi);
@@ -452,269 +383,6 @@ __global__ void __launch_bounds__(MAXT, MINB) k_dslash_pair(const __grid_constan
         }
     }
     store_pair<P>(a.y, n, p, ar, ai);
-}
-
-// Link product and reconstruction fused row by row: output colour i of both
-// half-spinor vectors is formed and added at once, so only one row of the
-// link and one colour of w are live.
-template <int MU, int S>
-__device__ __forceinline__ void link_mul_add(const float4* __restrict__ u4, const Hop& h, float2 nk, float2 pk,
-                                             float2 (&ar)[12], float2 (&ai)[12]) {
-    constexpr bool DAG = S > 0;
-    const float2* u2 = reinterpret_cast<const float2*>(u4);
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        float2 ur[3], ui[3], un[3];
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            const int e = DAG ? 3 * j + i : 3 * i + j;
-            const float4 q = __ldg(u4 + e);
-            ur[j] = make_float2(q.x, q.y);
-            ui[j] = make_float2(q.z, q.w);
-            un[j] = __ldg(u2 + 18 + e);
-        }
-        float2 wr[2], wi[2];
-#pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-            wr[hh] = make_float2(0.f, 0.f);
-            wi[hh] = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                const float2 hr = h.r[3 * hh + j], hi = h.i[3 * hh + j];
-                if constexpr (!DAG) {  // U_ij h_j
-                    wr[hh] = pfma(ur[j], hr, wr[hh]);
-                    wr[hh] = pfma(un[j], hi, wr[hh]);
-                    wi[hh] = pfma(ur[j], hi, wi[hh]);
-                    wi[hh] = pfma(ui[j], hr, wi[hh]);
-                } else {  // conj(U_ji) h_j
-                    wr[hh] = pfma(ur[j], hr, wr[hh]);
-                    wr[hh] = pfma(ui[j], hi, wr[hh]);
-                    wi[hh] = pfma(ur[j], hi, wi[hh]);
-                    wi[hh] = pfma(un[j], hr, wi[hh]);
-                }
-            }
-        }
-        reconstruct_colour<MU, S>(i, wr[0], wi[0], wr[1], wi[1], nk, pk, ar, ai);
-    }
-}
-
-// out = q - kappa C q with out holding q on entry; the two chiral blocks run
-// one after the other and add into out directly (fewer live registers than
-// clover_pair).
-__device__ __forceinline__ void clover_pair_inplace(const float4* __restrict__ c4, float2 nk, float2 (&ar)[12],
-                                                    float2 (&ai)[12]) {
-    const float2* c2 = reinterpret_cast<const float2*>(c4);
-    float2 vr[2][6], vi[2][6];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        vr[0][k] = padd(ar[k], ar[k + 6]);
-        vi[0][k] = padd(ai[k], ai[k + 6]);
-        vr[1][k] = psub(ar[k], ar[k + 6]);
-        vi[1][k] = psub(ai[k], ai[k + 6]);
-    }
-    const float2 pk = make_float2(-nk.x, -nk.y);
-#pragma unroll
-    for (int b = 0; b < 2; ++b) {
-        float2 yr[6], yi[6];
-#pragma unroll
-        for (int i = 0; i < 6; ++i) {
-            const float2 d = __ldg(c2 + 90 + 6 * b + i);
-            yr[i] = pmul(d, vr[b][i]);
-            yi[i] = pmul(d, vi[b][i]);
-        }
-        int q = 0;
-#pragma unroll
-        for (int i = 1; i < 6; ++i)
-#pragma unroll
-            for (int j = 0; j < i; ++j, ++q) {
-                const float4 A = __ldg(c4 + 15 * b + q);
-                const float2 AR = make_float2(A.x, A.y), AI = make_float2(A.z, A.w);
-                const float2 NAI = __ldg(c2 + 60 + 15 * b + q);
-                yr[i] = pfma(AR, vr[b][j], yr[i]);
-                yr[i] = pfma(NAI, vi[b][j], yr[i]);
-                yi[i] = pfma(AR, vi[b][j], yi[i]);
-                yi[i] = pfma(AI, vr[b][j], yi[i]);
-                yr[j] = pfma(AR, vr[b][i], yr[j]);
-                yr[j] = pfma(AI, vi[b][i], yr[j]);
-                yi[j] = pfma(AR, vi[b][i], yi[j]);
-                yi[j] = pfma(NAI, vr[b][i], yi[j]);
-            }
-        // upper half: -kappa y for both blocks; lower half: -kappa y (b = 0), +kappa y (b = 1)
-#pragma unroll
-        for (int k = 0; k < 6; ++k) {
-            ar[k] = pfma(nk, yr[k], ar[k]);
-            ai[k] = pfma(nk, yi[k], ai[k]);
-            ar[k + 6] = pfma(b == 0 ? nk : pk, yr[k], ar[k + 6]);
-            ai[k + 6] = pfma(b == 0 ? nk : pk, yi[k], ai[k + 6]);
-        }
-    }
-}
-
-// ---------------------------------------------------------------- staged form (FP32)
-//
-// The same operator with the spinor rows staged through shared memory by
-// asynchronous copies (cp.async, 16 bytes each, L2 to shared memory).  A
-// thread's work is ten stages: its own row (clover term), the eight hops, and
-// the right-hand side of the residual form; each stage's rows go into one of
-// NSLOT slots of the thread's own ring, and while a stage computes, the next
-// NSLOT - 1 stages are already on their way.  The copies hold no registers,
-// so a thread keeps whole hops in flight at the register cost of the
-// synchronous kernel.  No thread reads another thread's slots, so no barrier
-// is needed: each thread waits for its own copy groups only.
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
-
-constexpr int DA_STAGES = 10;  // own row, eight hops, right-hand side
-constexpr int DA_THREADS = 128;
-
-// rows of stage s at site `site` into the thread's slot (stride T float4)
-__device__ __forceinline__ void stage_issue(const DPairArgs& a, int s, int site, int p, float4* slot, int T) {
-    const Field& f = s == DA_STAGES - 1 ? a.b : a.x;
-    const float4* src = (const float4*)f.data + ((size_t)site * 12 * f.np + p);
-    const int k0 = s == 7 ? 6 : 0;   // forward t hop: spins 2, 3
-    const int k1 = s == 8 ? 6 : 12;  // backward t hop: spins 0, 1
-#pragma unroll
-    for (int k = 0; k < 12; ++k)
-        if (k >= k0 && k < k1) cp_async16(slot + k * T, src + (size_t)k * f.np);
-}
-
-template <int MU, int S>
-__device__ __forceinline__ void hop_staged(const float4* slot, int T, const float4* __restrict__ link, float2 nk,
-                                           float2 pk, float2 (&ar)[12], float2 (&ai)[12]) {
-    Hop h;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        float2 qr[12], qi[12];
-#pragma unroll
-        for (int sp = 0; sp < 4; ++sp) {
-            if (MU == 3 && ((S > 0) != (sp < 2))) continue;
-            const float4 q = slot[(3 * sp + c) * T];
-            qr[3 * sp + c] = make_float2(q.x, q.y);
-            qi[3 * sp + c] = make_float2(q.z, q.w);
-        }
-        Hop hc;
-        project_pair<MU, S>(qr, qi, hc, c);
-        h.r[c] = hc.r[c];
-        h.i[c] = hc.i[c];
-        h.r[3 + c] = hc.r[3 + c];
-        h.i[3 + c] = hc.i[3 + c];
-    }
-    link_mul_add<MU, S>(link, h, nk, pk, ar, ai);
-}
-
-// Stage S of the staged kernel: wait for its rows, compute, refill its slot
-// with stage S + NSLOT.  A template, so that every stage's hop, wait count
-// and slot are compile-time constants.
-template <int S, int NSLOT>
-__device__ __forceinline__ void run_stage(const DPairArgs& a, const int (&site)[DA_STAGES], int n, int p,
-                                          float4* ring, float2 nk, float2 pk, float2 (&ar)[12], float2 (&ai)[12]) {
-    constexpr int T = DA_THREADS;
-    // stage S complete; the later ones may still be in flight
-    constexpr int pending = (DA_STAGES - 1 - S) < (NSLOT - 1) ? (DA_STAGES - 1 - S) : (NSLOT - 1);
-    cp_async_wait<pending>();
-    const float4* slot = ring + (S % NSLOT) * 12 * T;
-    if constexpr (S == 0) {  // out = x - kappa C x
-#pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            const float4 q = slot[k * T];
-            ar[k] = make_float2(q.x, q.y);
-            ai[k] = make_float2(q.z, q.w);
-        }
-        clover_pair_inplace(a.C + (size_t)n * BK_CLOV32_F4, nk, ar, ai);
-    } else if constexpr (S < DA_STAGES - 1) {
-        constexpr int hop = S - 1, MU = hop >> 1, SG = (hop & 1) ? +1 : -1;
-        const float4* link = a.U + ((size_t)MU * a.V + ((hop & 1) ? site[S] : n)) * BK_LINK32_F4;
-        hop_staged<MU, SG>(slot, T, link, nk, pk, ar, ai);
-    } else {
-        if (a.residual) {  // b - D x
-#pragma unroll
-            for (int k = 0; k < 12; ++k) {
-                const float4 q = slot[k * T];
-                ar[k] = psub(make_float2(q.x, q.y), ar[k]);
-                ai[k] = psub(make_float2(q.z, q.w), ai[k]);
-            }
-        }
-    }
-    // refill the slot just read with stage S + NSLOT (its link lines prefetched)
-    constexpr int SN = S + NSLOT;
-    if constexpr (SN < DA_STAGES) {
-        if (SN < DA_STAGES - 1 || a.residual) stage_issue(a, SN, site[SN], p, ring + (SN % NSLOT) * 12 * T, T);
-        if constexpr (SN >= 1 && SN < DA_STAGES - 1) {
-            constexpr int hop = SN - 1;
-            const char* l =
-                (const char*)(a.U + ((size_t)(hop >> 1) * a.V + ((hop & 1) ? site[SN] : n)) * BK_LINK32_F4);
-            asm volatile("prefetch.global.L1 [%0];" ::"l"(l));
-            asm volatile("prefetch.global.L1 [%0];" ::"l"(l + 128));
-            asm volatile("prefetch.global.L1 [%0];" ::"l"(l + 223));
-        }
-        cp_async_commit();
-    }
-}
-
-template <int NSLOT, int MINB>
-__global__ void __launch_bounds__(DA_THREADS, MINB) k_dslash_staged(const __grid_constant__ DPairArgs a) {
-    extern __shared__ float4 da_ring[];  // [NSLOT][12][DA_THREADS]
-    constexpr int T = DA_THREADS;
-    const int t = threadIdx.x;
-    const long long g = (long long)blockIdx.x * T + t;
-    if (g >= (long long)a.V * a.npl) return;  // no barriers below
-    const long long per_group = (long long)a.V * a.G;
-    const int grp = (int)(g / per_group);
-    const long long r = g - (long long)grp * per_group;
-    const int gw = min(a.G, a.npl - grp * a.G);
-    const int n = (int)(r / gw);
-    const int pl = grp * a.G + (int)(r - (long long)n * gw);
-    const int p = a.p0 + pl;
-    int site[DA_STAGES];
-    {
-        int co[4], rr = n;
-        co[0] = rr % a.L[0];
-        rr /= a.L[0];
-        co[1] = rr % a.L[1];
-        rr /= a.L[1];
-        co[2] = rr % a.L[2];
-        co[3] = rr / a.L[2];
-        site[0] = n;
-#pragma unroll
-        for (int mu = 0; mu < 4; ++mu) {
-            const int Lm = a.L[mu], sm = a.st[mu];
-            site[1 + 2 * mu] = co[mu] == Lm - 1 ? n - (Lm - 1) * sm : n + sm;  // forward
-            site[2 + 2 * mu] = co[mu] == 0 ? n + (Lm - 1) * sm : n - sm;       // backward
-        }
-        site[DA_STAGES - 1] = n;
-    }
-    float4* ring = da_ring + t;
-    {   // the site's clover entries, needed first
-        const char* cl = (const char*)(a.C + (size_t)n * BK_CLOV32_F4);
-#pragma unroll
-        for (int l = 0; l < 7; ++l) asm volatile("prefetch.global.L1 [%0];" ::"l"(cl + 128 * l));
-    }
-#pragma unroll
-    for (int s = 0; s < NSLOT; ++s) {
-        stage_issue(a, s, site[s], p, ring + s * 12 * T, T);
-        cp_async_commit();
-    }
-    const float2 nk = a.nk[pl];
-    const float2 pk = make_float2(-nk.x, -nk.y);
-    float2 ar[12], ai[12];
-    run_stage<0, NSLOT>(a, site, n, p, ring, nk, pk, ar, ai);
-    run_stage<1, NSLOT>(a, site, n, p, ring, nk, pk, ar, ai);
-    run_stage<2, NSLOT>(a, site, n, p, ring, nk, pk, ar, ai);
-    run_stage<3, NSLOT>(a, site, n, p, ring, nk, pk, ar, ai);
-    run_stage<4, NSLOT>(a, site, n, p, ring, nk, pk, ar, ai);
-    run_stage<5, NSLOT>(a, site, n, p, ring, nk, pk, ar, ai);
-    run_stage<6, NSLOT>(a, site, n, p, ring, nk, pk, ar, ai);
-    run_stage<7, NSLOT>(a, site, n, p, ring, nk, pk, ar, ai);
-    run_stage<8, NSLOT>(a, site, n, p, ring, nk, pk, ar, ai);
-    run_stage<9, NSLOT>(a, site, n, p, ring, nk, pk, ar, ai);
-    store_pair<BK_FP32>(a.y, n, p, ar, ai);
 }
 
 // ================================================================= FP64 / double-float: one column per thread
@@ -1039,6 +707,12 @@ void geometry(const int dims[4], int (&L)[4], int (&st)[4]) {
     }
 }
 
+// Blocks an SM of the pair kernels.  Measured (us, 3 / 4): FP32 full operator
+// 16^3x32, 30 columns 291 / 284, 60 columns 543 / 537, 24^3x48, 96 columns
+// 4234 / 4245, 8^3x16, 12 columns (less than one wave) 12.6 / 14.7; FP16
+// 16^3x32, 30 columns 279 / 281.
+int pair_blocks(int prec, long long items) { return prec == BK_FP32 && items > 152LL * 3 * 128 ? 4 : 3; }
+
 template <int P>
 bk_status dslash_pair_impl(const DslashOp& op, cudaStream_t st) {
     // launch over whole pairs [col0 / 2, (col0 + ncol + 1) / 2)
@@ -1050,8 +724,8 @@ bk_status dslash_pair_impl(const DslashOp& op, cudaStream_t st) {
         a.x = op.x;
         a.y = op.y;
         a.b = op.b;
-        a.U = (const float4*)op.U;
-        a.C = (const float4*)op.clov;
+        a.U = (const float*)op.U;
+        a.C = (const float*)op.clov;
         geometry(op.dims, a.L, a.st);
         a.V = op.V;
         a.p0 = q0;
@@ -1065,41 +739,10 @@ bk_status dslash_pair_impl(const DslashOp& op, cudaStream_t st) {
             const double kb = (cb >= 0 && cb < op.ncol) ? op.kappa[cb] : 0.0;
             a.nk[j] = make_float2((float)-ka, (float)-kb);
         }
-        // variants: register cap 255 (1: 1 block of 256), 170 (2: 3 blocks of
-        // 128), 128 (3: 4 blocks of 128); FP32 staged form 4, 5 (k_dslash_staged)
-        int threads = op.threads > 0 ? op.threads : 128;
-        if (op.variant >= 2 && threads > 128) threads = 128;
-        a.G = op.group > 0 ? std::min(op.group, npl) : npl;
         const long long items = (long long)op.V * npl;
-        const unsigned blocks = (unsigned)((items + threads - 1) / threads);
-        // op.prefetch: 0 none, 1 into L2, 2 into L1 (see prefetch_hops)
-#define BK_DP(MT, MB)                                                                    \
-    if (op.prefetch == 1) k_dslash_pair<P, MT, MB, 1><<<blocks, threads, 0, st>>>(a);    \
-    else if (op.prefetch == 2) k_dslash_pair<P, MT, MB, 2><<<blocks, threads, 0, st>>>(a); \
-    else if (op.prefetch == 3) k_dslash_pair<P, MT, MB, 3><<<blocks, threads, 0, st>>>(a); \
-    else k_dslash_pair<P, MT, MB, 0><<<blocks, threads, 0, st>>>(a);
-        if (P == BK_FP32 && (op.variant == 4 || op.variant == 5)) {
-            // staged form: 128 threads, ring of 2 (variant 4) or 3 (variant 5) slots
-            const unsigned sb = (unsigned)((items + DA_THREADS - 1) / DA_THREADS);
-            if (op.variant == 4) {
-                const size_t smem = (size_t)2 * 12 * DA_THREADS * sizeof(float4);
-                BK_CUDA_TRY(cudaFuncSetAttribute(k_dslash_staged<2, 4>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-                k_dslash_staged<2, 4><<<sb, DA_THREADS, smem, st>>>(a);
-            } else {
-                const size_t smem = (size_t)3 * 12 * DA_THREADS * sizeof(float4);
-                BK_CUDA_TRY(cudaFuncSetAttribute(k_dslash_staged<3, 3>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-                k_dslash_staged<3, 3><<<sb, DA_THREADS, smem, st>>>(a);
-            }
-        } else if (op.variant == 1) {
-            BK_DP(256, 1)
-        } else if (op.variant == 3) {
-            BK_DP(128, 4)
-        } else {
-            BK_DP(128, 3)
-        }
-#undef BK_DP
+        const unsigned blocks = (unsigned)((items + 127) / 128);
+        if (pair_blocks(P, items) == 4) k_dslash_pair<P, 4><<<blocks, 128, 0, st>>>(a);
+        else k_dslash_pair<P, 3><<<blocks, 128, 0, st>>>(a);
         BK_CUDA_TRY(cudaGetLastError());
     }
     return BK_OK;
@@ -1307,82 +950,21 @@ __device__ __forceinline__ int eo_site(int h, int par, const int (&L)[4], int (&
     return n;
 }
 
-// out = A^-1 in for one column pair, in place: the table's blocks act on
-// v0 = u + l and v1 = u - l; u = y0 + y1, l = y0 - y1 (same packing as the clover)
-__device__ __forceinline__ void herm_pair_inplace(const float4* __restrict__ c4, float2 (&ar)[12], float2 (&ai)[12]) {
-    const float2* c2 = reinterpret_cast<const float2*>(c4);
-    float2 vr[2][6], vi[2][6];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        vr[0][k] = padd(ar[k], ar[k + 6]);
-        vi[0][k] = padd(ai[k], ai[k + 6]);
-        vr[1][k] = psub(ar[k], ar[k + 6]);
-        vi[1][k] = psub(ai[k], ai[k + 6]);
-    }
-#pragma unroll
-    for (int b = 0; b < 2; ++b) {
-        float2 yr[6], yi[6];
-#pragma unroll
-        for (int i = 0; i < 6; ++i) {
-            const float2 d = __ldg(c2 + 90 + 6 * b + i);
-            yr[i] = pmul(d, vr[b][i]);
-            yi[i] = pmul(d, vi[b][i]);
-        }
-        int q = 0;
-#pragma unroll
-        for (int i = 1; i < 6; ++i)
-#pragma unroll
-            for (int j = 0; j < i; ++j, ++q) {
-                const float4 A = __ldg(c4 + 15 * b + q);
-                const float2 AR = make_float2(A.x, A.y), AI = make_float2(A.z, A.w);
-                const float2 NAI = __ldg(c2 + 60 + 15 * b + q);
-                yr[i] = pfma(AR, vr[b][j], yr[i]);
-                yr[i] = pfma(NAI, vi[b][j], yr[i]);
-                yi[i] = pfma(AR, vi[b][j], yi[i]);
-                yi[i] = pfma(AI, vr[b][j], yi[i]);
-                yr[j] = pfma(AR, vr[b][i], yr[j]);
-                yr[j] = pfma(AI, vi[b][i], yr[j]);
-                yi[j] = pfma(AR, vi[b][i], yi[j]);
-                yi[j] = pfma(NAI, vr[b][i], yi[j]);
-            }
-#pragma unroll
-        for (int k = 0; k < 6; ++k) {
-            if (b == 0) {
-                ar[k] = yr[k];
-                ai[k] = yi[k];
-                ar[k + 6] = yr[k];
-                ai[k + 6] = yi[k];
-            } else {
-                ar[k] = padd(ar[k], yr[k]);
-                ai[k] = padd(ai[k], yi[k]);
-                ar[k + 6] = psub(ar[k + 6], yr[k]);
-                ai[k + 6] = psub(ai[k + 6], yi[k]);
-            }
-        }
-    }
-}
-
 struct EOPairArgs {
     Field in, xs, y;  // in: the other parity; xs: this parity (mode 2); y: the output (this parity)
-    const float4* __restrict__ U;      // packed-pair links, full-site index
-    const float4* Ci[BK_MAX_COLS / 2];  // packed-pair A^-1 table of launch pair p - p0 (its kappa)
+    const float* __restrict__ U;       // compact links, full-site index
+    const float* Ci[BK_MAX_COLS / 2];  // compact A^-1 table of launch pair p - p0 (its kappa)
     int L[4], st[4];
-    int V, Vh, p0, npl, par, mode, G;
+    int V, Vh, p0, npl, par, mode;
     float2 mk2[BK_MAX_COLS / 2];  // mode 2: {-kappa^2} of the pair's columns
 };
 
 // mode 1: y = A^-1 H in;  mode 2: y = xs - kappa^2 A^-1 H in  (FP32 / FP16 storage)
-template <int P, int MAXT, int MINB>
-__global__ void __launch_bounds__(MAXT, MINB) k_eo_pair(const __grid_constant__ EOPairArgs a) {
+template <int P, int MINB>
+__global__ void __launch_bounds__(128, MINB) k_eo_pair(const __grid_constant__ EOPairArgs a) {
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= (long long)a.Vh * a.npl) return;
-    const long long per_group = (long long)a.Vh * a.G;
-    const int grp = (int)(g / per_group);
-    const long long r = g - (long long)grp * per_group;
-    const int gw = min(a.G, a.npl - grp * a.G);
-    const int h = (int)(r / gw);
-    const int pl = grp * a.G + (int)(r - (long long)h * gw);
-    const int p = a.p0 + pl;
+    const int h = (int)(g / a.npl), pl = (int)(g - (long long)h * a.npl), p = a.p0 + pl;
     int co[4];
     const int n = eo_site(h, a.par, a.L, co);
     const float2 one = make_float2(1.f, 1.f), mone = make_float2(-1.f, -1.f);
@@ -1394,15 +976,15 @@ __global__ void __launch_bounds__(MAXT, MINB) k_eo_pair(const __grid_constant__ 
         const int Lm = a.L[MU], sm = a.st[MU];                                                                 \
         const int nf = co[MU] == Lm - 1 ? n - (Lm - 1) * sm : n + sm;                                          \
         const int nb = co[MU] == 0 ? n + (Lm - 1) * sm : n - sm;                                               \
-        hop_pair<P, MU, -1>(a.in, nf >> 1, p, a.U + ((size_t)MU * a.V + n) * BK_LINK32_F4, one, mone, ar, ai); \
-        hop_pair<P, MU, +1>(a.in, nb >> 1, p, a.U + ((size_t)MU * a.V + nb) * BK_LINK32_F4, one, mone, ar, ai); \
+        hop_pair<P, MU, -1>(a.in, nf >> 1, p, a.U + ((size_t)n * 4 + MU) * BK_LINKC, one, mone, ar, ai); \
+        hop_pair<P, MU, +1>(a.in, nb >> 1, p, a.U + ((size_t)nb * 4 + MU) * BK_LINKC, one, mone, ar, ai); \
     }
     BK_EO_DIR(0)
     BK_EO_DIR(1)
     BK_EO_DIR(2)
     BK_EO_DIR(3)
 #undef BK_EO_DIR
-    herm_pair_inplace(a.Ci[pl] + (size_t)n * BK_CLOV32_F4, ar, ai);
+    site_term<false>(GTab{reinterpret_cast<const float2*>(a.Ci[pl] + (size_t)n * BK_CLOVC)}, one, ar, ai);
     if (a.mode == 2) {
         float2 xr[12], xi[12];
         load_pair<P>(a.xs, h, p, xr, xi);
@@ -1414,111 +996,6 @@ __global__ void __launch_bounds__(MAXT, MINB) k_eo_pair(const __grid_constant__ 
         }
     }
     store_pair<P>(a.y, h, p, ar, ai);
-}
-
-// Staged form of k_eo_pair (FP32): the eight hops' rows of the other parity
-// and, in mode 2, the thread's own row of xs go through the same per-thread
-// cp.async ring as k_dslash_staged (stages: eight hops, then xs).
-constexpr int EA_STAGES = 9;
-
-__device__ __forceinline__ void eo_stage_issue(const EOPairArgs& a, int s, int hsite, int p, float4* slot, int T) {
-    const Field& f = s == EA_STAGES - 1 ? a.xs : a.in;
-    const float4* src = (const float4*)f.data + ((size_t)hsite * 12 * f.np + p);
-    const int k0 = s == 6 ? 6 : 0;   // forward t hop: spins 2, 3
-    const int k1 = s == 7 ? 6 : 12;  // backward t hop: spins 0, 1
-#pragma unroll
-    for (int k = 0; k < 12; ++k)
-        if (k >= k0 && k < k1) cp_async16(slot + k * T, src + (size_t)k * f.np);
-}
-
-template <int S, int NSLOT>
-__device__ __forceinline__ void eo_run_stage(const EOPairArgs& a, const int (&hs)[EA_STAGES], const int (&ls)[8],
-                                             int n, int p, int pl, float4* ring, float2 (&ar)[12], float2 (&ai)[12]) {
-    constexpr int T = DA_THREADS;
-    constexpr int pending = (EA_STAGES - 1 - S) < (NSLOT - 1) ? (EA_STAGES - 1 - S) : (NSLOT - 1);
-    cp_async_wait<pending>();
-    const float4* slot = ring + (S % NSLOT) * 12 * T;
-    if constexpr (S < EA_STAGES - 1) {
-        constexpr int MU = S >> 1, SG = (S & 1) ? +1 : -1;
-        const float4* link = a.U + ((size_t)MU * a.V + ls[S]) * BK_LINK32_F4;
-        hop_staged<MU, SG>(slot, T, link, make_float2(1.f, 1.f), make_float2(-1.f, -1.f), ar, ai);
-        if constexpr (S == EA_STAGES - 2) herm_pair_inplace(a.Ci[pl] + (size_t)n * BK_CLOV32_F4, ar, ai);
-    } else {
-        if (a.mode == 2) {  // xs - kappa^2 A^-1 H in
-            const float2 m = a.mk2[pl];
-#pragma unroll
-            for (int k = 0; k < 12; ++k) {
-                const float4 q = slot[k * T];
-                ar[k] = pfma(m, ar[k], make_float2(q.x, q.y));
-                ai[k] = pfma(m, ai[k], make_float2(q.z, q.w));
-            }
-        }
-    }
-    constexpr int SN = S + NSLOT;
-    if constexpr (SN < EA_STAGES) {
-        if (SN < EA_STAGES - 1 || a.mode == 2) eo_stage_issue(a, SN, hs[SN], p, ring + (SN % NSLOT) * 12 * T, T);
-        if constexpr (SN < EA_STAGES - 1) {
-            const char* l = (const char*)(a.U + ((size_t)(SN >> 1) * a.V + ls[SN]) * BK_LINK32_F4);
-            asm volatile("prefetch.global.L1 [%0];" ::"l"(l));
-            asm volatile("prefetch.global.L1 [%0];" ::"l"(l + 128));
-            asm volatile("prefetch.global.L1 [%0];" ::"l"(l + 223));
-        }
-        cp_async_commit();
-    }
-}
-
-template <int NSLOT, int MINB>
-__global__ void __launch_bounds__(DA_THREADS, MINB) k_eo_staged(const __grid_constant__ EOPairArgs a) {
-    extern __shared__ float4 ea_ring[];  // [NSLOT][12][DA_THREADS]
-    constexpr int T = DA_THREADS;
-    const int t = threadIdx.x;
-    const long long g = (long long)blockIdx.x * T + t;
-    if (g >= (long long)a.Vh * a.npl) return;  // no barriers below
-    const long long per_group = (long long)a.Vh * a.G;
-    const int grp = (int)(g / per_group);
-    const long long r = g - (long long)grp * per_group;
-    const int gw = min(a.G, a.npl - grp * a.G);
-    const int h = (int)(r / gw);
-    const int pl = grp * a.G + (int)(r - (long long)h * gw);
-    const int p = a.p0 + pl;
-    int co[4];
-    const int n = eo_site(h, a.par, a.L, co);
-    int hs[EA_STAGES], ls[8];  // half-lattice row of each stage; link site of each hop
-#pragma unroll
-    for (int mu = 0; mu < 4; ++mu) {
-        const int Lm = a.L[mu], sm = a.st[mu];
-        const int nf = co[mu] == Lm - 1 ? n - (Lm - 1) * sm : n + sm;
-        const int nb = co[mu] == 0 ? n + (Lm - 1) * sm : n - sm;
-        hs[2 * mu] = nf >> 1;
-        hs[2 * mu + 1] = nb >> 1;
-        ls[2 * mu] = n;
-        ls[2 * mu + 1] = nb;
-    }
-    hs[EA_STAGES - 1] = h;
-    float4* ring = ea_ring + t;
-    {   // the site's A^-1 entries, needed after the hops
-        const char* cl = (const char*)(a.Ci[pl] + (size_t)n * BK_CLOV32_F4);
-#pragma unroll
-        for (int l = 0; l < 7; ++l) asm volatile("prefetch.global.L2 [%0];" ::"l"(cl + 128 * l));
-    }
-#pragma unroll
-    for (int s = 0; s < NSLOT; ++s) {
-        eo_stage_issue(a, s, hs[s], p, ring + s * 12 * T, T);
-        cp_async_commit();
-    }
-    float2 ar[12], ai[12];
-#pragma unroll
-    for (int k = 0; k < 12; ++k) ar[k] = ai[k] = make_float2(0.f, 0.f);
-    eo_run_stage<0, NSLOT>(a, hs, ls, n, p, pl, ring, ar, ai);
-    eo_run_stage<1, NSLOT>(a, hs, ls, n, p, pl, ring, ar, ai);
-    eo_run_stage<2, NSLOT>(a, hs, ls, n, p, pl, ring, ar, ai);
-    eo_run_stage<3, NSLOT>(a, hs, ls, n, p, pl, ring, ar, ai);
-    eo_run_stage<4, NSLOT>(a, hs, ls, n, p, pl, ring, ar, ai);
-    eo_run_stage<5, NSLOT>(a, hs, ls, n, p, pl, ring, ar, ai);
-    eo_run_stage<6, NSLOT>(a, hs, ls, n, p, pl, ring, ar, ai);
-    eo_run_stage<7, NSLOT>(a, hs, ls, n, p, pl, ring, ar, ai);
-    eo_run_stage<8, NSLOT>(a, hs, ls, n, p, pl, ring, ar, ai);
-    store_pair<BK_FP32>(a.y, h, p, ar, ai);
 }
 
 template <int P>
@@ -1648,7 +1125,7 @@ bk_status eo_pair_impl(const EoOp& op, cudaStream_t st) {
         a.in = op.x;
         a.xs = op.xs;
         a.y = op.y;
-        a.U = (const float4*)op.U;
+        a.U = (const float*)op.U;
         int st4[4];
         geometry(op.dims, a.L, st4);
         for (int mu = 0; mu < 4; ++mu) a.st[mu] = st4[mu];
@@ -1664,32 +1141,13 @@ bk_status eo_pair_impl(const EoOp& op, cudaStream_t st) {
             const int ca = 2 * (q0 + j) - op.col0, cb = ca + 1;
             const bool ina = ca >= 0 && ca < op.ncol, inb = cb >= 0 && cb < op.ncol;
             const double ka = ina ? op.kappa[ca] : 0.0, kb = inb ? op.kappa[cb] : 0.0;
-            a.Ci[j] = (const float4*)op.Ci[ina ? ca : cb];
+            a.Ci[j] = (const float*)op.Ci[ina ? ca : cb];
             a.mk2[j] = make_float2((float)(-ka * ka), (float)(-kb * kb));
         }
-        const int threads = op.variant == 1 ? 256 : 128;
-        a.G = op.group > 0 ? std::min(op.group, npl) : npl;
         const long long items = (long long)a.Vh * npl;
-        const unsigned blocks = (unsigned)((items + threads - 1) / threads);
-        if (P == BK_FP32 && (op.variant == 4 || op.variant == 5)) {
-            // staged form: ring of 2 (variant 4) or 3 (variant 5) slots per thread
-            const unsigned sb = (unsigned)((items + DA_THREADS - 1) / DA_THREADS);
-            if (op.variant == 4) {
-                const size_t smem = (size_t)2 * 12 * DA_THREADS * sizeof(float4);
-                BK_CUDA_TRY(cudaFuncSetAttribute(k_eo_staged<2, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)smem));
-                k_eo_staged<2, 4><<<sb, DA_THREADS, smem, st>>>(a);
-            } else {
-                const size_t smem = (size_t)3 * 12 * DA_THREADS * sizeof(float4);
-                BK_CUDA_TRY(cudaFuncSetAttribute(k_eo_staged<3, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)smem));
-                k_eo_staged<3, 3><<<sb, DA_THREADS, smem, st>>>(a);
-            }
-        } else if (op.variant == 1) {
-            k_eo_pair<P, 256, 1><<<blocks, threads, 0, st>>>(a);
-        } else {
-            k_eo_pair<P, 128, 3><<<blocks, threads, 0, st>>>(a);
-        }
+        const unsigned blocks = (unsigned)((items + 127) / 128);
+        if (pair_blocks(P, items) == 4) k_eo_pair<P, 4><<<blocks, 128, 0, st>>>(a);
+        else k_eo_pair<P, 3><<<blocks, 128, 0, st>>>(a);
         BK_CUDA_TRY(cudaGetLastError());
     }
     return BK_OK;

@@ -4,16 +4,11 @@
 //  * FP64: [mu][9 = 3a + b][site] complex (double2), so that a warp reading
 //    one matrix element for 32 consecutive sites issues one coalesced
 //    transaction (the FP64 operator takes one column per thread);
-//  * FP32, for the packed-pair operator (one thread per site and column
-//    pair, every lane of a warp on the same site): per (mu, site) 224 bytes,
-//    float2 pairs {u_r, u_r}, {u_i, u_i} of element e at float4 e (e < 9),
-//    then {-u_i, -u_i} of element e at float2 18 + e (one pad pair), so
-//    that every product with a column pair is a packed multiply-add with no
-//    operand shuffling.
+//  * FP32: per site its four links side by side, each 9 complex elements and
+//    one of padding (80 bytes: a multiple of 16 for the tiled operator's copies).
 //
 // Clover: the FP64 copy is [36][site] double2 (72 reals per site); the FP32
-// copy is per site 816 bytes in the same packed-pair form (see
-// k_clover_build).  The site term C(n) = c_SW sum_{mu,nu} (i/2)
+// copy is the 72 reals of a site side by side.  The site term C(n) = c_SW sum_{mu,nu} (i/2)
 // sigma_mu_nu F_mu_nu(n) commutes with gamma_5, so in the basis
 // a = u + l, b = u - l (u = spins 0,1, l = spins 2,3) it is block diagonal:
 //     (C q)_u = A' a + B' b,   (C q)_l = A' a - B' b,
@@ -175,22 +170,19 @@ __device__ M3 field_strength(const double2* __restrict__ U, const Geo& g, const 
 }
 
 __global__ void k_gauge_convert(const double2* __restrict__ Uin, double2* __restrict__ U64,
-                                float4* __restrict__ U32, int V) {
+                                float* __restrict__ U32, int V) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     const int mu = blockIdx.y;
     if (s >= V) return;
     const double2* p = Uin + ((size_t)mu * V + s) * 9;
-    float4* o = U32 + ((size_t)mu * V + s) * BK_LINK32_F4;
-    float2* on = reinterpret_cast<float2*>(o) + 18;
+    float2* o = reinterpret_cast<float2*>(U32 + ((size_t)s * 4 + mu) * BK_LINKC);
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
         double2 q = p[k];
         U64[(size_t)(mu * 9 + k) * V + s] = q;
-        const float ur = (float)q.x, ui = (float)q.y;
-        o[k] = make_float4(ur, ur, ui, ui);
-        on[k] = make_float2(-ui, -ui);
+        o[k] = make_float2((float)q.x, (float)q.y);
     }
-    on[9] = make_float2(0.f, 0.f);
+    o[9] = make_float2(0.f, 0.f);
 }
 
 // Chiral 6x6 block from (G1, G2, G3), scaled: blk = scale * [[-G3, -G1 + iG2], [-G1 - iG2, G3]].
@@ -203,12 +195,9 @@ __device__ __forceinline__ cx<double> chiral_elem(const M3& G1, const M3& G2, co
     return mk(-g1.r, -g1.i) - ti(g2);
 }
 
-// FP32 packed-pair clover, per site (float2 index within the site's 816 bytes):
-//   [0, 60):    block b, entry q < 15: {A_r, A_r} at 2 (15 b + q), {A_i, A_i} at 2 (15 b + q) + 1
-//   [60, 90):   {-A_i, -A_i} of block b, entry q at 60 + 15 b + q
-//   [90, 102):  diagonal {d, d} of block b, row i at 90 + 6 b + i
+// The FP32 copy holds the same 72 reals of a site side by side.
 __global__ void k_clover_build(const double2* __restrict__ U, double2* __restrict__ C64,
-                               float4* __restrict__ C32, Geo g, int V, double csw) {
+                               float* __restrict__ C32, Geo g, int V, double csw) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= V) return;
     int c[4];
@@ -258,20 +247,10 @@ __global__ void k_clover_build(const double2* __restrict__ U, double2* __restric
     }
 #pragma unroll
     for (int q = 0; q < 36; ++q) C64[(size_t)q * V + s] = make_double2(out[2 * q], out[2 * q + 1]);
-    float2* c2 = reinterpret_cast<float2*>(C32 + (size_t)s * BK_CLOV32_F4);
+    float4* cc = reinterpret_cast<float4*>(C32 + (size_t)s * BK_CLOVC);
 #pragma unroll
-    for (int b = 0; b < 2; ++b) {
-        const double* o = out + 36 * b;
-#pragma unroll
-        for (int q = 0; q < 15; ++q) {
-            const float ar = (float)o[6 + 2 * q], ai = (float)o[7 + 2 * q];
-            c2[2 * (15 * b + q)] = make_float2(ar, ar);
-            c2[2 * (15 * b + q) + 1] = make_float2(ai, ai);
-            c2[60 + 15 * b + q] = make_float2(-ai, -ai);
-        }
-#pragma unroll
-        for (int i = 0; i < 6; ++i) c2[90 + 6 * b + i] = make_float2((float)o[i], (float)o[i]);
-    }
+    for (int q = 0; q < 18; ++q)
+        cc[q] = make_float4((float)out[4 * q], (float)out[4 * q + 1], (float)out[4 * q + 2], (float)out[4 * q + 3]);
 }
 
 // ---------------------------------------------------------------- clover inverse
@@ -282,13 +261,13 @@ __global__ void k_clover_build(const double2* __restrict__ U, double2* __restric
 // inverses of those two 6x6 matrices,
 //     (A^-1 q)_u = (Pa/2) a + (Pb/2) b,   (A^-1 q)_l = (Pa/2) a - (Pb/2) b,
 // the same form as C q: Pa/2 and Pb/2 are stored exactly like A' and B'
-// (FP64 [36][site] and FP32 packed pairs).  Each block is inverted in FP64 by
+// (FP64 [36][site] and FP32).  Each block is inverted in FP64 by
 // Gauss-Jordan elimination with partial pivoting.  bound[0] receives the
 // largest infinity norm of (1 - 2 kappa A'), (1 - 2 kappa B') over the sites
 // (>= the spectral norm of A(n), used to scale the Schur system's stopping
 // rule); bound[1] counts blocks whose pivot fell below 1e-12 (singular A).
 __global__ void k_clover_inverse(const double2* __restrict__ C64, double kappa, double2* __restrict__ Ci64,
-                                 float4* __restrict__ Ci32, int V, unsigned long long* __restrict__ bound) {
+                                 float* __restrict__ Ci32, int V, unsigned long long* __restrict__ bound) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= V) return;
     double out[72];
@@ -374,20 +353,10 @@ __global__ void k_clover_inverse(const double2* __restrict__ C64, double kappa, 
     }
 #pragma unroll
     for (int q = 0; q < 36; ++q) Ci64[(size_t)q * V + s] = make_double2(out[2 * q], out[2 * q + 1]);
-    float2* c2 = reinterpret_cast<float2*>(Ci32 + (size_t)s * BK_CLOV32_F4);
+    float4* cc = reinterpret_cast<float4*>(Ci32 + (size_t)s * BK_CLOVC);
 #pragma unroll
-    for (int b = 0; b < 2; ++b) {
-        const double* o = out + 36 * b;
-#pragma unroll
-        for (int q = 0; q < 15; ++q) {
-            const float ar = (float)o[6 + 2 * q], ai = (float)o[7 + 2 * q];
-            c2[2 * (15 * b + q)] = make_float2(ar, ar);
-            c2[2 * (15 * b + q) + 1] = make_float2(ai, ai);
-            c2[60 + 15 * b + q] = make_float2(-ai, -ai);
-        }
-#pragma unroll
-        for (int i = 0; i < 6; ++i) c2[90 + 6 * b + i] = make_float2((float)o[i], (float)o[i]);
-    }
+    for (int q = 0; q < 18; ++q)
+        cc[q] = make_float4((float)out[4 * q], (float)out[4 * q + 1], (float)out[4 * q + 2], (float)out[4 * q + 3]);
     // non-negative doubles order like their bit patterns
     atomicMax(bound, (unsigned long long)__double_as_longlong(nmax));
     if (singular) atomicAdd(bound + 1, 1ull);
@@ -395,14 +364,14 @@ __global__ void k_clover_inverse(const double2* __restrict__ C64, double kappa, 
 
 }  // namespace
 
-bk_status launch_gauge_convert(const double* Uin_dev, double2* U64, float4* U32, int V, cudaStream_t st) {
+bk_status launch_gauge_convert(const double* Uin_dev, double2* U64, float* U32, int V, cudaStream_t st) {
     dim3 grid((V + 127) / 128, 4);
     k_gauge_convert<<<grid, 128, 0, st>>>((const double2*)Uin_dev, U64, U32, V);
     BK_CUDA_TRY(cudaGetLastError());
     return BK_OK;
 }
 
-bk_status launch_clover_build(const double2* U64, double2* C64, float4* C32, const int dims[4], double csw,
+bk_status launch_clover_build(const double2* U64, double2* C64, float* C32, const int dims[4], double csw,
                               cudaStream_t st) {
     Geo g;
     int stride = 1;
@@ -417,7 +386,7 @@ bk_status launch_clover_build(const double2* U64, double2* C64, float4* C32, con
     return BK_OK;
 }
 
-bk_status launch_clover_inverse(const double2* C64, double kappa, double2* Ci64, float4* Ci32, int V,
+bk_status launch_clover_inverse(const double2* C64, double kappa, double2* Ci64, float* Ci32, int V,
                                 unsigned long long* bound, cudaStream_t st) {
     k_clover_inverse<<<(V + 63) / 64, 64, 0, st>>>(C64, kappa, Ci64, Ci32, V, bound);
     BK_CUDA_TRY(cudaGetLastError());
