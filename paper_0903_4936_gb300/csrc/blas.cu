@@ -996,7 +996,7 @@ bk_status gram_dispatch(int prec, Field A, Field B, Field B2, int NB, const SysP
 
 // partial-sum rows of a Gram matrix over the active systems
 static int gram_chunks(int prec, const SysPart& p, int V) {
-    return max_active_L(p) <= ROWS_MAXL ? gram_row_chunks(prec, V, row_tiles(p)) : wide_gram_chunks(p, V);
+    return max_active_L(p) <= ROWS_MAXL ? gram_row_chunks(prec, V, row_tiles(prec, p)) : wide_gram_chunks(p, V);
 }
 
 size_t gram_partial_bytes(const SysPart& p, int V) {

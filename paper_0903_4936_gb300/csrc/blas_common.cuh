@@ -179,7 +179,7 @@ inline int gram_row_chunks(int prec, int V, const PTiles& t) {
 inline int gram_row_chunks_max(int V) { return std::max(1, std::min(12 * V / 4, 304)); }
 bk_status rows_gram(int prec, Field A, Field B, Field B2, int NB, const SysPart& p, double2* partial, int nchunk,
                     int V, cudaStream_t st);
-PTiles row_tiles(const SysPart& p);
+PTiles row_tiles(int prec, const SysPart& p);
 bk_status rows_update(int prec, const GenOp& g, int V, int nchunk, int np, cudaStream_t st);
 // GenOp's unit flags and whether it uses M
 inline GenOp with_units(GenOp g) {

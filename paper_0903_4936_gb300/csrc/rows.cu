@@ -19,6 +19,20 @@ namespace {
 
 constexpr int GW = 8;  // warps per block
 
+// Consecutive row groups a warp takes at a time: up to 12 (a site's rows when
+// one row fills the warp), so that the lines its rows share and their DRAM
+// pages are used together (16^3x32, 60 columns, even sites, X and R update: 494
+// us with single rows strided over the grid, 340 with whole sites); fewer where
+// the groups do not go round.
+__device__ __forceinline__ unsigned row_run(unsigned units, unsigned warps) {
+    return min(12u, max(1u, units / warps));
+}
+// The warp's place among all warps: neighbours in a block take neighbouring
+// runs; where there are fewer row groups than warps the blocks share them out.
+__device__ __forceinline__ unsigned warp_place(unsigned units, int nchunk, int chunk, int w) {
+    return units < (unsigned)nchunk * GW ? (unsigned)w * nchunk + chunk : (unsigned)chunk * GW + w;
+}
+
 struct RLane {
     bool live;  // the lane holds a pair of an active system
     int sub, q, s, Ls, i0, nps, base;  // row of the group, pair, system, its size, first column, pairs, first lane
@@ -77,7 +91,8 @@ __global__ void __launch_bounds__(GW * 32, P == BK_FP64 ? 1 : 2) k_gram_r(Field 
         for (int ii = 0; ii < 2; ++ii)
 #pragma unroll
             for (int jp = 0; jp < MAXL / 2; ++jp) acc[b][ii][jp] = cp_zero<R2>();
-    const unsigned units = (rows + spw - 1) / spw, nw = (unsigned)nchunk * GW, wid = (unsigned)w * nchunk + chunk;
+    const unsigned units = (rows + spw - 1) / spw, nw = (unsigned)nchunk * GW;
+    const unsigned wid = warp_place(units, nchunk, chunk, w);
     bool first = true;
     int since = 0;
     auto flush = [&]() {
@@ -117,15 +132,17 @@ __global__ void __launch_bounds__(GW * 32, P == BK_FP64 ? 1 : 2) k_gram_r(Field 
         first = false;
         since = 0;
     };
-    for (unsigned u0 = wid; u0 < units; u0 += nw * UR) {
+    const unsigned run = row_run(units, nw);
+    for (unsigned u1 = wid * run; u1 < units; u1 += nw * run)
+    for (unsigned u0 = u1; u0 < min(u1 + run, units); u0 += UR) {
         CxPair<R2> av[UR], bv[UR][NB];
 #pragma unroll
         for (int x = 0; x < UR; ++x) {
-            const unsigned u = u0 + x * nw, row = u * spw + L.sub;
+            const unsigned u = u0 + x, row = u * spw + L.sub;
             av[x] = cp_zero<R2>();
 #pragma unroll
             for (int b = 0; b < NB; ++b) bv[x][b] = cp_zero<R2>();
-            if (L.live && u < units && row < rows) {
+            if (L.live && u < min(u1 + run, units) && row < rows) {
                 const size_t e = (size_t)row * np + L.q;
                 R2 sa = pzero<R2>(), sb[NB];
 #pragma unroll
@@ -167,11 +184,12 @@ __global__ void __launch_bounds__(GW * 32, P == BK_FP64 ? 1 : 2) k_gram_r(Field 
             if (since >= ROW_FLUSH) flush();
         }
     }
-    if (wid < units && (first || since > 0)) flush();
+    if (wid * run < units && (first || since > 0)) flush();
     __syncthreads();
     // the block's partial sums: one thread per (operand, column of the pair, column, pair)
     const int ne = p.coef_off[p.nsys];
-    const int nact = min(GW, (int)((units - min(units, (unsigned)chunk) + nchunk - 1) / nchunk));  // warps with rows
+    int nact = 0;  // warps with rows (the first of the block)
+    while (nact < GW && warp_place(units, nchunk, chunk, nact) * run < units) ++nact;
     const int estr = P == BK_FP64 || spw == 1 ? 32 : tnp, nsub = P == BK_FP64 ? spw : 1;
     for (int x = threadIdx.x; x < tnp * NACC; x += GW * 32) {
         const int e = x / tnp, pr = x - e * tnp, j = e % MAXL, ii = (e / MAXL) & 1, b = e / (2 * MAXL);
@@ -203,7 +221,7 @@ bk_status run_gram_r(Field A, Field B0, Field B1, const SysPart& p, const PTiles
 template <int P>
 bk_status rows_gram_p(Field A, Field B, Field B2, int NB, const SysPart& p, double2* part, int nchunk, int V,
                       cudaStream_t st) {
-    const PTiles wt = row_tiles(p);
+    const PTiles wt = row_tiles(P, p);
     const int maxL = max_active_L(p);
     const int ne = p.coef_off[p.nsys];
     constexpr int UR = P == BK_FP64 ? 2 : 4;
@@ -247,7 +265,8 @@ __global__ void __launch_bounds__(GW * 32, MINB) k_update_r(const __grid_constan
     const int chunk = blockIdx.y;
     const int tp0 = wt.p0[blockIdx.x], tnp = wt.np[blockIdx.x];
     const int spw = 32 / tnp;
-    const unsigned units = (rows + spw - 1) / spw, nw = (unsigned)nchunk * GW, wid = (unsigned)w * nchunk + chunk;
+    const unsigned units = (rows + spw - 1) / spw, nw = (unsigned)nchunk * GW;
+    const unsigned wid = warp_place(units, nchunk, chunk, w);
     if (wid >= units && !g.ynorm) return;
     const RLane L = rlane(g.p, tp0, tnp, lane);
     const bool act = L.live && !(g.skip && g.skip[L.s]);
@@ -299,14 +318,16 @@ __global__ void __launch_bounds__(GW * 32, MINB) k_update_r(const __grid_constan
     int since = 0;
     const CxPair<R2> zero = cp_zero<R2>();
     constexpr int XP = P;  // X accumulates in the block's precision (FP32 or FP64)
-    for (unsigned u0 = wid; u0 < units; u0 += nw * UR) {
+    const unsigned run = row_run(units, nw);
+    for (unsigned u1 = wid * run; u1 < units; u1 += nw * run)
+    for (unsigned u0 = u1; u0 < min(u1 + run, units); u0 += UR) {
         CxPair<R2> vm[UR][MMI > 0 ? MMI : 1], ve[UR][ME > 0 ? ME : 1], vx[UR], xo[UR];
         bool on[UR];
         size_t ee[UR];
 #pragma unroll
         for (int x = 0; x < UR; ++x) {
-            const unsigned u = u0 + x * nw, row = u * spw + L.sub;
-            on[x] = act && u < units && row < rows;
+            const unsigned u = u0 + x, row = u * spw + L.sub;
+            on[x] = act && u < min(u1 + run, units) && row < rows;
             ee[x] = (size_t)row * np + L.q;
             const R2 one = bcast(R(1));
 #pragma unroll
@@ -421,13 +442,15 @@ __global__ void __launch_bounds__(GW * 32, MINB) k_update_r(const __grid_constan
 
 }  // namespace
 
-// Tiles of the row kernels: runs of whole active systems, their width chosen
-// to keep the most lanes busy.  A tile of tnp pairs costs 1 / floor(32 / tnp)
-// of a warp step per row; the widest of the cheapest splittings wins (wider
-// tiles read longer contiguous runs).
-PTiles row_tiles(const SysPart& p) {
-    PTiles best;
-    best.n = 0;
+// Tiles of the row kernels: runs of whole active systems.  FP32 / FP16: the
+// widest that fit a warp, since memory bounds them and a narrow tile reads
+// scattered pieces of the rows (10 systems of 6, 6 and 2 columns, X and R
+// update: six tiles of 5 pairs 594 us, one of 30 pairs 380).  FP64: the width
+// that keeps the most lanes busy (a tile of tnp pairs costs 1 / floor(32 /
+// tnp) of a warp step per row; the widest of the cheapest splittings).
+PTiles row_tiles(int prec, const SysPart& p) {
+    PTiles best = make_ptiles(p, 32);
+    if (prec != BK_FP64) return best;
     double cost = 1e30;
     for (int maxp = 32; maxp >= ROWS_MAXL / 2; --maxp) {
         const PTiles t = make_ptiles(p, maxp);
@@ -452,7 +475,7 @@ bk_status rows_gram(int prec, Field A, Field B, Field B2, int NB, const SysPart&
 }
 
 bk_status rows_update(int prec, const GenOp& g, int V, int nchunk, int np, cudaStream_t st) {
-    const PTiles wt = row_tiles(g.p);
+    const PTiles wt = row_tiles(prec, g.p);
     const dim3 grid(wt.n, nchunk);
     const int ncols = g.p.col0[g.p.nsys];
     const unsigned rows = 12u * (unsigned)V;
