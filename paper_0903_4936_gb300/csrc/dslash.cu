@@ -711,6 +711,9 @@ void geometry(const int dims[4], int (&L)[4], int (&st)[4]) {
 // 16^3x32, 30 columns 291 / 284, 60 columns 543 / 537, 24^3x48, 96 columns
 // 4234 / 4245, 8^3x16, 12 columns (less than one wave) 12.6 / 14.7; FP16
 // 16^3x32, 30 columns 279 / 281.
+// Below one wave single-warp blocks even out the SMs' shares (192 blocks of 128
+// threads give 40 SMs twice the work of the others).
+int pair_threads(long long items) { return items <= 152LL * 3 * 128 ? 32 : 128; }
 int pair_blocks(int prec, long long items) { return prec == BK_FP32 && items > 152LL * 3 * 128 ? 4 : 3; }
 
 template <int P>
@@ -740,9 +743,10 @@ bk_status dslash_pair_impl(const DslashOp& op, cudaStream_t st) {
             a.nk[j] = make_float2((float)-ka, (float)-kb);
         }
         const long long items = (long long)op.V * npl;
-        const unsigned blocks = (unsigned)((items + 127) / 128);
-        if (pair_blocks(P, items) == 4) k_dslash_pair<P, 4><<<blocks, 128, 0, st>>>(a);
-        else k_dslash_pair<P, 3><<<blocks, 128, 0, st>>>(a);
+        const int T = pair_threads(items);
+        const unsigned blocks = (unsigned)((items + T - 1) / T);
+        if (pair_blocks(P, items) == 4) k_dslash_pair<P, 4><<<blocks, T, 0, st>>>(a);
+        else k_dslash_pair<P, 3><<<blocks, T, 0, st>>>(a);
         BK_CUDA_TRY(cudaGetLastError());
     }
     return BK_OK;
@@ -787,10 +791,97 @@ bk_status dslash_col_impl(const DslashOp& op, cudaStream_t st) {
 
 // ================================================================= conversions
 
-// canonical column j (of a chunk of ncan columns) -> device column dcol[j]
-// (dcol == nullptr: dbase + j).  Threads: x = canonical column, y = site.
-template <int P>
-__global__ void k_pack(const double2* __restrict__ canon, int ncan, const int* __restrict__ dcol, int dbase, Field f) {
+// FP64 / FP32: canonical column j (of a chunk of ncan columns) <-> device column
+// dcol[j] (dcol == nullptr: dbase + j), through a shared-memory tile of CT_S
+// sites x CT_C columns: a canonical column is contiguous along (site,
+// component), a device row along the columns, so one side of a direct copy
+// touches a separate line per lane (12 columns, 16^3x32, FP64: 205 us each way,
+// now 100; 60 columns out: 1980, now 480).
+constexpr int CT_S = 8, CT_C = 16, CT_R = CT_S * 12;
+
+__device__ __forceinline__ int dev_col(const int* dcol, int dbase, int j) { return dcol ? __ldg(dcol + j) : dbase + j; }
+
+template <int P, bool PACK>
+__global__ void __launch_bounds__(256) k_convert(double2* __restrict__ canon, int ncan, const int* __restrict__ dcol,
+                                                 int dbase, Field f) {
+    __shared__ double2 tile[CT_R][CT_C + 1];
+    const int j0 = blockIdx.y * CT_C, nj = min(CT_C, ncan - j0);
+    const int n0 = blockIdx.x * CT_S, nr = 12 * min(CT_S, f.V - n0);
+    const int t = threadIdx.x;
+    auto canonical = [&]() {  // rows fastest
+        for (int e = t; e < nj * CT_R; e += 256) {
+            const int j = e / CT_R, r = e - j * CT_R;
+            if (r >= nr) continue;
+            double2* q = canon + ((size_t)(j0 + j) * f.V + n0) * 12 + r;
+            if (PACK) tile[r][j] = *q;
+            else *q = tile[r][j];
+        }
+    };
+    auto device = [&]() {  // columns fastest
+        int cw = CT_C;  // columns side by side: a power of two that covers the tile's
+        while (cw / 2 >= nj) cw /= 2;
+        const int j = t & (cw - 1);
+        if (j >= nj) return;
+        const int c = dev_col(dcol, dbase, j0 + j), half = c & 1;
+        // both columns of a pair in the tile side by side: the even one's thread takes them
+        const bool both = !half && j + 1 < nj && dev_col(dcol, dbase, j0 + j + 1) == c + 1;
+        if (half && j > 0 && dev_col(dcol, dbase, j0 + j - 1) == c - 1) return;
+        for (int r = t / cw; r < nr; r += 256 / cw) {
+            const size_t e = ((size_t)n0 * 12 + r) * f.np + (c >> 1);
+            if constexpr (P == BK_FP64) {
+                double2* q = (double2*)f.data + 2 * e;
+                if (both) {
+                    if (PACK) {
+                        const double2 a = tile[r][j], b = tile[r][j + 1];
+                        q[0] = make_double2(a.x, b.x);
+                        q[1] = make_double2(a.y, b.y);
+                    } else {
+                        const double2 re = q[0], im = q[1];
+                        tile[r][j] = make_double2(re.x, im.x);
+                        tile[r][j + 1] = make_double2(re.y, im.y);
+                    }
+                } else {
+                    double* s = (double*)q + half;
+                    if (PACK) {
+                        s[0] = tile[r][j].x;
+                        s[2] = tile[r][j].y;
+                    } else {
+                        tile[r][j] = make_double2(s[0], s[2]);
+                    }
+                }
+            } else {
+                float4* q = (float4*)f.data + e;
+                if (both) {
+                    if (PACK) {
+                        const double2 a = tile[r][j], b = tile[r][j + 1];
+                        *q = make_float4(d2f(a.x), d2f(b.x), d2f(a.y), d2f(b.y));
+                    } else {
+                        const float4 v = *q;
+                        tile[r][j] = make_double2(f2d(v.x), f2d(v.z));
+                        tile[r][j + 1] = make_double2(f2d(v.y), f2d(v.w));
+                    }
+                } else {
+                    float* s = (float*)q + half;
+                    if (PACK) {
+                        s[0] = d2f(tile[r][j].x);
+                        s[2] = d2f(tile[r][j].y);
+                    } else {
+                        tile[r][j] = make_double2(f2d(s[0]), f2d(s[2]));
+                    }
+                }
+            }
+        }
+    };
+    if (PACK) canonical();
+    else device();
+    __syncthreads();
+    if (PACK) device();
+    else canonical();
+}
+
+// FP16: the same with one thread per (canonical column, site), which forms or
+// applies the column's scale, its largest component rounded to FP32 first.
+__global__ void k_pack16(const double2* __restrict__ canon, int ncan, const int* __restrict__ dcol, int dbase, Field f) {
     const int j = blockIdx.y * blockDim.x + threadIdx.x;
     const int n = blockIdx.x * blockDim.y + threadIdx.y;
     if (j >= ncan || n >= f.V) return;
@@ -801,40 +892,20 @@ __global__ void k_pack(const double2* __restrict__ canon, int ncan, const int* _
     double2 v[12];
 #pragma unroll
     for (int k = 0; k < 12; ++k) v[k] = src[k];
-    if constexpr (P == BK_FP64) {
-        double* q = (double*)f.data + 4 * e0 + half;
+    float m = 0.f;
 #pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            q[4 * (size_t)k * f.np] = v[k].x;
-            q[4 * (size_t)k * f.np + 2] = v[k].y;
-        }
-    } else if constexpr (P == BK_FP32) {
-        float* q = (float*)f.data + 4 * e0 + half;
+    for (int k = 0; k < 12; ++k) m = fmaxf(m, fmaxf(fabsf((float)v[k].x), fabsf((float)v[k].y)));
+    const float inv = m > 0.f ? 1.0f / m : 0.f;
+    __half* q = (__half*)f.data + 4 * e0 + half;
 #pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            q[4 * (size_t)k * f.np] = (float)v[k].x;
-            q[4 * (size_t)k * f.np + 2] = (float)v[k].y;
-        }
-    } else {
-        // the column's scale: its largest component, rounded to FP32 first
-        float m = 0.f;
-#pragma unroll
-        for (int k = 0; k < 12; ++k) m = fmaxf(m, fmaxf(fabsf((float)v[k].x), fabsf((float)v[k].y)));
-        const float inv = m > 0.f ? 1.0f / m : 0.f;
-        __half* q = (__half*)f.data + 4 * e0 + half;
-#pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            q[4 * (size_t)k * f.np] = __float2half_rn((float)v[k].x * inv);
-            q[4 * (size_t)k * f.np + 2] = __float2half_rn((float)v[k].y * inv);
-        }
-        float* sc = (float*)(f.norm + (size_t)n * f.np + (c >> 1));
-        sc[half] = m;
+    for (int k = 0; k < 12; ++k) {
+        q[4 * (size_t)k * f.np] = __float2half_rn((float)v[k].x * inv);
+        q[4 * (size_t)k * f.np + 2] = __float2half_rn((float)v[k].y * inv);
     }
+    float* sc = (float*)(f.norm + (size_t)n * f.np + (c >> 1));
+    sc[half] = m;
 }
-
-// device column dcol[j] (or dbase + j) -> canonical column j of the chunk
-template <int P>
-__global__ void k_unpack(Field f, const int* __restrict__ dcol, int dbase, double2* __restrict__ canon, int ncan) {
+__global__ void k_unpack16(Field f, const int* __restrict__ dcol, int dbase, double2* __restrict__ canon, int ncan) {
     const int j = blockIdx.y * blockDim.x + threadIdx.x;
     const int n = blockIdx.x * blockDim.y + threadIdx.y;
     if (j >= ncan || n >= f.V) return;
@@ -842,22 +913,12 @@ __global__ void k_unpack(Field f, const int* __restrict__ dcol, int dbase, doubl
     double2* dst = canon + ((size_t)j * f.V + n) * 12;
     const size_t e0 = (size_t)n * 12 * f.np + (c >> 1);
     const int half = c & 1;
-    if constexpr (P == BK_FP64) {
-        const double* q = (const double*)f.data + 4 * e0 + half;
+    const __half* q = (const __half*)f.data + 4 * e0 + half;
+    const float m = ((const float*)(f.norm + (size_t)n * f.np + (c >> 1)))[half];
 #pragma unroll
-        for (int k = 0; k < 12; ++k) dst[k] = make_double2(q[4 * (size_t)k * f.np], q[4 * (size_t)k * f.np + 2]);
-    } else if constexpr (P == BK_FP32) {
-        const float* q = (const float*)f.data + 4 * e0 + half;
-#pragma unroll
-        for (int k = 0; k < 12; ++k) dst[k] = make_double2(q[4 * (size_t)k * f.np], q[4 * (size_t)k * f.np + 2]);
-    } else {
-        const __half* q = (const __half*)f.data + 4 * e0 + half;
-        const float m = ((const float*)(f.norm + (size_t)n * f.np + (c >> 1)))[half];
-#pragma unroll
-        for (int k = 0; k < 12; ++k)
-            dst[k] = make_double2((double)(__half2float(q[4 * (size_t)k * f.np]) * m),
-                                  (double)(__half2float(q[4 * (size_t)k * f.np + 2]) * m));
-    }
+    for (int k = 0; k < 12; ++k)
+        dst[k] = make_double2((double)(__half2float(q[4 * (size_t)k * f.np]) * m),
+                              (double)(__half2float(q[4 * (size_t)k * f.np + 2]) * m));
 }
 
 // zero device column c (both parts, every site and component)
@@ -1145,9 +1206,10 @@ bk_status eo_pair_impl(const EoOp& op, cudaStream_t st) {
             a.mk2[j] = make_float2((float)(-ka * ka), (float)(-kb * kb));
         }
         const long long items = (long long)a.Vh * npl;
-        const unsigned blocks = (unsigned)((items + 127) / 128);
-        if (pair_blocks(P, items) == 4) k_eo_pair<P, 4><<<blocks, 128, 0, st>>>(a);
-        else k_eo_pair<P, 3><<<blocks, 128, 0, st>>>(a);
+        const int T = pair_threads(items);
+        const unsigned blocks = (unsigned)((items + T - 1) / T);
+        if (pair_blocks(P, items) == 4) k_eo_pair<P, 4><<<blocks, T, 0, st>>>(a);
+        else k_eo_pair<P, 3><<<blocks, T, 0, st>>>(a);
         BK_CUDA_TRY(cudaGetLastError());
     }
     return BK_OK;
@@ -1200,12 +1262,14 @@ bk_status launch_dslash(int prec, const DslashOp& op, cudaStream_t st) {
 bk_status launch_pack(int prec, const double* canon, int ncan, const int* dcol, int dbase, Field f, cudaStream_t st) {
     if (ncan <= 0) return BK_OK;
     // sites on grid.x (up to 2^31 - 1 blocks), columns on grid.y
-    dim3 blk(32, 8), grid((f.V + 7) / 8, (ncan + 31) / 32);
-    const double2* c = (const double2*)canon;
+    const dim3 tiles((f.V + CT_S - 1) / CT_S, (ncan + CT_C - 1) / CT_C);
+    double2* c = (double2*)canon;
     switch (prec) {
-        case BK_FP64: k_pack<BK_FP64><<<grid, blk, 0, st>>>(c, ncan, dcol, dbase, f); break;
-        case BK_FP32: k_pack<BK_FP32><<<grid, blk, 0, st>>>(c, ncan, dcol, dbase, f); break;
-        case BK_FP16: k_pack<BK_FP16><<<grid, blk, 0, st>>>(c, ncan, dcol, dbase, f); break;
+        case BK_FP64: k_convert<BK_FP64, true><<<tiles, 256, 0, st>>>(c, ncan, dcol, dbase, f); break;
+        case BK_FP32: k_convert<BK_FP32, true><<<tiles, 256, 0, st>>>(c, ncan, dcol, dbase, f); break;
+        case BK_FP16:
+            k_pack16<<<dim3((f.V + 7) / 8, (ncan + 31) / 32), dim3(32, 8), 0, st>>>(c, ncan, dcol, dbase, f);
+            break;
         default: return BK_ERR_INVALID_ARG;
     }
     BK_CUDA_TRY(cudaGetLastError());
@@ -1214,13 +1278,14 @@ bk_status launch_pack(int prec, const double* canon, int ncan, const int* dcol, 
 
 bk_status launch_unpack(int prec, Field f, const int* dcol, int dbase, double* canon, int ncan, cudaStream_t st) {
     if (ncan <= 0) return BK_OK;
-    // sites on grid.x (up to 2^31 - 1 blocks), columns on grid.y
-    dim3 blk(32, 8), grid((f.V + 7) / 8, (ncan + 31) / 32);
+    const dim3 tiles((f.V + CT_S - 1) / CT_S, (ncan + CT_C - 1) / CT_C);
     double2* c = (double2*)canon;
     switch (prec) {
-        case BK_FP64: k_unpack<BK_FP64><<<grid, blk, 0, st>>>(f, dcol, dbase, c, ncan); break;
-        case BK_FP32: k_unpack<BK_FP32><<<grid, blk, 0, st>>>(f, dcol, dbase, c, ncan); break;
-        case BK_FP16: k_unpack<BK_FP16><<<grid, blk, 0, st>>>(f, dcol, dbase, c, ncan); break;
+        case BK_FP64: k_convert<BK_FP64, false><<<tiles, 256, 0, st>>>(c, ncan, dcol, dbase, f); break;
+        case BK_FP32: k_convert<BK_FP32, false><<<tiles, 256, 0, st>>>(c, ncan, dcol, dbase, f); break;
+        case BK_FP16:
+            k_unpack16<<<dim3((f.V + 7) / 8, (ncan + 31) / 32), dim3(32, 8), 0, st>>>(f, dcol, dbase, c, ncan);
+            break;
         default: return BK_ERR_INVALID_ARG;
     }
     BK_CUDA_TRY(cudaGetLastError());

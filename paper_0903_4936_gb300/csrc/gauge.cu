@@ -100,6 +100,16 @@ struct Geo {
     int st[4];
 };
 
+__device__ __forceinline__ void coords(const Geo& g, int s, int (&c)[4]) {
+    int r = s;
+    c[0] = r % g.L[0];
+    r /= g.L[0];
+    c[1] = r % g.L[1];
+    r /= g.L[1];
+    c[2] = r % g.L[2];
+    c[3] = r / g.L[2];
+}
+
 __device__ __forceinline__ int hop(const Geo& g, const int (&c)[4], int s, int mu, int d) {
     int x = c[mu] + d;
     int s2 = s + d * g.st[mu];
@@ -114,59 +124,98 @@ __device__ __forceinline__ int hop(const Geo& g, const int (&c)[4], int s, int m
 //   P3 = U_mu(n-mu)^+ U_nu(n-mu-nu)^+ U_mu(n-mu-nu) U_nu(n-nu)
 //   P4 = U_nu(n-nu)^+ U_mu(n-nu) U_nu(n+mu-nu) U_mu(n)^+
 // F = (1/4) sum_i (P_i - P_i^+) / (2i).
-__device__ M3 field_strength(const double2* __restrict__ U, const Geo& g, const int (&c)[4], int s, int V,
-                             int mu, int nu) {
-    const int sp_m = hop(g, c, s, mu, +1), sm_m = hop(g, c, s, mu, -1);
-    const int sp_n = hop(g, c, s, nu, +1), sm_n = hop(g, c, s, nu, -1);
-    int cm[4] = {c[0], c[1], c[2], c[3]};
-    cm[mu] = (c[mu] + g.L[mu] - 1) % g.L[mu];
-    const int sm_m_p_n = hop(g, cm, sm_m, nu, +1);
-    const int sm_m_m_n = hop(g, cm, sm_m, nu, -1);
-    int cp[4] = {c[0], c[1], c[2], c[3]};
-    cp[mu] = (c[mu] + 1) % g.L[mu];
-    const int sp_m_m_n = hop(g, cp, sp_m, nu, -1);
+//
+// The four leaves that contain one plaquette (corner x) are the cyclic
+// products of its links, so with its two corner products
+//   M(x) = U_nu(x+mu) U_mu(x+nu)^+,  N(x) = U_nu(x)^+ U_mu(x)
+// they read P1(x) = U_mu(x) M(x) U_nu(x)^+, P2(x+mu) = M(x) N(x), P3(x+mu+nu) =
+// U_mu(x+nu)^+ N(x) U_nu(x+mu) and P4(x+nu) = N(x) M(x): 8 products of 3 x 3
+// matrices per site and plane instead of 12 (FP64 multiply-adds are what the
+// clover term costs: 16^3x32 1940 us in one kernel with 12, see
+// launch_clover_build).  Plane by plane: k_corner writes M and N, k_leaves
+// gathers the leaves at a site.
 
-    const M3 Um = ldU(U, mu, s, V), Un = ldU(U, nu, s, V);
+// blockIdx.y 0: M, 1: N.  MN: [18][V].
+__global__ void __launch_bounds__(64) k_corner(const double2* __restrict__ U, double2* __restrict__ MN, Geo g, int V,
+                                               int mu, int nu) {
+    const int x = blockIdx.x * 64 + threadIdx.x;
+    if (x >= V) return;
+    M3 r;
+    if (blockIdx.y == 0) {
+        int c[4];
+        coords(g, x, c);
+        r = mmd(ldU(U, nu, hop(g, c, x, mu, +1), V), ldU(U, mu, hop(g, c, x, nu, +1), V));
+    } else {
+        r = mdm(ldU(U, nu, x, V), ldU(U, mu, x, V));
+    }
+#pragma unroll
+    for (int k = 0; k < 9; ++k) MN[(size_t)(9 * blockIdx.y + k) * V + x] = make_double2(r.m[k / 3][k % 3].r, r.m[k / 3][k % 3].i);
+}
+
+__device__ __forceinline__ void add3(M3& a, const M3& b) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) a.m[i][j] = a.m[i][j] + b.m[i][j];
+}
+
+// F of one plane, Hermitian, as 9 reals in 5 slots of F [5][V]: {F00, F11},
+// {F22, 0}, F01, F02, F12.  Two warps share 32 sites, two leaves each.
+__global__ void __launch_bounds__(64) k_leaves(const double2* __restrict__ U, const double2* __restrict__ MN,
+                                               double2* __restrict__ F, Geo g, int V, int mu, int nu) {
+    __shared__ double2 other[9][32];
+    const int lane = threadIdx.x & 31, half = threadIdx.x >> 5;
+    const int s = blockIdx.x * 32 + lane;
     M3 Q;
-    // P1
-    M3 t = mm(Um, ldU(U, nu, sp_m, V));
-    t = mmd(t, ldU(U, mu, sp_n, V));
-    M3 P = mmd(t, Un);
-    Q = P;
-    // P2
-    t = mmd(Un, ldU(U, mu, sm_m_p_n, V));
-    t = mmd(t, ldU(U, nu, sm_m, V));
-    P = mm(t, ldU(U, mu, sm_m, V));
+    if (s < V) {
+        int c[4];
+        coords(g, s, c);
+        const int sm = hop(g, c, s, mu, -1), sn = hop(g, c, s, nu, -1);
+        if (half == 0) {  // P1 and P4
+            Q = mmd(mm(ldU(U, mu, s, V), ldU(MN, 0, s, V)), ldU(U, nu, s, V));
+            add3(Q, mm(ldU(MN, 1, sn, V), ldU(MN, 0, sn, V)));
+        } else {  // P2 and P3
+            int cm[4] = {c[0], c[1], c[2], c[3]};
+            cm[mu] = (c[mu] + g.L[mu] - 1) % g.L[mu];
+            Q = mm(ldU(MN, 0, sm, V), ldU(MN, 1, sm, V));
+            add3(Q, mm(mdm(ldU(U, mu, sm, V), ldU(MN, 1, hop(g, cm, sm, nu, -1), V)), ldU(U, nu, sn, V)));
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) Q.m[i][j] = Q.m[i][j] + P.m[i][j];
-    // P3
-    t = mdd(ldU(U, mu, sm_m, V), ldU(U, nu, sm_m_m_n, V));
-    t = mm(t, ldU(U, mu, sm_m_m_n, V));
-    P = mm(t, ldU(U, nu, sm_n, V));
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) Q.m[i][j] = Q.m[i][j] + P.m[i][j];
-    // P4
-    t = mdm(ldU(U, nu, sm_n, V), ldU(U, mu, sm_n, V));
-    t = mm(t, ldU(U, nu, sp_m_m_n, V));
-    P = mmd(t, Um);
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) Q.m[i][j] = Q.m[i][j] + P.m[i][j];
-    // F = -(i/8) (Q - Q^+)
-    M3 F;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            cx<double> d = Q.m[i][j] - cj(Q.m[j][i]);
-            F.m[i][j] = mk(d.i * 0.125, -d.r * 0.125);
+            for (int k = 0; k < 9; ++k) other[k][lane] = make_double2(Q.m[k / 3][k % 3].r, Q.m[k / 3][k % 3].i);
         }
-    return F;
+    }
+    __syncthreads();
+    if (half || s >= V) return;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const double2 o = other[k][lane];
+        Q.m[k / 3][k % 3] = Q.m[k / 3][k % 3] + mk(o.x, o.y);
+    }
+    // F = -(i/8) (Q - Q^+)
+    auto f = [&](int i, int j) {
+        const cx<double> d = Q.m[i][j] - cj(Q.m[j][i]);
+        return make_double2(d.i * 0.125, -d.r * 0.125);
+    };
+    F[s] = make_double2(f(0, 0).x, f(1, 1).x);
+    F[(size_t)V + s] = make_double2(f(2, 2).x, 0.0);
+    F[(size_t)2 * V + s] = f(0, 1);
+    F[(size_t)3 * V + s] = f(0, 2);
+    F[(size_t)4 * V + s] = f(1, 2);
+}
+
+__device__ __forceinline__ M3 load_F(const double2* __restrict__ F, int plane, int V, int s) {
+    const double2* q = F + (size_t)5 * plane * V + s;
+    const double2 d = q[0], e = q[V], a = q[(size_t)2 * V], b = q[(size_t)3 * V], c = q[(size_t)4 * V];
+    M3 r;
+    r.m[0][0] = mk(d.x, 0.0);
+    r.m[1][1] = mk(d.y, 0.0);
+    r.m[2][2] = mk(e.x, 0.0);
+    r.m[0][1] = mk(a.x, a.y);
+    r.m[0][2] = mk(b.x, b.y);
+    r.m[1][2] = mk(c.x, c.y);
+    r.m[1][0] = cj(r.m[0][1]);
+    r.m[2][0] = cj(r.m[0][2]);
+    r.m[2][1] = cj(r.m[1][2]);
+    return r;
 }
 
 __global__ void k_gauge_convert(const double2* __restrict__ Uin, double2* __restrict__ U64,
@@ -196,28 +245,15 @@ __device__ __forceinline__ cx<double> chiral_elem(const M3& G1, const M3& G2, co
 }
 
 // The FP32 copy holds the same 72 reals of a site side by side.
-__global__ void k_clover_build(const double2* __restrict__ U, double2* __restrict__ C64,
-                               float* __restrict__ C32, Geo g, int V, double csw) {
+// C64 holds the six planes' F (5 slots each) on entry and is overwritten site by site.
+__global__ void __launch_bounds__(64) k_clover_build(double2* __restrict__ C64, float* __restrict__ C32, int V,
+                                                     double csw) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= V) return;
-    int c[4];
-    {
-        int r = s;
-        c[0] = r % g.L[0];
-        r /= g.L[0];
-        c[1] = r % g.L[1];
-        r /= g.L[1];
-        c[2] = r % g.L[2];
-        c[3] = r / g.L[2];
-    }
     // F indices: 0=x,1=y,2=z,3=t.  Paper F_23 = F(1,2), F_14 = F(0,3), F_31 = F(2,0),
     // F_24 = F(1,3), F_12 = F(0,1), F_34 = F(2,3).
-    const M3 F12 = field_strength(U, g, c, s, V, 0, 1);
-    const M3 F23 = field_strength(U, g, c, s, V, 1, 2);
-    const M3 F31 = field_strength(U, g, c, s, V, 2, 0);
-    const M3 F14 = field_strength(U, g, c, s, V, 0, 3);
-    const M3 F24 = field_strength(U, g, c, s, V, 1, 3);
-    const M3 F34 = field_strength(U, g, c, s, V, 2, 3);
+    const M3 F12 = load_F(C64, 0, V, s), F23 = load_F(C64, 1, V, s), F31 = load_F(C64, 2, V, s);
+    const M3 F14 = load_F(C64, 3, V, s), F24 = load_F(C64, 4, V, s), F34 = load_F(C64, 5, V, s);
     double out[72];
     const double h = 0.5 * csw;
 #pragma unroll
@@ -250,7 +286,7 @@ __global__ void k_clover_build(const double2* __restrict__ U, double2* __restric
     float4* cc = reinterpret_cast<float4*>(C32 + (size_t)s * BK_CLOVC);
 #pragma unroll
     for (int q = 0; q < 18; ++q)
-        cc[q] = make_float4((float)out[4 * q], (float)out[4 * q + 1], (float)out[4 * q + 2], (float)out[4 * q + 3]);
+        cc[q] = make_float4(d2f(out[4 * q]), d2f(out[4 * q + 1]), d2f(out[4 * q + 2]), d2f(out[4 * q + 3]));
 }
 
 // ---------------------------------------------------------------- clover inverse
@@ -356,7 +392,7 @@ __global__ void k_clover_inverse(const double2* __restrict__ C64, double kappa, 
     float4* cc = reinterpret_cast<float4*>(Ci32 + (size_t)s * BK_CLOVC);
 #pragma unroll
     for (int q = 0; q < 18; ++q)
-        cc[q] = make_float4((float)out[4 * q], (float)out[4 * q + 1], (float)out[4 * q + 2], (float)out[4 * q + 3]);
+        cc[q] = make_float4(d2f(out[4 * q]), d2f(out[4 * q + 1]), d2f(out[4 * q + 2]), d2f(out[4 * q + 3]));
     // non-negative doubles order like their bit patterns
     atomicMax(bound, (unsigned long long)__double_as_longlong(nmax));
     if (singular) atomicAdd(bound + 1, 1ull);
@@ -381,7 +417,18 @@ bk_status launch_clover_build(const double2* U64, double2* C64, float* C32, cons
         stride *= dims[mu];
     }
     const int V = stride;
-    k_clover_build<<<(V + 63) / 64, 64, 0, st>>>(U64, C64, C32, g, V, csw);
+    // The planes one after the other: M and N in C32's memory (288 bytes a site,
+    // as many), F in C64's; then the site terms over both.
+    const int plane[6][2] = {{0, 1}, {1, 2}, {2, 0}, {0, 3}, {1, 3}, {2, 3}};
+    double2* MN = reinterpret_cast<double2*>(C32);
+    static_assert(BK_CLOVC * sizeof(float) == 18 * sizeof(double2), "M and N fill the FP32 table");
+    for (int p = 0; p < 6; ++p) {
+        const int mu = plane[p][0], nu = plane[p][1];
+        k_corner<<<dim3((V + 63) / 64, 2), 64, 0, st>>>(U64, MN, g, V, mu, nu);
+        k_leaves<<<(V + 31) / 32, 64, 0, st>>>(U64, MN, C64 + (size_t)5 * p * V, g, V, mu, nu);
+        BK_CUDA_TRY(cudaGetLastError());
+    }
+    k_clover_build<<<(V + 63) / 64, 64, 0, st>>>(C64, C32, V, csw);
     BK_CUDA_TRY(cudaGetLastError());
     return BK_OK;
 }

@@ -425,15 +425,25 @@ __global__ void __launch_bounds__(GW * 32, MINB) k_update_r(const __grid_constan
         }
     }
     if (g.ynorm) {
+        // rows of a column pair: first within each warp, then over the warps (an
+        // FP64 add of one warp takes 64 cycles, so few of them in a row)
         ynred[w][lane] = make_double2(yn0 + f2d(sa), yn1 + f2d(sb));
+        __syncwarp();
+        if (lane < tnp) {
+            double2 v = ynred[w][lane];
+            for (int sub = 1; sub < spw; ++sub) {
+                v.x += ynred[w][sub * tnp + lane].x;
+                v.y += ynred[w][sub * tnp + lane].y;
+            }
+            ynred[w][lane] = v;
+        }
         __syncthreads();
         if (act && threadIdx.x < tnp) {
-            double2 v = make_double2(0.0, 0.0);
-            for (int ww = 0; ww < GW; ++ww)
-                for (int sub = 0; sub < spw; ++sub) {
-                    v.x += ynred[ww][sub * tnp + lane].x;
-                    v.y += ynred[ww][sub * tnp + lane].y;
-                }
+            double2 v = ynred[0][lane];
+            for (int ww = 1; ww < GW; ++ww) {
+                v.x += ynred[ww][lane].x;
+                v.y += ynred[ww][lane].y;
+            }
             g.ynorm[(size_t)chunk * ncols + 2 * L.q] = v.x;
             g.ynorm[(size_t)chunk * ncols + 2 * L.q + 1] = v.y;
         }
