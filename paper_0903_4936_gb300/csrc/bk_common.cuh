@@ -162,7 +162,8 @@ __host__ inline Field field_pairs(Field f, int p0, int prec) {
 // like an FP64 operation (64 cycles of a scheduler per warp), which made the
 // casts and the coefficient loads of the FP32 kernels wait for it.  For zero
 // and normal numbers that stay normal the same bits come from a few integer
-// instructions; everything else takes the instruction.
+// instructions; everything else takes the instruction (volatile, so that the
+// compiler does not convert every number both ways and select).
 
 // round to nearest even, as (float)x
 __device__ __forceinline__ float d2f(double x) {
@@ -176,7 +177,9 @@ __device__ __forceinline__ float d2f(double x) {
         return __uint_as_float(f | (hi & 0x80000000u));
     }
     if (((hi << 1) | lo) == 0u) return __uint_as_float(hi);  // +-0
-    return __double2float_rn(x);
+    float r;
+    asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(r) : "d"(x));
+    return r;
 }
 // exact, as (double)x
 __device__ __forceinline__ double f2d(float x) {
@@ -184,7 +187,9 @@ __device__ __forceinline__ double f2d(float x) {
     if (ex - 1u < 254u)
         return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
     if ((b << 1) == 0u) return __hiloint2double((int)b, 0);
-    return (double)x;
+    double r;
+    asm volatile("cvt.f64.f32 %0, %1;" : "=d"(r) : "f"(x));
+    return r;
 }
 __device__ __forceinline__ double f2d(double x) { return x; }
 __device__ __forceinline__ float2 d2f(double2 v) { return make_float2(d2f(v.x), d2f(v.y)); }

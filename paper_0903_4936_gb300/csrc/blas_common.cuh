@@ -144,17 +144,26 @@ __device__ __forceinline__ void store_at(const Field& f, size_t e, typename Prec
     }
 }
 
+__device__ __forceinline__ float flip_sign(float v) { return __int_as_float(__float_as_int(v) ^ 0x80000000); }
+__device__ __forceinline__ double flip_sign(double v) {
+    return __hiloint2double(__double2hiint(v) ^ 0x80000000, __double2loint(v));
+}
+// (a call: general factors are rare, and FP64 arithmetic on either side of a
+// select would be paid for by every FP32 kernel)
+static __device__ __noinline__ void scale2(double& re, double& im, double mult) {
+    re *= mult;
+    im *= mult;
+}
+
 // complex coefficient mult * (ptr ? ptr[s] : 1); unit: 1 or -1 when mult is that
 template <int P>
 __device__ __forceinline__ cx<typename Prec<P>::real> coef(const double* ptr, double mult, int unit, int s) {
     using R = typename Prec<P>::real;
     if (!ptr) return mk(d2r<R>(mult), R(0));
     double re = __ldg(ptr + 2 * s), im = __ldg(ptr + 2 * s + 1);
-    if (unit == 0) {
-        re *= mult;
-        im *= mult;
-    }
-    return unit < 0 ? mk(d2r<R>(-re), d2r<R>(-im)) : mk(d2r<R>(re), d2r<R>(im));
+    if (unit == 0) scale2(re, im, mult);
+    R r = d2r<R>(re), i = d2r<R>(im);
+    return unit < 0 ? mk(flip_sign(r), flip_sign(i)) : mk(r, i);
 }
 
 // FP32 products are summed in FP32 over at most this many (site, component)

@@ -249,6 +249,20 @@ bk_status rows_gram_p(Field A, Field B, Field B2, int NB, const SysPart& p, doub
 // Unit coefficients cost nothing (FP64 instructions are what bounds the FP64
 // updates of wide systems; memory bounds the FP32 ones).
 
+// (a call, so that the kernels that need no FP64 arithmetic do none)
+__device__ __noinline__ void scale_coefs(const GenOp& g, int s, cx<double>& m0, cx<double>& m1) {
+    const cx<double> f = coef<BK_FP64>(g.ma[0], g.ma_mult[0], g.ma_unit[0], s);
+    m0 = f * m0;
+    m1 = f * m1;
+}
+// sign flipped by its bit
+__device__ __forceinline__ float flip(float v, bool neg) {
+    return __int_as_float(__float_as_int(v) ^ (neg ? 0x80000000 : 0));
+}
+__device__ __forceinline__ double flip(double v, bool neg) {
+    return __hiloint2double(__double2hiint(v) ^ (neg ? 0x80000000 : 0), __double2loint(v));
+}
+
 template <int P, int MAXL, int UR, int MINB, int NMI, int NE, int HX>
 __global__ void __launch_bounds__(GW * 32, MINB) k_update_r(const __grid_constant__ GenOp g,
                                                             const __grid_constant__ PTiles wt, unsigned rows,
@@ -288,27 +302,25 @@ __global__ void __launch_bounds__(GW * 32, MINB) k_update_r(const __grid_constan
     {
         const double2* M = reinterpret_cast<const double2*>(g.M) + (act && mat ? g.p.coef_off[s] : 0);
         const bool j1ok = L.i0 + 1 < L.Ls;
-        // one operand: its coefficient goes into M (a real one as a factor, +-1 without arithmetic)
-        const bool fold = nmi == 1 && mat, fcx = fold && g.ma[0] != nullptr;
-        const double fr = fold ? g.ma_mult[0] : 1.0;
-        const cx<double> f = fcx ? coef<BK_FP64>(g.ma[0], g.ma_mult[0], g.ma_unit[0], s) : mk(fr, 0.0);
-        auto times_f = [&](double2 a) {
-            if (fcx) return f * mk(a.x, a.y);
-            if (!fold || g.ma_unit[0] == 1) return mk(a.x, a.y);
-            if (g.ma_unit[0] == -1) return mk(-a.x, -a.y);
-            return mk(fr * a.x, fr * a.y);
-        };
+        // one operand: its coefficient goes into M; 1 and -1 without FP64 arithmetic
+        const int unit = nmi != 1 || !mat ? 1 : (g.ma[0] ? 0 : g.ma_unit[0]);
+        const bool neg = unit < 0;
 #pragma unroll
         for (int i = 0; i < MAXL; ++i) {
             cx<double> m0 = mk(0.0, 0.0), m1 = mk(0.0, 0.0);
             if (act && mat && i < L.Ls) {
-                m0 = times_f(__ldg(M + i * L.Ls + L.i0));
-                if (j1ok) m1 = times_f(__ldg(M + i * L.Ls + L.i0 + 1));
+                const double2 a = __ldg(M + i * L.Ls + L.i0);
+                m0 = mk(a.x, a.y);
+                if (j1ok) {
+                    const double2 b = __ldg(M + i * L.Ls + L.i0 + 1);
+                    m1 = mk(b.x, b.y);
+                }
+                if (unit == 0) scale_coefs(g, s, m0, m1);
             }
-            Mr[i].x = d2r<R>(m0.r);
-            Mr[i].y = d2r<R>(m1.r);
-            Mi[i].x = d2r<R>(m0.i);
-            Mi[i].y = d2r<R>(m1.i);
+            Mr[i].x = flip(d2r<R>(m0.r), neg);
+            Mr[i].y = flip(d2r<R>(m1.r), neg);
+            Mi[i].x = flip(d2r<R>(m0.i), neg);
+            Mi[i].y = flip(d2r<R>(m1.i), neg);
         }
     }
     const bool yunit = g.y_unit == 1, xunit = g.x_unit == 1;
