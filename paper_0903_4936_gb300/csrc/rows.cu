@@ -225,7 +225,9 @@ bk_status rows_gram_p(Field A, Field B, Field B2, int NB, const SysPart& p, doub
     const int maxL = max_active_L(p);
     const int ne = p.coef_off[p.nsys];
     constexpr int UR = P == BK_FP64 ? 2 : 4;
-    if (NB == 2 && maxL <= 6) return run_gram_r<P, 2, 6, UR>(A, B, B2, p, wt, part, nchunk, V, st);
+    // two operands: 3 row groups (16^3x32 even sites, 60 columns: 4 groups spill 74 bytes and take 320 us, 3 take
+    // 238, 2 take 260; the three blocks once are 167 us of memory time)
+    if (NB == 2 && maxL <= 6) return run_gram_r<P, 2, 6, P == BK_FP64 ? 2 : 3>(A, B, B2, p, wt, part, nchunk, V, st);
     for (int b = 0; b < NB; ++b) {
         Field Bb = b == 0 ? B : B2;
         double2* pb = part + (size_t)b * nchunk * ne;
