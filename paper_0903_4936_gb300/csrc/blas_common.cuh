@@ -49,6 +49,24 @@ inline PTiles make_ptiles(const SysPart& p, int maxp) {
     }
     return t;
 }
+// Neighbouring tiles joined over the inactive systems between them (the
+// kernel skips their lanes), where the wider tile takes no more warp steps per
+// row (1 / floor(32 / pairs)) than the two.
+inline PTiles join_ptiles(const PTiles& a, int maxp) {
+    auto steps = [](int pairs) { return 1.0 / std::max(1, 32 / pairs); };
+    PTiles t;
+    t.n = 0;
+    for (int i = 0; i < a.n; ++i) {
+        const int l = t.n - 1, wide = t.n ? a.p0[i] + a.np[i] - t.p0[l] : 0;
+        if (t.n && wide <= maxp && steps(wide) <= steps(t.np[l]) + steps(a.np[i]) + 1e-9) {
+            t.np[l] = wide;
+        } else {
+            t.p0[t.n] = a.p0[i];
+            t.np[t.n++] = a.np[i];
+        }
+    }
+    return t;
+}
 
 inline int max_active_L(const SysPart& p) {
     int m = 0;

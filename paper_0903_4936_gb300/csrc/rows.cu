@@ -21,9 +21,9 @@ constexpr int GW = 8;  // warps per block
 
 // Consecutive row groups a warp takes at a time: up to 12 (a site's rows when
 // one row fills the warp), so that the lines its rows share and their DRAM
-// pages are used together (16^3x32, 60 columns, even sites, X and R update: 494
-// us with single rows strided over the grid, 340 with whole sites); fewer where
-// the groups do not go round.
+// pages are used together (16^3x32, 60 columns, even sites, X and R update: 489
+// us with single rows strided over the grid, 470 in runs, both with narrow
+// tiles); fewer where the groups do not go round.
 __device__ __forceinline__ unsigned row_run(unsigned units, unsigned warps) {
     return min(12u, max(1u, units / warps));
 }
@@ -41,9 +41,9 @@ struct RLane {
 __device__ __forceinline__ RLane rlane(const SysPart& p, int tp0, int tnp, int lane) {
     RLane w;
     w.sub = lane / tnp;
-    w.live = w.sub < 32 / tnp;
     w.q = tp0 + lane - w.sub * tnp;
     w.s = sys_of_pair(p, w.q);
+    w.live = w.sub < 32 / tnp && ((p.active >> w.s) & 1ull);
     w.Ls = p.L[w.s];
     w.i0 = 2 * w.q - p.col0[w.s];
     w.nps = (w.Ls + 1) / 2;
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(GW * 32, P == BK_FP64 ? 1 : 2) k_gram_r(Field 
     for (int x = threadIdx.x; x < tnp * NACC; x += GW * 32) {
         const int e = x / tnp, pr = x - e * tnp, j = e % MAXL, ii = (e / MAXL) & 1, b = e / (2 * MAXL);
         const int s = sys_of_pair(p, tp0 + pr), Ls = p.L[s], i = 2 * (tp0 + pr) - p.col0[s] + ii;
-        if (i >= Ls || j >= Ls) continue;
+        if (i >= Ls || j >= Ls || !((p.active >> s) & 1ull)) continue;
         double2 v = make_double2(0.0, 0.0);
         for (int ww = 0; ww < nact; ++ww)
             for (int sub = 0; sub < nsub; ++sub) {
@@ -466,18 +466,20 @@ __global__ void __launch_bounds__(GW * 32, MINB) k_update_r(const __grid_constan
 
 }  // namespace
 
-// Tiles of the row kernels: runs of whole active systems.  FP32 / FP16: the
-// widest that fit a warp, since memory bounds them and a narrow tile reads
-// scattered pieces of the rows (10 systems of 6, 6 and 2 columns, X and R
-// update: six tiles of 5 pairs 594 us, one of 30 pairs 380).  FP64: the width
+// Tiles of the row kernels: runs of whole systems, with inactive ones between
+// active ones where that saves a tile.  FP32 / FP16: the widest that fit a
+// warp, since memory bounds them and a narrow tile reads scattered pieces of
+// the rows (16^3x32 even sites, ten systems of 6 columns, X and R update: six
+// tiles of 5 pairs 594 us, one of 30 pairs 350; with one system in the middle
+// inactive, two tiles 600 us, one over the gap 357).  FP64: the width
 // that keeps the most lanes busy (a tile of tnp pairs costs 1 / floor(32 /
 // tnp) of a warp step per row; the widest of the cheapest splittings).
 PTiles row_tiles(int prec, const SysPart& p) {
-    PTiles best = make_ptiles(p, 32);
+    PTiles best = join_ptiles(make_ptiles(p, 32), 32);
     if (prec != BK_FP64) return best;
     double cost = 1e30;
     for (int maxp = 32; maxp >= ROWS_MAXL / 2; --maxp) {
-        const PTiles t = make_ptiles(p, maxp);
+        const PTiles t = join_ptiles(make_ptiles(p, maxp), maxp);
         double c = 0.0;
         for (int i = 0; i < t.n; ++i) c += 1.0 / (32 / t.np[i]);
         if (c < cost - 1e-9) {

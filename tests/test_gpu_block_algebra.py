@@ -76,3 +76,27 @@ def test_fp64_operator_split_over_warps(dims, L):
     kap = np.linspace(0.11, 0.13, L)
     Y = lat.dslash(torch.from_numpy(X).cuda(), list(kap), "fp64").cpu().numpy()
     assert _rel(Y, dirac.apply_dirac(U, X, kap, 1.0)) < 1e-13
+
+
+@pytest.mark.parametrize("prec,Ls", [("fp64", (3, 2, 4)), ("fp64", (6, 20, 5)), ("fp64", (12, 12, 12)),
+                                     ("fp64", (30, 24, 6)), ("fp32", (3, 2, 4)), ("fp32", (6, 6, 6)),
+                                     ("fp32", (2, 12, 2))])
+def test_systems_around_a_converged_one(prec, Ls):
+    """The middle system (small kappa) converges first; the others go on with its columns between theirs."""
+    dims = (4, 4, 4, 4)
+    lat, U = _lat(dims, 11)
+    B = synth.z4_noise(dims, sum(Ls), 33)
+    kappas = [0.12, 0.03, 0.12]
+    X, infos = lat.block_solve_batched(torch.from_numpy(B).cuda(), kappas, list(Ls), method="bicgstab", prec=prec,
+                                       tol=1e-10, maxiter=500, delta=0.0 if prec == "fp64" else 0.03)
+    assert all(i["converged"] == 1 for i in infos)
+    assert infos[1]["iterations"] < min(infos[0]["iterations"], infos[2]["iterations"])
+    got = dense.to_columns(X.cpu().numpy())
+    rhs = dense.to_columns(B)
+    c = 0
+    for kappa, L in zip(kappas, Ls):
+        ref = np.linalg.solve(dense.dense_matrix(U, kappa, 1.0), rhs[:, c:c + L])
+        # ||x - x*|| <= ||D^-1|| ||r||, ||D^-1|| < 20 at these kappas
+        err = np.linalg.norm(got[:, c:c + L] - ref, axis=0) / np.linalg.norm(rhs[:, c:c + L], axis=0)
+        assert np.max(err) < 2e-9
+        c += L
