@@ -615,26 +615,46 @@ __global__ void __launch_bounds__(FIN_E * FIN_ROWS) k_norm_finish(const double* 
     }
 }
 
-// X64 += Xlo; Xlo = 0 over pairs [p0, p0 + np)
-// (sub: -=) over pairs [p0, p0 + np); zero_lo: then Xlo = 0
-__global__ void k_accum(Field x64, Field xlo, int p0, int np, int sub, int zero_lo) {
-    const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= (long long)x64.V * np) return;
-    const int n = (int)(g / np), q = p0 + (int)(g - (long long)(g / np) * np);
-    double2 xr[12], xi[12];
-    float2 lr[12], li[12];
-    load_pair<BK_FP64>(x64, n, q, xr, xi);
-    load_pair<BK_FP32>(xlo, n, q, lr, li);
+// Sums into FP64 by element: a block takes rpb consecutive rows (site,
+// component) of np pairs, a thread EL_U of their elements, all loaded before
+// the first store.  Memory bounds it.  A thread per (site, pair), holding 12
+// components 12 rows apart, kept too few loads in flight (16^3x32 even sites,
+// all 60 columns: 704 us, now 528; 6 of 60, where each row's piece is half a
+// line: 93, now 83).
+constexpr int EL_U = 4, EL_THREADS = 256;
+inline unsigned rows_per_block(unsigned rows, int np) {
+    return std::max(1u, std::min(EL_U * EL_THREADS / (unsigned)np, rows / 304));
+}
+
+// X64 += Xlo (sub: -=) over pairs [p0, p0 + np); zero_lo: then Xlo = 0
+__global__ void __launch_bounds__(EL_THREADS) k_accum(Field x64, Field xlo, int p0, int np, int sub, int zero_lo,
+                                                      unsigned rows, unsigned rpb) {
+    const unsigned r0 = blockIdx.x * rpb, items = min(rpb, rows - r0) * np;
+    for (unsigned i0 = threadIdx.x; i0 < items; i0 += EL_U * EL_THREADS) {
+        CxPair<double2> x[EL_U];
+        CxPair<float2> l[EL_U];
+        size_t row[EL_U];
+        int q[EL_U];
 #pragma unroll
-    for (int k = 0; k < 12; ++k) {
-        const double2 r = f2d(lr[k]), i = f2d(li[k]);
-        xr[k] = sub ? psub(xr[k], r) : padd(xr[k], r);
-        xi[k] = sub ? psub(xi[k], i) : padd(xi[k], i);
-        lr[k] = make_float2(0.f, 0.f);
-        li[k] = make_float2(0.f, 0.f);
+        for (int u = 0; u < EL_U; ++u) {
+            const unsigned i = i0 + u * EL_THREADS, r = i / np;
+            row[u] = r0 + r;
+            q[u] = p0 + (int)(i - r * np);
+            if (i < items) {
+                x[u] = load_at<BK_FP64>(x64, row[u] * x64.np + q[u]);
+                l[u] = load_at<BK_FP32>(xlo, row[u] * xlo.np + q[u]);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < EL_U; ++u) {
+            if (i0 + u * EL_THREADS >= items) break;
+            const double2 r = f2d(l[u].re), i = f2d(l[u].im);
+            store_at<BK_FP64>(x64, row[u] * x64.np + q[u], sub ? psub(x[u].re, r) : padd(x[u].re, r),
+                              sub ? psub(x[u].im, i) : padd(x[u].im, i));
+            if (zero_lo)
+                store_at<BK_FP32>(xlo, row[u] * xlo.np + q[u], make_float2(0.f, 0.f), make_float2(0.f, 0.f));
+        }
     }
-    store_pair<BK_FP64>(x64, n, q, xr, xi);
-    if (zero_lo) store_pair<BK_FP32>(xlo, n, q, lr, li);
 }
 
 // Seeded Gaussian block: SplitMix64 of (seed, canonical index), Box-Muller.
@@ -1149,20 +1169,22 @@ bk_status launch_xmy(int prec, Field X, const double* M, const double* c_dev, Fi
     return launch_genop(prec, g, V, st);
 }
 
-bk_status launch_accum(Field X64, Field Xlo, int p0, int np, cudaStream_t st) {
+namespace {
+bk_status accum(Field X64, Field Xlo, int p0, int np, int sub, int zero_lo, cudaStream_t st) {
     if (np <= 0) return BK_OK;
-    const long long items = (long long)X64.V * np;
-    k_accum<<<(unsigned)((items + 127) / 128), 128, 0, st>>>(X64, Xlo, p0, np, 0, 1);
+    const unsigned rows = 12u * (unsigned)X64.V, rpb = rows_per_block(rows, np);
+    k_accum<<<(rows + rpb - 1) / rpb, EL_THREADS, 0, st>>>(X64, Xlo, p0, np, sub, zero_lo, rows, rpb);
     BK_CUDA_TRY(cudaGetLastError());
     return BK_OK;
 }
+}  // namespace
+
+bk_status launch_accum(Field X64, Field Xlo, int p0, int np, cudaStream_t st) {
+    return accum(X64, Xlo, p0, np, 0, 1, st);
+}
 
 bk_status launch_sub_lo(Field X64, Field Ylo, int p0, int np, cudaStream_t st) {
-    if (np <= 0) return BK_OK;
-    const long long items = (long long)X64.V * np;
-    k_accum<<<(unsigned)((items + 127) / 128), 128, 0, st>>>(X64, Ylo, p0, np, 1, 0);
-    BK_CUDA_TRY(cudaGetLastError());
-    return BK_OK;
+    return accum(X64, Ylo, p0, np, 1, 0, st);
 }
 
 bk_status launch_random(int prec, Field f, int L, uint64_t seed, cudaStream_t st) {
