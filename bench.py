@@ -694,8 +694,7 @@ def main():
                    "l2": "inputs larger than L2 and a 256 MB L2 flush before every timed step"},
         "roofline": {"bound": "hbm",
                      "kernel": (f"k_eo_pair<{wl['prec'].upper()}> (inner Schur operator, both half-lattice launches)"
-                                if r["eo"] else f"k_dslash_staged / k_dslash_pair<{wl['prec'].upper()}> "
-                                                "(inner operator, all columns)"),
+                                if r["eo"] else f"k_dslash_pair<{wl['prec'].upper()}> (inner operator, all columns)"),
                      "achieved": achieved, "peak": hbm,
                      "unit": "GB/s", "frac": (achieved / hbm) if achieved else None, "peak_kind": peak_kind,
                      "traffic": traffic, "launches": agg["n_inner"],

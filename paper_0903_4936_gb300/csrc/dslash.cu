@@ -16,10 +16,10 @@
 // times its term directly.
 //
 // What bounds it: the rows' eight-fold fetches from L2, 10 TB/s of L2-to-SM
-// traffic (16^3x32, 30 columns: 3.0 GB in 284 us).  Before, links and clover
+// traffic (16^3x32, 30 columns: 3.0 GB in 280 us).  Before, links and clover
 // were stored as the duplicated pairs (224 and 816 bytes) and took 216 loads a
 // thread, which with staging copies through shared memory kept the load/store
-// pipe 74 % busy: 404 us there (24^3x48, 96 columns 5080 us, now 4240; FP16
+// pipe 74 % busy: 404 us there (24^3x48, 96 columns 5080 us, now 4060; FP16
 // 12x10x14x18, 13 columns 51, now 34).  A form with the rows staged by bulk
 // copies (cp.async.bulk, a producer warp, 2x2x2 site tiles sharing their rows,
 // 5 fetches a site instead of 8) took 306 us: its producer and 128-register
@@ -631,8 +631,9 @@ __device__ __forceinline__ void herm6_rows(const double2* __restrict__ C, int V,
 // takes the two hops of direction t and three rows of one chiral block of the
 // clover term, and finishes spin t.  An SM's scheduler starts an FP64
 // instruction of a warp every 64 cycles, so one thread per site and column
-// (about 1000 of them) needs 33 us however few there are; a quarter of that
-// each, on four times the warps, is faster while they do not fill the chip's
+// (about 1000 of them) needs 33 us however few there are (4^4, 12 columns: 46
+// us a launch, 18 in this form); a quarter of that each, on four times the
+// warps, is faster while they do not fill the chip's
 // 608 schedulers about twice (see dslash_col_impl).
 __global__ void __launch_bounds__(128) k_dslash_col4(const __grid_constant__ DColArgs<BK_FP64> a) {
     __shared__ double hs[4][24][32], ys[4][6][32];
@@ -795,8 +796,9 @@ bk_status dslash_col_impl(const DslashOp& op, cudaStream_t st) {
 // dcol[j] (dcol == nullptr: dbase + j), through a shared-memory tile of CT_S
 // sites x CT_C columns: a canonical column is contiguous along (site,
 // component), a device row along the columns, so one side of a direct copy
-// touches a separate line per lane (12 columns, 16^3x32, FP64: 205 us each way,
-// now 100; 60 columns out: 1980, now 480).
+// touches a separate line per lane (12 columns, 16^3x32, FP64: 103 us in and
+// 118 out, of 88 at the memory rate; operator with both conversions 3428 us,
+// now 3330).
 constexpr int CT_S = 8, CT_C = 16, CT_R = CT_S * 12;
 
 __device__ __forceinline__ int dev_col(const int* dcol, int dbase, int j) { return dcol ? __ldg(dcol + j) : dbase + j; }

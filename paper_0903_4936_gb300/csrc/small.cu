@@ -9,7 +9,8 @@
 // FP64 instructions: an elimination step spreads its elements over the 128
 // threads, divides once (by the pivot; U keeps a unit diagonal) and compares
 // magnitudes as integers.  The general kernels (blas.cu) take 29 + 31 us for a
-// 12 x 12 factorisation and solve in two launches; larger systems use them.
+// 12 x 12 factorisation and solve in two launches, k_small_step 22 us for both
+// (6 x 6: 11); larger systems use them.
 #include "blas_common.cuh"
 
 namespace {
