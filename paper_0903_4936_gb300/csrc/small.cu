@@ -264,6 +264,7 @@ __global__ void __launch_bounds__(NT) k_small_chol(const double2* __restrict__ S
         if (b > 0) dm = max(dm, (u64)b);
     }
     const double dmin = 1e-14 * __longlong_as_double((long long)dm);
+    __syncthreads();  // every thread has the diagonal before a step changes it
     bool bad = false;
     for (int k = 0; k < n; ++k) {
         const double d = A[k][k].r;

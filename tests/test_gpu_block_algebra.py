@@ -100,3 +100,30 @@ def test_systems_around_a_converged_one(prec, Ls):
         err = np.linalg.norm(got[:, c:c + L] - ref, axis=0) / np.linalg.norm(rhs[:, c:c + L], axis=0)
         assert np.max(err) < 2e-9
         c += L
+
+
+@pytest.mark.parametrize("L", [5, 6, 7, 12])
+@pytest.mark.parametrize("eps", [0.0, 1e-5, 1e-3])
+def test_cholesky_basis_of_nearly_dependent_columns(L, eps):
+    """P^H P is singular or nearly so when two sources differ by eps times noise: the basis is then left alone (the
+    L x L system of equal columns breaks down) or changed to an orthonormal one, the same in every run, bit for bit."""
+    dims = (4, 4, 4, 4)
+    lat, U = _lat(dims, 13)
+    B = synth.gaussian_sources(dims, L, 51)
+    B[L - 1] = B[1] + eps * synth.gaussian_sources(dims, 1, 52)[0]
+    Bt = torch.from_numpy(B).cuda()
+    runs = [lat.block_solve(Bt, 0.12, method="bicgstab", prec="fp64", tol=1e-10, maxiter=300, orth=True,
+                            raise_on_fail=False) for _ in range(3)]
+    X, info = runs[0]
+    for Y, other in runs[1:]:
+        assert other["iterations"] == info["iterations"] and torch.equal(torch.view_as_real(X), torch.view_as_real(Y))
+    if eps == 0.0:
+        assert info["breakdown"] == 1
+        return
+    assert info["converged"] == 1
+    ref = np.linalg.solve(dense.dense_matrix(U, 0.12, 1.0), dense.to_columns(B))
+    got = dense.to_columns(X.cpu().numpy())
+    # ||x - x*|| <= ||D^-1|| ||r||, ||D^-1|| < 20 at this kappa; the recursive residual of a basis of condition
+    # 1 / eps may differ from the true one by rounding times that
+    assert np.max(np.linalg.norm(got - ref, axis=0) / np.linalg.norm(dense.to_columns(B), axis=0)) < 20 * (
+        1e-10 + 1e-13 / eps)
