@@ -127,3 +127,26 @@ def test_cholesky_basis_of_nearly_dependent_columns(L, eps):
     # 1 / eps may differ from the true one by rounding times that
     assert np.max(np.linalg.norm(got - ref, axis=0) / np.linalg.norm(dense.to_columns(B), axis=0)) < 20 * (
         1e-10 + 1e-13 / eps)
+
+
+@pytest.mark.parametrize("L", [889, 1000, 1024])
+def test_gram_of_the_widest_blocks(L):
+    """FP32 Gram matrices up to the width (1024) at which 256 threads a block fill the work list."""
+    dims = (2, 2, 2, 2)
+    lat, _ = _lat(dims)
+    A, B = (synth.gaussian_sources(dims, L, s) for s in (61, 62))
+    G = lat.gram(lat.pack(torch.from_numpy(A).cuda(), "fp32"), lat.pack(torch.from_numpy(B).cuda(), "fp32"), L,
+                 "fp32").cpu().numpy()
+    assert _rel(G, A.reshape(L, -1).conj() @ B.reshape(L, -1).T) < GRAM_TOL["fp32"]
+
+
+@pytest.mark.parametrize("nsys,L", [(64, 112), (48, 122), (64, 128)])
+def test_many_wide_systems(nsys, L):
+    """Partitions whose Gram matrices fill the work list are accepted: one iteration of each system."""
+    dims = (2, 2, 2, 2)
+    lat, _ = _lat(dims)
+    B = torch.from_numpy(synth.gaussian_sources(dims, L, 63)).cuda().repeat(nsys, 1, 1, 1, 1, 1, 1)
+    _, infos = lat.block_solve_batched(B, [0.1] * nsys, [L] * nsys, method="bicgstab", prec="fp64", tol=1e-10,
+                                       maxiter=1, raise_on_fail=False)
+    assert infos[0]["status"] == "BK_ERR_NOT_CONVERGED"
+    assert all(i["iterations"] == 1 and np.isfinite(i["rec_res_max"]) for i in infos)
