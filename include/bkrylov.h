@@ -287,7 +287,9 @@ typedef struct bk_solve_params {
                               P^H P = T^H T (Cholesky, FP64) before every
                               V = A P; the iterates are unchanged in exact
                               arithmetic and R~_0^H V stays well
-                              conditioned in low precision                */
+                              conditioned in low precision.  FP32/FP16
+                              blocks: pivots below 2e-7 L of their diagonal
+                              entry, which are rounding, count as that    */
     int record_history;    /* 1: info->history[k] = max_i rel. residual       */
     int timing;            /* 1: time every dslash launch with CUDA events    */
     int update_prec;       /* mixed precision: arithmetic of the residual

@@ -1399,7 +1399,9 @@ struct Solve {
     bk_status cholesky_basis() {
         BK_TRY(gram(Pb, Pb, G_Z));
         launches += 1;
-        BK_TRY(small_systems() ? launch_small_chol(G_Z, gam, part, st) : launch_chol_inv(G_Z, gam, part, st));
+        const double floor = P == BK_FP64 ? 0.0 : CHOL_FLOOR32;
+        BK_TRY(small_systems() ? launch_small_chol(G_Z, gam, part, floor, st)
+                               : launch_chol_inv(G_Z, gam, part, st, 0.0, floor));
         GenOp g = genop0();
         g.nmi = 1;
         g.Mi[0] = Pb;

@@ -180,9 +180,24 @@ bk_status launch_lu_factor(const double* G, double* LU, int* piv, int* info, con
 bk_status launch_lu_solve(const double* LU, const int* piv, const double* H, const double* scale_dev,
                           const double* scale_host, double* Xs, int* info, const SysPart& p, cudaStream_t st);
 // S_s + shift_rel trace(S_s) I = T^H T (Cholesky, FP64, one block per
-// system), Tinv_s = T^-1; identity if not numerically positive definite.
-// L <= 118 per system.
-bk_status launch_chol_inv(const double* S, double* Tinv, const SysPart& p, cudaStream_t st, double shift_rel = 0.0);
+// system), Tinv_s = T^-1.  floor > 0: a pivot below floor L S_kk is replaced by
+// that, unless it is below CHOL_EXACT S_kk.  Identity if S is not numerically
+// positive definite.  L <= 118 per system.
+//
+// CHOL_FLOOR32 is for Gram matrices of FP32 / FP16 blocks.  Their FP32 sums carry
+// errors of about three roundings (2^-24) of sqrt(S_ii S_jj), so up to L times
+// that in a pivot.  P's columns soon depend on one another to that accuracy,
+// and then a small pivot is as often negative as not.  To leave the basis alone
+// because of it loses the convergence: 4^4, 12 columns of Z4 or Gaussian sources, eight
+// shadow blocks, 35 to 328 iterations; 35 to 46 (one of sixteen 93) with the floor,
+// 33 to 36 in FP64.  Any regular T leaves the iterates as they are in exact
+// arithmetic.  (In a model of the iteration half the floor leaves counts above
+// 100, and S exact gives the same counts as this floor.)
+// Columns that are equal give a pivot of FP64 rounding: there is no basis, and
+// the L x L solve has to report it.
+constexpr double CHOL_FLOOR32 = 2e-7, CHOL_EXACT = 1e-14;
+bk_status launch_chol_inv(const double* S, double* Tinv, const SysPart& p, cudaStream_t st, double shift_rel = 0.0,
+                          double floor = 0.0);
 
 // ---------------------------------------------------------------- small.cu
 // The L x L steps of an iteration for systems of at most SMALL_MAXL columns,
@@ -209,5 +224,5 @@ struct SmallStep {
     int* zbad;
 };
 bk_status launch_small_step(const SmallStep& a, cudaStream_t st);
-// S_s = T^H T, Tinv_s = T^-1 (identity if not numerically positive definite)
-bk_status launch_small_chol(const double* S, double* Tinv, const SysPart& p, cudaStream_t st);
+// S_s = T^H T, Tinv_s = T^-1; floor as for launch_chol_inv
+bk_status launch_small_chol(const double* S, double* Tinv, const SysPart& p, double floor, cudaStream_t st);

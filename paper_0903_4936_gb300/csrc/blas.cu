@@ -909,10 +909,11 @@ __global__ void __launch_bounds__(128) k_lu_solve(const double2* __restrict__ LU
 // k_chol_inv: one thread block per system.  S = V^H V (Hermitian positive
 // definite, FP64) is factored as S = T^H T with T upper triangular, and
 // Tinv = T^-1 is written (row-major, zeros below the diagonal).  If S is not
-// numerically positive definite, Tinv = identity (the basis is left as it is).
+// numerically positive definite, Tinv = identity (the basis is left as it is);
+// floor as in bk_kernels.h.
 
 __global__ void __launch_bounds__(256) k_chol_inv(const double2* __restrict__ S, double2* __restrict__ Tinv,
-                                                  SysPart p, double shift_rel) {
+                                                  SysPart p, double shift_rel, double floor) {
     extern __shared__ double2 ch_smem_raw[];
     const int s = blockIdx.x;
     if (!((p.active >> s) & 1u)) return;
@@ -943,8 +944,10 @@ __global__ void __launch_bounds__(256) k_chol_inv(const double2* __restrict__ S,
     __syncthreads();
     for (int k = 0; k < n; ++k) {
         if (tid == 0) {
-            const double d = A[k * n + k].r;
-            if (!(d > 1e-14 * dmax) || !isfinite(d)) bad = 1;
+            double d = A[k * n + k].r;
+            const double low = floor * n * S[off + k * n + k].x;
+            if (low > 0.0 && d <= low && fabs(d) > CHOL_EXACT / (floor * n) * low) d = low;
+            if (!(d > (floor > 0.0 ? 0.0 : 1e-14 * dmax)) || !isfinite(d)) bad = 1;
             else A[k * n + k] = mk(sqrt(d), 0.0);
         }
         __syncthreads();
@@ -1229,7 +1232,8 @@ bk_status launch_lu_solve(const double* LU, const int* piv, const double* H, con
     return BK_OK;
 }
 
-bk_status launch_chol_inv(const double* S, double* Tinv, const SysPart& p, cudaStream_t st, double shift_rel) {
+bk_status launch_chol_inv(const double* S, double* Tinv, const SysPart& p, cudaStream_t st, double shift_rel,
+                          double floor) {
     int maxL = 0;
     for (int s = 0; s < p.nsys; ++s) maxL = std::max(maxL, p.L[s]);
     if (maxL > 118) {
@@ -1238,7 +1242,7 @@ bk_status launch_chol_inv(const double* S, double* Tinv, const SysPart& p, cudaS
     }
     const size_t smem = (size_t)maxL * maxL * sizeof(double2);
     BK_CUDA_TRY(cudaFuncSetAttribute(k_chol_inv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_chol_inv<<<p.nsys, 256, smem, st>>>((const double2*)S, (double2*)Tinv, p, shift_rel);
+    k_chol_inv<<<p.nsys, 256, smem, st>>>((const double2*)S, (double2*)Tinv, p, shift_rel, floor);
     BK_CUDA_TRY(cudaGetLastError());
     return BK_OK;
 }

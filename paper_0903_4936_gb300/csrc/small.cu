@@ -240,15 +240,15 @@ __global__ void __launch_bounds__(NT + 32) k_small_step(const __grid_constant__ 
     }
 }
 
-// Tinv_s = T^-1 with S_s = T^H T, T upper triangular; identity if S is not
-// numerically positive definite.  Elimination on [S | 1] without pivoting
-// gives S = L D L^H and the rows of L^-1; T^-1 = L^-H D^-1/2.  One barrier a
-// step: a step writes only rows below k, and column k no more.
+// Tinv_s = T^-1 with S_s = T^H T, T upper triangular.  Elimination on [S | 1]
+// without pivoting gives S = L D L^H and the rows of L^-1; T^-1 = L^-H D^-1/2.
+// One barrier a step: a step writes only rows below k, and column k no more.
+// floor as for launch_chol_inv.
 template <int N>
 __global__ void __launch_bounds__(NT) k_small_chol(const double2* __restrict__ S, double2* __restrict__ Tinv,
-                                                  const __grid_constant__ SysPart p) {
+                                                  const __grid_constant__ SysPart p, double floor) {
     __shared__ cx<double> A[N][N], R[N][N];
-    __shared__ double rs[N];
+    __shared__ double rs[N], lows[N];
     const int s = blockIdx.x, tid = threadIdx.x;
     if (!((p.active >> s) & 1ull)) return;
     const int n = p.L[s], off = p.coef_off[s];
@@ -256,6 +256,7 @@ __global__ void __launch_bounds__(NT) k_small_chol(const double2* __restrict__ S
         const double2 g = S[off + e];
         A[e / n][e % n] = mk(g.x, g.y);
         R[e / n][e % n] = mk(e / n == e % n ? 1.0 : 0.0, 0.0);
+        if (e / n == e % n) lows[e / n] = floor * n * g.x;
     }
     __syncthreads();
     u64 dm = 0;
@@ -267,8 +268,16 @@ __global__ void __launch_bounds__(NT) k_small_chol(const double2* __restrict__ S
     __syncthreads();  // every thread has the diagonal before a step changes it
     bool bad = false;
     for (int k = 0; k < n; ++k) {
-        const double d = A[k][k].r;
-        if (!(d > dmin) || !isfinite(d)) {
+        const double low = floor > 0.0 ? lows[k] : dmin;
+        double d = A[k][k].r;
+        if (!(d > low)) {
+            if (!(floor > 0.0) || !(low > 0.0) || !(fabs(d) > CHOL_EXACT / (floor * n) * low)) {
+                bad = true;
+                break;
+            }
+            d = low;
+        }
+        if (!isfinite(d)) {
             bad = true;
             break;
         }
@@ -307,15 +316,15 @@ bk_status launch_small_step(const SmallStep& a, cudaStream_t st) {
     return BK_OK;
 }
 
-bk_status launch_small_chol(const double* S, double* Tinv, const SysPart& p, cudaStream_t st) {
+bk_status launch_small_chol(const double* S, double* Tinv, const SysPart& p, double floor, cudaStream_t st) {
     int maxL = 0;
     for (int s = 0; s < p.nsys; ++s) maxL = std::max(maxL, p.L[s]);
     if (maxL > SMALL_MAXL) {
         bk_set_error("the one-launch Cholesky supports L <= %d per system", SMALL_MAXL);
         return BK_ERR_INVALID_ARG;
     }
-    if (maxL <= 6) k_small_chol<6><<<p.nsys, NT, 0, st>>>((const double2*)S, (double2*)Tinv, p);
-    else k_small_chol<12><<<p.nsys, NT, 0, st>>>((const double2*)S, (double2*)Tinv, p);
+    if (maxL <= 6) k_small_chol<6><<<p.nsys, NT, 0, st>>>((const double2*)S, (double2*)Tinv, p, floor);
+    else k_small_chol<12><<<p.nsys, NT, 0, st>>>((const double2*)S, (double2*)Tinv, p, floor);
     BK_CUDA_TRY(cudaGetLastError());
     return BK_OK;
 }

@@ -429,3 +429,24 @@ def test_fp64_anchor_replacements(c1, method, eo):
     assert _dev(X.cpu().numpy(), Xd) <= 1e-8
     assert info["matvecs_fp64"] < ref["matvecs_fp64"], (info["matvecs_fp64"], ref["matvecs_fp64"])
     assert info["iterations"] <= 1.5 * ref["iterations"] + 5
+
+
+@pytest.mark.parametrize("anchor", [0.0, 1e-4])
+@pytest.mark.parametrize("source", ["gauss", "z4"])
+def test_fp32_blocks_keep_the_fp64_iteration_count(c1, source, anchor):
+    """P's columns come to depend on one another to FP32 accuracy, so P^H P (FP32 sums) has pivots that are rounding.
+    The basis change has to go on all the same: without it most of these eight shadow blocks take 75 to 330
+    iterations.  Bound as for the anchored replacements, half as many iterations again as in FP64 and five, over
+    the eight together (single FP32 solves take twice the count now and then, with exact Gram matrices too)."""
+    dims, lat, U, B, Xd, A = c1
+    B = (synth.gaussian_sources if source == "gauss" else synth.z4_noise)(dims, 12, 41)
+    Bt = torch.from_numpy(B).cuda()
+    total = want = 0
+    for seed in range(8):
+        kw = dict(method="bicgstab", tol=1e-10, maxiter=1000, seed=seed)
+        X, info = lat.block_solve(Bt, 0.12, prec="fp32", delta=0.003, anchor=anchor, **kw)
+        _, ref = lat.block_solve(Bt, 0.12, prec="fp64", orth=True, **kw)
+        assert info["converged"] == 1 and info["true_res_max"] <= 1e-10
+        total += info["iterations"]
+        want += 1.5 * ref["iterations"] + 5
+    assert total <= want
