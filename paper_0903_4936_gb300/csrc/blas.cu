@@ -1017,13 +1017,23 @@ bk_status gram_dispatch(int prec, Field A, Field B, Field B2, int NB, const SysP
 
 }  // namespace
 
+// Partial-sum rows a partition may use, whichever of its systems are active: no
+// more partial sums than a block has elements.  That binds for wide systems on
+// small lattices (4^4, 512 columns: 6 rows and 50 MB; 304 rows of 512^2 sums
+// are 2.5 GB).
+static int gram_chunk_limit(const SysPart& p, int V) {
+    const long long rows = 12LL * V * p.col0[p.nsys] / std::max(1, p.coef_off[p.nsys]);
+    return (int)std::max(1LL, std::min<long long>(rows, gram_row_chunks_max(V)));
+}
+
 // partial-sum rows of a Gram matrix over the active systems
 static int gram_chunks(int prec, const SysPart& p, int V) {
-    return max_active_L(p) <= ROWS_MAXL ? gram_row_chunks(prec, V, row_tiles(prec, p)) : wide_gram_chunks(p, V);
+    const int n = max_active_L(p) <= ROWS_MAXL ? gram_row_chunks(prec, V, row_tiles(prec, p)) : wide_gram_chunks(p, V);
+    return std::min(n, gram_chunk_limit(p, V));
 }
 
 size_t gram_partial_bytes(const SysPart& p, int V) {
-    return (size_t)2 * gram_row_chunks_max(V) * std::max(1, p.coef_off[p.nsys]) * sizeof(double2);
+    return (size_t)2 * gram_chunk_limit(p, V) * std::max(1, p.coef_off[p.nsys]) * sizeof(double2);
 }
 
 bk_status launch_gram(int prec, Field A, Field B, const SysPart& p, double* G, double* partial, int V,
@@ -1047,8 +1057,12 @@ bk_status launch_gram_slots(int prec, Field A, Field B, const SysPart& p, double
     return gram_dispatch(prec, A, B, B, 1, p, G, nullptr, partial, nchunk, V, st);
 }
 
+// For any range of the L columns: a range of nq pairs takes at most one row
+// chunk per 32 rows, and MAX_CHUNKS over its groups of 32 pairs, so at most 64
+// MAX_CHUNKS sums in all (one chunk from MAX_CHUNKS groups on).
 size_t coldot_partial_bytes(int L, int npair, int V) {
-    return (size_t)MAX_CHUNKS * npair * (2 * npairs(L) + 2) * sizeof(double2);
+    const size_t cols = 2 * (size_t)npairs(L), chunks = std::max(1, std::min(MAX_CHUNKS, 12 * V / 32));
+    return std::max(std::min(chunks * cols, (size_t)64 * MAX_CHUNKS), cols) * npair * sizeof(double2);
 }
 
 bk_status launch_coldot(int prec, int npair, const Field* A, const Field* B, int c0, int n, double* out, int ldo,

@@ -150,3 +150,18 @@ def test_many_wide_systems(nsys, L):
                                        maxiter=1, raise_on_fail=False)
     assert infos[0]["status"] == "BK_ERR_NOT_CONVERGED"
     assert all(i["iterations"] == 1 and np.isfinite(i["rec_res_max"]) for i in infos)
+
+
+def test_wide_gram_workspace_on_a_small_lattice():
+    """The partial sums of a wide Gram matrix take no more memory than a few blocks of its operands' size."""
+    dims, L = (4, 4, 4, 4), 512
+    lat, _ = _lat(dims)
+    A = lat.pack(torch.from_numpy(synth.gaussian_sources(dims, L, 64)).cuda(), "fp64")
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    G = lat.gram(A, A, L, "fp64")
+    torch.cuda.synchronize()
+    # G, its partial sums (two operands' worth) and a 2 MB allocation granule for each, with room for one block more
+    assert before - torch.cuda.mem_get_info()[0] <= 4 * A.numel() + 16 * L * L + (4 << 20)
+    a = lat.unpack(A, L, "fp64").cpu().numpy().reshape(L, -1)
+    assert _rel(G.cpu().numpy(), a.conj() @ a.T) < GRAM_TOL["fp64"]
