@@ -158,10 +158,9 @@ bk_status bk_gamma5(bk_ctx* ctx, const double* X, double* Y, int L, void* stream
 /* Block inner product (Section 3, the L x L matrices R~_0^H V_k etc.):
  *     G[i][j] = sum_{n, alpha, a} conj(A_i(n,alpha,a)) B_j(n,alpha,a)
  * for device-layout blocks A, B of L columns in prec.  G: device array of
- * L*L complex FP64 {re, im}, row-major.  Products, per-thread partial sums
- * and the sum across one warp are in the arithmetic precision of prec; sums
- * across warps and thread blocks are FP64.  Uses library workspace for the
- * per-block partial sums.
+ * L*L complex FP64 {re, im}, row-major.  Products and sums of at most 96
+ * rows (site, component) are in the arithmetic precision of prec, all further
+ * sums in FP64.  Uses library workspace for the per-block partial sums.
  * Errors: INVALID_ARG, CUDA.                                              */
 bk_status bk_block_gram(bk_ctx* ctx, const void* A, const void* B, int L, bk_prec prec,
                         double* G, void* stream);

@@ -185,7 +185,7 @@ __device__ __forceinline__ cx<typename Prec<P>::real> coef(const double* ptr, do
 }
 
 // FP32 products are summed in FP32 over at most this many (site, component)
-// rows per lane, then moved to FP64
+// rows, the lanes added in FP32 included, then in FP64
 constexpr int ROW_FLUSH = 96;
 
 // rows.cu: systems of at most ROWS_MAXL columns

@@ -63,11 +63,11 @@ __device__ __forceinline__ RLane rlane(const SysPart& p, int tp0, int tnp, int l
 // writes one partial row per chunk.
 //
 // FP32 / FP16 products are summed in FP32 registers (packed pairs over j).
-// Every ROW_FLUSH rows these go to FP64 accumulators in shared memory; with
-// several rows side by side (spw > 1) the lanes of one column pair are added
-// in FP32 first, so that the conversion and the FP64 add, 16 cycles of the
-// SM's FP64 pipe per warp instruction, are done once per entry by a full warp
-// instead of once per lane.
+// Every ROW_FLUSH rows these go to FP64 accumulators in shared memory.  With
+// several rows side by side (spw > 1) a full warp does that for all lanes of a
+// column pair, and where the lanes have few rows each (small lattices: 8) it
+// adds them in FP32 first, up to ROW_FLUSH rows to a sum: an FP64 add takes 16
+// cycles of the SM's FP64 pipe per warp instruction.
 // FP64 sums stay in registers and are added over the rows in the tail.
 
 template <int P, int NB, int MAXL, int UR>
@@ -119,13 +119,21 @@ __global__ void __launch_bounds__(GW * 32, P == BK_FP64 ? 1 : 2) k_gram_r(Field 
                     c = cp_zero<R2>();
                 }
         if (staged) {
+            const int lanes = ROW_FLUSH / max(since, 1);  // of an FP32 sum
             __syncwarp();
+#pragma unroll 1
             for (int x = lane; x < NACC * tnp; x += 32) {
                 const int e = x / tnp, pr = x - e * tnp;
-                float2 v = stage[e * 32 + pr];
-                for (int sub = 1; sub < spw; ++sub) v = padd(v, stage[e * 32 + sub * tnp + pr]);
-                if (first) my[x] = make_double2(f2d(v.x), f2d(v.y));
-                else my[x] = make_double2(my[x].x + f2d(v.x), my[x].y + f2d(v.y));
+                double2 sum = first ? make_double2(0.0, 0.0) : my[x];
+#pragma unroll 1
+                for (int s0 = 0; s0 < spw; s0 += lanes) {
+                    float2 v = stage[e * 32 + s0 * tnp + pr];
+                    for (int sub = s0 + 1; sub < min(s0 + lanes, spw); ++sub)
+                        v = padd(v, stage[e * 32 + sub * tnp + pr]);
+                    if (first && s0 == 0) sum = f2d(v);
+                    else sum = make_double2(sum.x + f2d(v.x), sum.y + f2d(v.y));
+                }
+                my[x] = sum;
             }
             __syncwarp();
         }

@@ -42,21 +42,13 @@ __device__ __forceinline__ void stage_elem(CxPair<typename Prec<P>::pair>* dst, 
     }
 }
 
-// s + e = a + b exactly (Knuth), on packed pairs
-__device__ __forceinline__ void two_sum(float2 a, float2 b, float2& s, float2& e) {
-    s = padd(a, b);
-    const float2 t = psub(s, a);
-    e = padd(psub(a, psub(s, t)), psub(b, t));
-}
-
 // ---------------------------------------------------------------- Gram
 //
 // A block takes one system (and at most `threads` of its 4 x 4 column tiles)
 // and one chunk of rows; `slices` groups of threads share the rows of a stage.
-// FP32 sums of ROW_FLUSH rows are added to unevaluated sums of two floats
-// (error-free addition, 48 bits) in registers instead of FP64, whose pipe would
-// take a third of the kernel's time for it; slices and chunks are added in
-// FP64.
+// FP32 sums of at most ROW_FLUSH rows are added to FP64 sums in shared memory.
+// The FP64 pipe needs a third of the multiply-adds' time for that, so a thread
+// moves a quarter of its sums at a time and goes on multiplying meanwhile.
 
 struct WideWork {
     int n;
@@ -83,15 +75,15 @@ __global__ void __launch_bounds__(320, P == BK_FP64 ? 1 : 2) k_gram_t(Field A, F
     const int ia[2] = {ti, min(ti + side, nps - 1)}, jb[2] = {tj, min(tj + side, nps - 1)};
     E* buf = reinterpret_cast<E*>(wide_smem);  // [2][A, B][half]: KR rows of nps elements
     R2 acr[4][2], aci[4][2];  // [column of A][pair of B]
-    // FP32 / FP16: the thread's sums of two floats, [entry][thread] {hi pair, lo pair}
-    float4* sums = reinterpret_cast<float4*>(buf + (size_t)4 * half) + threadIdx.x;
+    // FP32 / FP16: the thread's FP64 sums, [entry][thread] {pair}
+    double2* sums = reinterpret_cast<double2*>(buf + (size_t)4 * half) + threadIdx.x;
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
         for (int b = 0; b < 2; ++b) acr[a][b] = aci[a][b] = pzero<R2>();
     if constexpr (P != BK_FP64)
 #pragma unroll
-        for (int k = 0; k < 16; ++k) sums[k * T] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int k = 0; k < 16; ++k) sums[k * T] = make_double2(0.0, 0.0);
     const unsigned per = (rows + nchunk - 1) / nchunk, r0 = (unsigned)chunk * per;
     const unsigned r1 = min(rows, r0 + per);
     const int nst = r0 < r1 ? (int)((r1 - r0 + KR - 1) / KR) : 0;
@@ -115,26 +107,29 @@ __global__ void __launch_bounds__(320, P == BK_FP64 ? 1 : 2) k_gram_t(Field A, F
         }
         copy_commit();
     };
-    int since = 0;
-    auto flush = [&]() {
+    // row a of the 4 x 4 columns; all of them for a < 0
+    auto flush = [&](int row) {
         if constexpr (P != BK_FP64) {
 #pragma unroll
-            for (int a = 0; a < 4; ++a)
+            for (int a = 0; a < 4; ++a) {
+                if (row >= 0 && a != row) continue;
 #pragma unroll
                 for (int b = 0; b < 2; ++b)
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
                         float2& v = c ? aci[a][b] : acr[a][b];
-                        float4& t = sums[((a * 2 + b) * 2 + c) * T];
-                        float2 h, e;
-                        two_sum(make_float2(t.x, t.y), v, h, e);
-                        e = padd(make_float2(t.z, t.w), e);
-                        t = make_float4(h.x, h.y, e.x, e.y);
+                        double2& t = sums[((a * 2 + b) * 2 + c) * T];
+                        t = make_double2(t.x + f2d(v.x), t.y + f2d(v.y));
                         v = make_float2(0.f, 0.f);
                     }
+            }
         }
-        since = 0;
     };
+    // rows of a stage that a thread takes; a quarter of the sums after every
+    // ROW_FLUSH / 4 rows, or all after ROW_FLUSH where a stage is longer than that
+    const int per_stage = (KR + slices - 1) / slices;
+    const bool quarters = per_stage <= ROW_FLUSH / 4;
+    int since = 0, next = 0;
     if (nst > 0) issue(0);
     for (int st = 0; st < nst; ++st) {
         if (st + 1 < nst) {
@@ -172,12 +167,16 @@ __global__ void __launch_bounds__(320, P == BK_FP64 ? 1 : 2) k_gram_t(Field A, F
                     }
                 }
             }
-            since += (nr + slices - 1) / slices;
-            if (since >= ROW_FLUSH) flush();
+            since += per_stage;
+            if (P != BK_FP64 && since + per_stage > (quarters ? ROW_FLUSH / 4 : ROW_FLUSH)) {
+                flush(quarters ? next : -1);
+                next = (next + 1) & 3;
+                since = 0;
+            }
         }
         __syncthreads();
     }
-    flush();
+    flush(-1);
     // slices in FP64 through shared memory, 8 of the 16 entries at a time
     double2* red = reinterpret_cast<double2*>(wide_smem);  // [slice][8][ntile]
     const int ne = p.coef_off[p.nsys], tl = threadIdx.x - slice * ntile;
@@ -194,9 +193,9 @@ __global__ void __launch_bounds__(320, P == BK_FP64 ? 1 : 2) k_gram_t(Field A, F
                         re = y ? acr[a][b].y : acr[a][b].x;
                         im = y ? aci[a][b].y : aci[a][b].x;
                     } else {
-                        const float4 r = sums[(a * 2 + b) * 2 * T], i = sums[((a * 2 + b) * 2 + 1) * T];
-                        re = f2d(y ? r.y : r.x) + f2d(y ? r.w : r.z);
-                        im = f2d(y ? i.y : i.x) + f2d(y ? i.w : i.z);
+                        const double2 r = sums[(a * 2 + b) * 2 * T], i = sums[((a * 2 + b) * 2 + 1) * T];
+                        re = y ? r.y : r.x;
+                        im = y ? i.y : i.x;
                     }
                     red[((size_t)slice * 8 + 2 * a + y) * ntile + tl] = make_double2(re, im);
                 }
@@ -277,8 +276,8 @@ bk_status wide_gram_p(Field A, Field B, const SysPart& p, double2* partial, int 
         bk_set_error("Gram supports systems of at most 512 columns");
         return BK_ERR_INVALID_ARG;
     }
-    // rows a stage: two stages in at most 32 KB beside the two-float sums (FP64: 96 KB), so that two blocks fit
-    const size_t lim = (P == BK_FP64 ? 48 : 16) * 1024, sums = P == BK_FP64 ? 0 : (size_t)T * 16 * sizeof(float4);
+    // rows a stage: two stages in at most 32 KB beside the FP64 sums (FP64: 96 KB), so that two blocks fit
+    const size_t lim = (P == BK_FP64 ? 48 : 16) * 1024, sums = P == BK_FP64 ? 0 : (size_t)T * 16 * sizeof(double2);
     const int KR = (int)std::max<size_t>(1, std::min<size_t>(64, lim / row));
     // (the slices' sums overwrite the stages: 128 bytes a thread)
     const size_t stage = std::max((size_t)2 * KR * row, (size_t)T * 8 * sizeof(double2));

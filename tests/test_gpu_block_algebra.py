@@ -165,3 +165,17 @@ def test_wide_gram_workspace_on_a_small_lattice():
     assert before - torch.cuda.mem_get_info()[0] <= 4 * A.numel() + 16 * L * L + (4 << 20)
     a = lat.unpack(A, L, "fp64").cpu().numpy().reshape(L, -1)
     assert _rel(G.cpu().numpy(), a.conj() @ a.T) < GRAM_TOL["fp64"]
+
+
+@pytest.mark.parametrize("dims,L", [((8, 8, 8, 8), 2), ((8, 8, 8, 8), 6), ((8, 8, 8, 8), 12), ((16, 16, 16, 8), 13),
+                                    ((16, 16, 16, 8), 48)])
+def test_fp32_gram_beyond_the_fp32_range(dims, L):
+    """Sums of at most 96 rows are in FP32 and the rest in FP64: 96 rows of these blocks stay within FP32's range
+    (2.8e38 of 3.4e38), all of them are 500 times above it."""
+    lat, _ = _lat(dims)
+    c = np.float32(1.2e18)
+    F = lat.empty_field(L, "fp32")
+    F.view(torch.float32).fill_(float(c))
+    G = lat.gram(F, F, L, "fp32").cpu().numpy()
+    want = 2.0 * float(c) ** 2 * 12 * np.prod(dims)  # conj(c + ic)(c + ic) per row
+    assert np.all(np.isfinite(G)) and np.max(np.abs(G - want)) < GRAM_TOL["fp32"] * want
