@@ -35,6 +35,10 @@
  *  - stream: a cudaStream_t cast to void* (NULL = legacy default stream).
  *    Work is enqueued on it; functions that must read results back to the
  *    host (bk_block_solve*) synchronise it.
+ *  - Library workspace belongs to the context.  Calls of one context that use
+ *    it, or that change the gauge field or the clover term, must follow one
+ *    another on the device (one stream, or events between streams) and be
+ *    made by one host thread at a time.
  */
 #ifndef BKRYLOV_H
 #define BKRYLOV_H
@@ -96,7 +100,10 @@ bk_status bk_upload_gauge(bk_ctx* ctx, const double* U, int U_on_device, void* s
  * stores the kappa-independent site matrix
  *     C(n) = c_SW * sum_{mu,nu} (i/2) sigma_mu_nu F_mu_nu(n)
  * as two 6x6 Hermitian blocks (chiral basis) in FP64 and FP32.
- * csw = 0 gives the plain Wilson operator.  Errors: NO_GAUGE, CUDA.        */
+ * csw = 0 gives the plain Wilson operator.  The stored term is written once,
+ * with its final values: to rebuild the same term changes nothing for calls
+ * that read it meanwhile on other streams.  Uses library workspace (768 bytes
+ * per site).  Errors: NO_GAUGE, CUDA (the context then has no clover term). */
 bk_status bk_build_clover(bk_ctx* ctx, double csw, void* stream);
 
 /* bk_build_clover on the legacy default stream, returning once the clover

@@ -101,7 +101,8 @@ struct bk_ctx {
     int dims[4];
     int V;
     int device;
-    DevBuf U64, U32, C64, C32, Utmp;
+    DevBuf U64, U32, C64, C32;
+    DevBuf Utmp;  // links on their way from the host; scratch of a clover build
     bool has_gauge = false, has_clover = false;
     double csw = 0.0;
     // scratch of the single-operation entry points
@@ -174,7 +175,8 @@ extern "C" bk_status bk_create(const int dims[4], int device, bk_ctx** out) {
     if ((s = c->U64.ensure((size_t)36 * V * sizeof(double2))) != BK_OK ||
         (s = c->U32.ensure((size_t)4 * V * BK_LINKC * sizeof(float))) != BK_OK ||
         (s = c->C64.ensure((size_t)36 * V * sizeof(double2))) != BK_OK ||
-        (s = c->C32.ensure((size_t)V * BK_CLOVC * sizeof(float))) != BK_OK) {
+        (s = c->C32.ensure((size_t)V * BK_CLOVC * sizeof(float))) != BK_OK ||
+        (s = c->Utmp.ensure(clover_scratch_bytes((int)V))) != BK_OK) {
         bk_destroy(c);
         return s;
     }
@@ -208,7 +210,7 @@ extern "C" bk_status bk_upload_gauge(bk_ctx* c, const double* U, int on_device, 
     BK_CUDA_TRY(cudaSetDevice(c->device));
     const double* src = U;
     if (!on_device) {
-        BK_TRY(c->Utmp.ensure((size_t)36 * c->V * sizeof(double2)));
+        // (36 of the 48 double2 a site that clover_scratch_bytes() gives)
         BK_CUDA_TRY(cudaMemcpyAsync(c->Utmp.p, U, (size_t)36 * c->V * sizeof(double2), cudaMemcpyHostToDevice, st));
         src = c->Utmp.as<double>();
     }
@@ -227,8 +229,13 @@ extern "C" bk_status bk_build_clover(bk_ctx* c, double csw, void* stream) {
         return BK_ERR_NO_GAUGE;
     }
     BK_CUDA_TRY(cudaSetDevice(c->device));
-    BK_TRY(launch_clover_build(c->U64.as<double2>(), c->C64.as<double2>(), c->C32.as<float>(), c->dims, csw,
-                               (cudaStream_t)stream));
+    const bk_status r = launch_clover_build(c->U64.as<double2>(), c->C64.as<double2>(), c->C32.as<float>(),
+                                            c->Utmp.as<double2>(), c->dims, csw, (cudaStream_t)stream);
+    if (r != BK_OK) {  // the launches before the failed one may have gone through
+        c->has_clover = false;
+        c->cinv.clear();
+        return r;
+    }
     c->csw = csw;
     c->has_clover = true;
     c->cinv.clear();

@@ -8,8 +8,10 @@
 
 // ---------------------------------------------------------------- gauge.cu
 bk_status launch_gauge_convert(const double* Uin_dev, double2* U64, float* U32, int V, cudaStream_t st);
-bk_status launch_clover_build(const double2* U64, double2* C64, float* C32, const int dims[4], double csw,
-                              cudaStream_t st);
+// scratch: clover_scratch_bytes() bytes; C64 and C32 are written by the last kernel alone
+size_t clover_scratch_bytes(int V);
+bk_status launch_clover_build(const double2* U64, double2* C64, float* C32, double2* scratch, const int dims[4],
+                              double csw, cudaStream_t st);
 // Even-odd form: A(n)^-1 = (1 - kappa C(n))^-1 for one kappa, stored like the
 // clover (FP64 [36][V], FP32 compact); bound[0] = the largest infinity
 // norm of A's chiral blocks (as double bits), bound[1] += singular blocks.

@@ -244,16 +244,16 @@ __device__ __forceinline__ cx<double> chiral_elem(const M3& G1, const M3& G2, co
     return mk(-g1.r, -g1.i) - ti(g2);
 }
 
-// The FP32 copy holds the same 72 reals of a site side by side.
-// C64 holds the six planes' F (5 slots each) on entry and is overwritten site by site.
-__global__ void __launch_bounds__(64) k_clover_build(double2* __restrict__ C64, float* __restrict__ C32, int V,
-                                                     double csw) {
+// The FP32 copy holds the same 72 reals of a site side by side.  F: the six
+// planes, 5 slots each.
+__global__ void __launch_bounds__(64) k_clover_build(const double2* __restrict__ F, double2* __restrict__ C64,
+                                                     float* __restrict__ C32, int V, double csw) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= V) return;
     // F indices: 0=x,1=y,2=z,3=t.  Paper F_23 = F(1,2), F_14 = F(0,3), F_31 = F(2,0),
     // F_24 = F(1,3), F_12 = F(0,1), F_34 = F(2,3).
-    const M3 F12 = load_F(C64, 0, V, s), F23 = load_F(C64, 1, V, s), F31 = load_F(C64, 2, V, s);
-    const M3 F14 = load_F(C64, 3, V, s), F24 = load_F(C64, 4, V, s), F34 = load_F(C64, 5, V, s);
+    const M3 F12 = load_F(F, 0, V, s), F23 = load_F(F, 1, V, s), F31 = load_F(F, 2, V, s);
+    const M3 F14 = load_F(F, 3, V, s), F24 = load_F(F, 4, V, s), F34 = load_F(F, 5, V, s);
     double out[72];
     const double h = 0.5 * csw;
 #pragma unroll
@@ -407,8 +407,10 @@ bk_status launch_gauge_convert(const double* Uin_dev, double2* U64, float* U32, 
     return BK_OK;
 }
 
-bk_status launch_clover_build(const double2* U64, double2* C64, float* C32, const int dims[4], double csw,
-                              cudaStream_t st) {
+size_t clover_scratch_bytes(int V) { return (size_t)(18 + 30) * V * sizeof(double2); }
+
+bk_status launch_clover_build(const double2* U64, double2* C64, float* C32, double2* scratch, const int dims[4],
+                              double csw, cudaStream_t st) {
     Geo g;
     int stride = 1;
     for (int mu = 0; mu < 4; ++mu) {
@@ -417,18 +419,18 @@ bk_status launch_clover_build(const double2* U64, double2* C64, float* C32, cons
         stride *= dims[mu];
     }
     const int V = stride;
-    // The planes one after the other: M and N in C32's memory (288 bytes a site,
-    // as many), F in C64's; then the site terms over both.
+    // The planes one after the other, each with M and N in the same 18 slots a
+    // site (they pass through L2), F in 30 more; then the site terms, written
+    // once: a rebuild of the same term never changes what an operator reads.
     const int plane[6][2] = {{0, 1}, {1, 2}, {2, 0}, {0, 3}, {1, 3}, {2, 3}};
-    double2* MN = reinterpret_cast<double2*>(C32);
-    static_assert(BK_CLOVC * sizeof(float) == 18 * sizeof(double2), "M and N fill the FP32 table");
+    double2 *MN = scratch, *F = scratch + (size_t)18 * V;
     for (int p = 0; p < 6; ++p) {
         const int mu = plane[p][0], nu = plane[p][1];
         k_corner<<<dim3((V + 63) / 64, 2), 64, 0, st>>>(U64, MN, g, V, mu, nu);
-        k_leaves<<<(V + 31) / 32, 64, 0, st>>>(U64, MN, C64 + (size_t)5 * p * V, g, V, mu, nu);
+        k_leaves<<<(V + 31) / 32, 64, 0, st>>>(U64, MN, F + (size_t)5 * p * V, g, V, mu, nu);
         BK_CUDA_TRY(cudaGetLastError());
     }
-    k_clover_build<<<(V + 63) / 64, 64, 0, st>>>(C64, C32, V, csw);
+    k_clover_build<<<(V + 63) / 64, 64, 0, st>>>(F, C64, C32, V, csw);
     BK_CUDA_TRY(cudaGetLastError());
     return BK_OK;
 }

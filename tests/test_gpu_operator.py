@@ -260,3 +260,26 @@ def test_dslash_benchmark_sizes_sampled_sites(prec, dims, L, kappas):
         ref = dirac.apply_dirac_at(U, Xp, kap[cols], 1.0, sites, dims) * cj[cols][:, None, None, None]
         err = max(err, _rel(got[cols], ref))
     assert err < TOL[prec], err
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_clover_rebuild_beside_operator_calls(prec):
+    """To build the same clover term again, as every backward pass does, changes nothing for operator calls that run
+    meanwhile on another stream: the same result bit for bit."""
+    import paper_0903_4936_gb300 as bk
+    dims, L = (8, 8, 8, 16), 12
+    lat = bk.Lattice(dims)
+    lat.upload_gauge(synth.random_su3_field(dims, 0.5, 1002))
+    lat.build_clover(1.0)
+    X = lat.pack(torch.from_numpy(synth.gaussian_sources(dims, L, 3)).cuda(), prec)
+    want = lat.dslash_dev(X, L, 0.12, prec).clone()
+    outs = [torch.zeros_like(X) for _ in range(30)]
+    torch.cuda.synchronize()
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    for Y in outs:
+        with torch.cuda.stream(a):
+            lat.dslash_dev(X, L, 0.12, prec, out=Y)
+        with torch.cuda.stream(b):
+            lat.build_clover(1.0)
+    torch.cuda.synchronize()
+    assert all(torch.equal(Y, want) for Y in outs)
