@@ -53,7 +53,7 @@ __device__ __forceinline__ void stage_elem(CxPair<typename Prec<P>::pair>* dst, 
 struct WideWork {
     int n;
     int sys[256];
-    int t0[256];  // first tile
+    int t0[256];  // Gram: first tile; update: pairs of comb a stage
 };
 
 template <int P>
@@ -302,7 +302,7 @@ constexpr int UQ = 128;
 template <int P>
 __global__ void __launch_bounds__(UT, P == BK_FP64 ? 1 : 2) k_update_t(const __grid_constant__ GenOp g,
                                                                       const __grid_constant__ WideWork w,
-                                                                      unsigned rows, int nchunk, int ncols, int KCmax) {
+                                                                      unsigned rows, int nchunk, int ncols) {
     using R = typename Prec<P>::real;
     using R2 = typename Prec<P>::pair;
     using E = CxPair<R2>;
@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(UT, P == BK_FP64 ? 1 : 2) k_update_t(const __g
     const int rt = NR * nrg;  // rows of a tile
     const int rg = threadIdx.x / ng, cg = threadIdx.x - rg * ng;
     const bool on = rg < nrg, has1 = cg + ng < wps;
-    const int KC = min(nps, KCmax), cstr = KC | 1;  // odd row stride: rows in different banks
+    const int KC = w.t0[blockIdx.x], cstr = KC | 1;  // odd row stride: rows in different banks
     E* Cs = reinterpret_cast<E*>(wide_smem);  // [rt][cstr]
     E* Ms = Cs + (size_t)rt * cstr;           // [2 KC][wps]: {M_i,2q, M_i,2q+1} real parts, imaginary parts
     const bool mat = g.mat != 0, hx = g.hasX != 0;
@@ -542,28 +542,31 @@ bk_status wide_update_p(const GenOp& g, int V, int nchunk, cudaStream_t st) {
     using E = CxPair<typename Prec<P>::pair>;
     WideWork w;
     w.n = 0;
-    for (int s = 0; s < g.p.nsys; ++s)
-        if ((g.p.active >> s) & 1ull) {
-            w.sys[w.n] = s;
-            w.t0[w.n++] = 0;
-        }
-    const int maxnps = (max_active_L(g.p) + 1) / 2;
-    // pairs of comb a stage: 80 KB a block (two blocks an SM) for every system of the launch
-    int KC = maxnps;
-    size_t smem = 0;
-    for (;; KC = (KC + 1) / 2) {
-        smem = 2 * UT * sizeof(double2);
-        for (int i = 0; i < w.n; ++i) {
-            const int nps = (g.p.L[w.sys[i]] + 1) / 2, kc = std::min(nps, KC);
+    int maxnps = 0;
+    size_t smem = 2 * UT * sizeof(double2);
+    for (int s = 0; s < g.p.nsys; ++s) {
+        if (!((g.p.active >> s) & 1ull)) continue;
+        // pairs of comb a stage: each system's own, the most that fits 80 KB (two
+        // blocks an SM).  Not one number for all: a system of 2 pairs takes tiles
+        // of 1024 rows and would put the wide ones to one pair a stage.
+        const int nps = (g.p.L[s] + 1) / 2;
+        int KC = nps;
+        size_t need;
+        for (;; KC = (KC + 1) / 2) {
+            need = 0;
             for (int q0 = 0; q0 < nps; q0 += UQ) {
                 const int wps = std::min(UQ, nps - q0), rt = 4 * (UT / ((wps + 1) / 2));
-                smem = std::max(smem, ((size_t)rt * (kc | 1) + (size_t)2 * kc * wps) * sizeof(E));
+                need = std::max(need, ((size_t)rt * (KC | 1) + (size_t)2 * KC * wps) * sizeof(E));
             }
+            if (need <= (size_t)80 * 1024 || KC == 1) break;
         }
-        if (smem <= (size_t)80 * 1024 || KC == 1) break;
+        smem = std::max(smem, need);
+        maxnps = std::max(maxnps, nps);
+        w.sys[w.n] = s;
+        w.t0[w.n++] = KC;
     }
     BK_CUDA_TRY(cudaFuncSetAttribute(k_update_t<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_update_t<P><<<dim3(w.n, nchunk, (maxnps + UQ - 1) / UQ), UT, smem, st>>>(g, w, 12u * (unsigned)V, nchunk, g.p.col0[g.p.nsys], KC);
+    k_update_t<P><<<dim3(w.n, nchunk, (maxnps + UQ - 1) / UQ), UT, smem, st>>>(g, w, 12u * (unsigned)V, nchunk, g.p.col0[g.p.nsys]);
     BK_CUDA_TRY(cudaGetLastError());
     return BK_OK;
 }

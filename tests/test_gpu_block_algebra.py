@@ -179,3 +179,19 @@ def test_fp32_gram_beyond_the_fp32_range(dims, L):
     G = lat.gram(F, F, L, "fp32").cpu().numpy()
     want = 2.0 * float(c) ** 2 * 12 * np.prod(dims)  # conj(c + ic)(c + ic) per row
     assert np.all(np.isfinite(G)) and np.max(np.abs(G - want)) < GRAM_TOL["fp32"] * want
+
+
+@pytest.mark.parametrize("prec,Ls", [("fp64", (30, 4)), ("fp64", (20, 8)), ("fp64", (3, 40, 1)), ("fp32", (30, 4))])
+def test_wide_systems_beside_narrow_ones(prec, Ls):
+    """Updates of one launch whose systems stage different numbers of columns (3 and 4 columns take tiles of 1024
+    rows), against dense LU."""
+    dims = (4, 4, 4, 4)
+    lat, U = _lat(dims, 17)
+    B = synth.z4_noise(dims, sum(Ls), 35)
+    X, infos = lat.block_solve_batched(torch.from_numpy(B).cuda(), [0.11] * len(Ls), list(Ls), method="bicgstab",
+                                       prec=prec, tol=1e-10, maxiter=1000, delta=0.0 if prec == "fp64" else 0.03)
+    assert all(i["converged"] == 1 for i in infos)
+    ref = np.linalg.solve(dense.dense_matrix(U, 0.11, 1.0), dense.to_columns(B))
+    got = dense.to_columns(X.cpu().numpy())
+    # ||x - x*|| <= ||D^-1|| ||r||, ||D^-1|| < 20 at this kappa
+    assert np.max(np.linalg.norm(got - ref, axis=0) / np.linalg.norm(dense.to_columns(B), axis=0)) < 2e-9
