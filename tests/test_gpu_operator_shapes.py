@@ -74,3 +74,30 @@ def test_runs_of_columns(prec, eo):
         dev = np.linalg.norm(got[:, c0:c0 + L] - ref, axis=0) / np.linalg.norm(ref, axis=0)
         assert dev.max() <= 1e-8
         c0 += L
+
+
+# One warp a block up to 152 * 3 * 128 = 58368 (site, pair) items, four above: items on that line, the last block full
+# or not.
+@pytest.mark.parametrize("prec", ["fp32", "fp16"])
+@pytest.mark.parametrize("dims,L", [((8, 8, 6, 8), 38), ((8, 8, 6, 8), 39), ((5, 7, 9, 13), 28), ((5, 7, 9, 13), 29)])
+def test_operator_block_sizes(prec, dims, L):
+    lat, U = _lat(dims, 31 + L)
+    X = synth.gaussian_sources(dims, L, 7)
+    kap = np.linspace(0.10, 0.13, L)
+    Y = lat.dslash(torch.from_numpy(X).cuda(), list(kap), prec).cpu().numpy()
+    for j in (0, 1, L // 2, L - 1):
+        assert _rel(Y[j:j + 1], dirac.apply_dirac(U, X[j:j + 1], kap[j:j + 1], 1.0)) < TOL[prec]
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp16"])
+@pytest.mark.parametrize("dims,L", [((8, 8, 6, 16), 38), ((8, 8, 6, 16), 39), ((10, 10, 6, 14), 26),
+                                    ((10, 10, 6, 14), 27)])
+def test_schur_block_sizes(prec, dims, L):
+    lat, U = _lat(dims, 41 + L)
+    X = synth.gaussian_sources(dims, L, 8)
+    kap = np.repeat(np.linspace(0.10, 0.13, (L + 1) // 2), 2)[:L]
+    Y = lat.schur_dslash(torch.from_numpy(X).cuda(), list(kap), prec).cpu().numpy()
+    odd = evenodd.parity_mask(dims, 1)
+    for j in (0, L - 1):
+        assert np.all(Y[j][odd] == 0)
+        assert _rel(Y[j:j + 1], evenodd.schur_apply(U, X[j:j + 1], kap[j], 1.0)) < SCHUR_TOL[prec]
