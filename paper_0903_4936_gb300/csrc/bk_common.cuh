@@ -372,6 +372,7 @@ void bk_set_error(const char* fmt, ...);
 
 // Maximum columns handled by one operator launch (kernel-argument kappa list).
 #define BK_MAX_COLS 256
+// Maximum number of systems of a batched solve (one bit each in a 64-bit mask).
 #define BK_MAX_SYS 64
 // FP32 tables, in floats: a link (row-major {re, im}, padded to 80 bytes; the
 // four of a site together) and a site term (per chiral block 6 diagonal

@@ -1,15 +1,13 @@
 // Block linear algebra of block BiCGSTAB / block BiCGGR (Section 3 of
-// arXiv:0903.4936): L x L Gram matrices R~_0^H V, column dot products for
-// the traces Tr(W^H R) and the residual norms, fused block combinations
-// with an L x L coefficient matrix (S_k alpha_k, U_k gamma_k, ...), and the
-// FP64 L x L solves.
+// arXiv:0903.4936): column dot products for the traces Tr(W^H R) and the
+// residual norms, the finishing sums of every reduction, block updates of
+// FP16 blocks, sums into FP64, seeded blocks, the L x L solves of any size
+// (FP64), and the launchers.  Gram matrices and the updates of FP64 / FP32
+// blocks: rows.cu (systems of up to 12 columns) and wide.cu.
 //
 // All block kernels are block-diagonal over a partition of the columns into
 // independent systems (one system for a plain solve).  Blocks are in the
-// RHS-interleaved pair layout of bk_common.cuh: every column of a site is
-// in one row, so a thread block that takes a run of whole systems and a
-// few sites finds each system's columns side by side and combines them in
-// shared memory (no column is read twice from DRAM).
+// RHS-interleaved pair layout of bk_common.cuh.
 #include <algorithm>
 #include <cstring>
 
@@ -38,37 +36,20 @@ SysPart single_part(int L) { return make_part(1, &L); }
 
 namespace {
 
-// pairs of a tile of the any-size update kernel
+// pairs of a tile of the any-size FP16 update
 constexpr int TILE_MAXP = 64;
 
-// Site chunks of the reductions and updates: grid.y, independent of the
-// tiles so that per-chunk partial sums have a fixed row count for a lattice.
+// row chunks (partial-sum rows) of the column dots, at most
 constexpr int MAX_CHUNKS = 304;  // 2 per SM of 152
-
-// element store (FP32 / FP64 pair layouts)
-template <int P>
-__device__ __forceinline__ void store_elem(const Field& f, int n, int k, int p, typename Prec<P>::pair re,
-                                           typename Prec<P>::pair im) {
-    if constexpr (P == BK_FP64) {
-        double2* q = (double2*)f.data + 2 * (((size_t)n * 12 + k) * f.np + p);
-        q[0] = re;
-        q[1] = im;
-    } else {
-        static_assert(P == BK_FP32, "element stores are for FP32 / FP64 blocks");
-        ((float4*)f.data)[((size_t)n * 12 + k) * f.np + p] = make_float4(re.x, re.y, im.x, im.y);
-    }
-}
 
 // ---------------------------------------------------------------- warp tiles
 //
-// The small-system kernels (systems of at most 12 columns, so at most 6
-// pairs) give every warp a run of whole active systems of at most 32 pairs,
-// one pair per lane, and let the warps of a block take different sites.  A
-// lane loads only its own pair of each operand (a warp reads contiguous
-// 16-byte elements, and no element is read twice); the pairs of the other
-// columns of its system come from the lanes that hold them by register
-// shuffles.  No shared-memory round trip, no barrier, no dependence between
-// the warps inside the site loop.
+// The FP16 update of systems of at most 12 columns gives every warp a run of
+// whole active systems of at most 32 pairs, one pair per lane, and lets the
+// warps of a block take different sites (a site's 12 components stay with one
+// lane, which forms the scale of the stored column).  A lane loads only its own
+// pair of each operand; the pairs of the other columns of its system come from
+// the lanes that hold them by register shuffles.
 constexpr int WT_PAIRS = 32;
 
 struct WLane {
@@ -275,36 +256,30 @@ __global__ void __launch_bounds__(FIN_E * FIN_ROWS) k_coldot_finish(const double
 //   X_j      += xa Xin_j + xm matpart_j          (X in FP64 for FP64 blocks, else FP32)
 // coefficient value = mult * (ptr ? ptr[s] : 1), ptr complex FP64 per system.
 //
-// Systems of at most 12 columns run in k_genop_w (warp tiles, below);
-// larger ones in k_genop: SR site rows x 64 pair slots over a tile of whole
-// systems, grid (tiles, site chunks).  Each thread forms the comb columns of
-// its system pair by pair (the system's threads share the reads through L1)
-// and combines them with its two columns of M, read through the read-only
-// path, then writes its pair of Y and X.  Optionally the squared norms of
-// the Y columns are summed per chunk (the residual norms of the stopping
-// rule come with the R update).
+// FP64 and FP32 blocks: k_update_r (rows.cu), k_update_t (wide.cu).  FP16 blocks
+// here: systems of at most 12 columns in k_genop_w (warp tiles, below), larger
+// ones in k_genop: SR site rows x 64 pair slots over a tile of whole systems,
+// grid (tiles, site chunks, 64 pairs of a wider system).  Each thread forms the
+// comb columns of its system pair by pair (the system's threads share the reads
+// through L1) and combines them with its two columns of M, read through the
+// read-only path, then writes its pair of Y and X.  Optionally the squared
+// norms of the Y columns are summed per chunk.
 
-// FP16 elements come with a per-(site, pair) scale: load_scaled applies it.
-template <int P>
-__device__ __forceinline__ CxPair<typename Prec<P>::pair> load_scaled(const Field& f, int n, int k, int q,
-                                                                       typename Prec<P>::pair sc) {
-    CxPair<typename Prec<P>::pair> v;
-    load_elem<P>(f, n, k, q, v.re, v.im);
-    if constexpr (P == BK_FP16) {
-        v.re = pmul(v.re, sc);
-        v.im = pmul(v.im, sc);
-    }
+// element with its (site, pair) scale applied
+__device__ __forceinline__ CxPair<float2> load_scaled(const Field& f, int n, int k, int q, float2 sc) {
+    CxPair<float2> v;
+    load_elem<BK_FP16>(f, n, k, q, v.re, v.im);
+    v.re = pmul(v.re, sc);
+    v.im = pmul(v.im, sc);
     return v;
 }
 
-template <int P, int SR>
+template <int SR>
 __global__ void __launch_bounds__(256) k_genop(const __grid_constant__ GenOp g, PTiles tl, int V, int nchunk,
                                                int ncols) {
-    using R = typename Prec<P>::real;
-    using R2 = typename Prec<P>::pair;
-    constexpr int XP = P == BK_FP64 ? BK_FP64 : BK_FP32;
-    using XR = typename Prec<XP>::real;
-    using X2 = typename Prec<XP>::pair;
+    constexpr int P = BK_FP16, XP = BK_FP32;
+    using R = float;
+    using R2 = float2;
     __shared__ double2 ynred[SR][TILE_MAXP];
     const int tx = threadIdx.x, t = tx + (int)blockIdx.z * TILE_MAXP, r = threadIdx.y;  // systems wider than a tile: grid.z
     const int tile = blockIdx.x, chunk = blockIdx.y;
@@ -332,9 +307,7 @@ __global__ void __launch_bounds__(256) k_genop(const __grid_constant__ GenOp g, 
     R2 ym2;
     ym2.x = (R)g.ym;
     ym2.y = (R)g.ym;
-    X2 xm2;
-    xm2.x = (XR)g.xm;
-    xm2.y = (XR)g.xm;
+    const R2 xm2 = bcast((R)g.xm);
     double yn[2] = {0.0, 0.0};
     const int iters = (V + SR * nchunk - 1) / (SR * nchunk);
     for (int it = 0; it < iters; ++it) {
@@ -345,7 +318,7 @@ __global__ void __launch_bounds__(256) k_genop(const __grid_constant__ GenOp g, 
         for (int e = 0; e < GENOP_MAXE; ++e)
             if (e < g.ne) esc[e] = pair_scale<P>(g.E[e], n, q);
         const R2 xsc = g.hasX ? pair_scale<P>(g.Xin, n, q) : pzero<R2>();
-        R2 yr[P == BK_FP16 ? 12 : 1], yi[P == BK_FP16 ? 12 : 1];
+        R2 yr[12], yi[12];
         R sa = R(0), sb = R(0);
 #pragma unroll 2
         for (int k = 0; k < 12; ++k) {
@@ -364,7 +337,7 @@ __global__ void __launch_bounds__(256) k_genop(const __grid_constant__ GenOp g, 
 #pragma unroll
                     for (int u = 0; u < GENOP_MAXMI; ++u)
                         if (u < g.nmi)
-                            cpair_mac<R, R2>(c, ma[u], load_scaled<P>(g.Mi[u], n, k, qs + ip,
+                            cpair_mac<R, R2>(c, ma[u], load_scaled(g.Mi[u], n, k, qs + ip,
                                                                       pair_scale<P>(g.Mi[u], n, qs + ip)));
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
@@ -408,40 +381,25 @@ __global__ void __launch_bounds__(256) k_genop(const __grid_constant__ GenOp g, 
                 y.im = pmul(ym2, mp.im);
 #pragma unroll
                 for (int e = 0; e < GENOP_MAXE; ++e)
-                    if (e < g.ne) cpair_mac<R, R2>(y, ea[e], load_scaled<P>(g.E[e], n, k, q, esc[e]));
+                    if (e < g.ne) cpair_mac<R, R2>(y, ea[e], load_scaled(g.E[e], n, k, q, esc[e]));
                 if (g.ynorm) {
                     sa = fma(y.re.x, y.re.x, sa);
                     sa = fma(y.im.x, y.im.x, sa);
                     sb = fma(y.re.y, y.re.y, sb);
                     sb = fma(y.im.y, y.im.y, sb);
                 }
-                if constexpr (P == BK_FP16) {
-                    yr[k] = y.re;
-                    yi[k] = y.im;
-                } else {
-                    store_elem<P>(g.Y, n, k, q, y.re, y.im);
-                }
+                yr[k] = y.re;
+                yi[k] = y.im;
             }
             if (g.hasX) {
-                const CxPair<R2> v = load_scaled<P>(g.Xin, n, k, q, xsc);
-                CxPair<X2> x, vx;
-                load_elem<XP>(g.X, n, k, q, x.re, x.im);
-                vx.re.x = v.re.x;
-                vx.re.y = v.re.y;
-                vx.im.x = v.im.x;
-                vx.im.y = v.im.y;
-                cpair_mac<XR, X2>(x, mk((XR)xa.r, (XR)xa.i), vx);
-                X2 mr, mi;
-                mr.x = mp.re.x;
-                mr.y = mp.re.y;
-                mi.x = mp.im.x;
-                mi.y = mp.im.y;
-                store_elem<XP>(g.X, n, k, q, pfma(xm2, mr, x.re), pfma(xm2, mi, x.im));
+                const CxPair<R2> v = load_scaled(g.Xin, n, k, q, xsc);
+                const size_t e = ((size_t)n * 12 + k) * g.X.np + q;
+                CxPair<R2> x = load_at<XP>(g.X, e);
+                cpair_mac<R, R2>(x, xa, v);
+                store_at<XP>(g.X, e, pfma(xm2, mp.re, x.re), pfma(xm2, mp.im, x.im));
             }
         }
-        if constexpr (P == BK_FP16) {
-            if (g.hasY) store_pair<P>(g.Y, n, q, yr, yi);
-        }
+        if (g.hasY) store_pair<P>(g.Y, n, q, yr, yi);
         yn[0] += (double)sa;
         yn[1] += (double)sb;
     }
@@ -460,16 +418,12 @@ __global__ void __launch_bounds__(256) k_genop(const __grid_constant__ GenOp g, 
     }
 }
 
-// Update kernel over warp tiles (systems of at most MAXL <= 12 columns).
-// Each lane forms comb = sum_u ma_u Mi_u for its own pair, takes the comb
-// pairs of its system's other lanes by shuffles and combines them with its
-// two columns of M (registers), then adds the elementwise terms and writes
-// its pair of Y and X.  The loads of UK spinor components are issued before
-// any of their arithmetic and stores; the operands read through the
-// read-only path are never written by another thread of the launch.  NMI,
-// NE and HX fix the operand counts of the hot updates at compile time (-1:
-// taken from the GenOp); every operand has the layout's pair count np, so
-// one element offset serves them all.
+// FP16 update over warp tiles (systems of at most MAXL <= 12 columns).  Each
+// lane forms comb = sum_u ma_u Mi_u for its own pair, takes the comb pairs of
+// its system's other lanes by shuffles and combines them with its two columns
+// of M (registers), then adds the elementwise terms and writes its pair of Y
+// and X.  Every operand has the layout's pair count np, so one element offset
+// serves them all.
 template <int MAXL>
 __global__ void __launch_bounds__(GW_WARPS * 32) k_genop_w(const __grid_constant__ GenOp g, PTiles wt, int V,
                                                           int nchunk, int ncols, int np) {
@@ -1150,7 +1104,7 @@ bk_status launch_genop(int prec, const GenOp& g, int V, cudaStream_t st, bool* y
         constexpr int SR = 4;
         int widest = 1;
         for (int i = 0; i < tl.n; ++i) widest = std::max(widest, tl.np[i]);
-        k_genop<BK_FP16, SR><<<dim3(tl.n, nchunk, (widest + TILE_MAXP - 1) / TILE_MAXP), dim3(TILE_MAXP, SR), 0, st>>>(
+        k_genop<SR><<<dim3(tl.n, nchunk, (widest + TILE_MAXP - 1) / TILE_MAXP), dim3(TILE_MAXP, SR), 0, st>>>(
             g, tl, V, nchunk, ncols);
     }
     BK_CUDA_TRY(cudaGetLastError());

@@ -194,8 +194,9 @@ constexpr int ROWS_MAXL = 12;
 // per 4 warp steps, so that a small lattice still fills every SM's FP64 pipe
 // (4^4, 12 columns: 615 steps).  FP32 / FP16: a chunk per 64 steps, 8 a warp,
 // since there a block's fixed costs (FP64 conversions, the finishing sums)
-// outweigh a few more rows.  At most the blocks that are resident at once
-// (FP64: 1 an SM, else 2), over all tiles: a 153rd block would double the time.
+// outweigh a few more rows.  Up to two tiles (FP64) or four: at most the blocks
+// that are resident at once (FP64: 1 an SM, else 2), since a 153rd block would
+// double the time; more tiles take several waves anyway, of 76 chunks each.
 inline int gram_row_chunks(int prec, int V, const PTiles& t) {
     int spw = 32;
     for (int i = 0; i < t.n; ++i) spw = std::min(spw, 32 / std::max(1, t.np[i]));

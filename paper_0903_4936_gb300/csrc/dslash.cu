@@ -183,30 +183,19 @@ __device__ __forceinline__ void reconstruct_colour(int a, float2 w0r, float2 w0i
     }
 }
 
-// Compact complex table entries (gauge.cu), in global or in shared memory.  All
-// lanes of a site read the same 8 bytes, and the pairs {u, u} of the packed
-// arithmetic are formed by moves: a 64-bit shared read takes two passes of the
-// load pipe and a 128-bit one four, whatever it broadcasts, so 72 bytes a link
-// cost a third of links stored as pairs (216 bytes).
+// Compact complex table entries (gauge.cu).  All lanes of a site read the same
+// 8 bytes, and the pairs {u, u} of the packed arithmetic are formed by moves.
 struct GTab {
     const float2* p;
     __device__ __forceinline__ float2 at(int e) const { return __ldg(p + e); }
-};
-struct STab {
-    unsigned a;
-    __device__ __forceinline__ float2 at(int e) const {
-        float2 v;
-        asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a + 8 * e));
-        return v;
-    }
 };
 __device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
 
 // Product with the link U (forward) or U^+ (backward) and reconstruction, fused
 // row by row: output colour i of both half-spinor vectors is formed and added
 // at once, so only one row of the link and one colour of w are live.
-template <int MU, int S, typename T>
-__device__ __forceinline__ void link_mul_add(T u, const Hop& h, float2 nk, float2 pk, float2 (&ar)[12],
+template <int MU, int S>
+__device__ __forceinline__ void link_mul_add(GTab u, const Hop& h, float2 nk, float2 pk, float2 (&ar)[12],
                                              float2 (&ai)[12]) {
     constexpr bool DAG = S > 0;
 #pragma unroll
@@ -235,8 +224,7 @@ __device__ __forceinline__ void link_mul_add(T u, const Hop& h, float2 nk, float
 
 // y = H_b v for chiral block b (6 diagonal entries, then 15 complex ones below
 // the diagonal) of a compact site term
-template <typename T>
-__device__ __forceinline__ void herm6_pair(T c, int b, const float2 (&vr)[6], const float2 (&vi)[6], float2 (&yr)[6],
+__device__ __forceinline__ void herm6_pair(GTab c, int b, const float2 (&vr)[6], const float2 (&vi)[6], float2 (&yr)[6],
                                            float2 (&yi)[6]) {
 #pragma unroll
     for (int i = 0; i < 6; i += 2) {
@@ -267,8 +255,8 @@ __device__ __forceinline__ void herm6_pair(T c, int b, const float2 (&vr)[6], co
 
 // The site term on (ar, ai) in place: CLOVER: out = q - kappa C q (nk =
 // {-kappa}); else out = A^-1 q.  The blocks act on u + l and u - l.
-template <bool CLOVER, typename T>
-__device__ __forceinline__ void site_term(T c, float2 nk, float2 (&ar)[12], float2 (&ai)[12]) {
+template <bool CLOVER>
+__device__ __forceinline__ void site_term(GTab c, float2 nk, float2 (&ar)[12], float2 (&ai)[12]) {
     float2 vr[2][6], vi[2][6];
 #pragma unroll
     for (int k = 0; k < 6; ++k) {

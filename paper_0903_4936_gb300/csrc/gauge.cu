@@ -5,7 +5,7 @@
 //    one matrix element for 32 consecutive sites issues one coalesced
 //    transaction (the FP64 operator takes one column per thread);
 //  * FP32: per site its four links side by side, each 9 complex elements and
-//    one of padding (80 bytes: a multiple of 16 for the tiled operator's copies).
+//    one of padding (80 bytes: every link starts on a 16-byte boundary).
 //
 // Clover: the FP64 copy is [36][site] double2 (72 reals per site); the FP32
 // copy is the 72 reals of a site side by side.  The site term C(n) = c_SW sum_{mu,nu} (i/2)
@@ -75,21 +75,6 @@ __device__ __forceinline__ M3 mdm(const M3& a, const M3& b) {
             cx<double> s = mk(0.0, 0.0);
 #pragma unroll
             for (int k = 0; k < 3; ++k) cjmac(s, a.m[k][i], b.m[k][j]);
-            r.m[i][j] = s;
-        }
-    return r;
-}
-
-// a^dag * b^dag
-__device__ __forceinline__ M3 mdd(const M3& a, const M3& b) {
-    M3 r;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            cx<double> s = mk(0.0, 0.0);
-#pragma unroll
-            for (int k = 0; k < 3; ++k) cmac(s, cj(a.m[k][i]), cj(b.m[j][k]));
             r.m[i][j] = s;
         }
     return r;
