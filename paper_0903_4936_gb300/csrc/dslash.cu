@@ -619,10 +619,8 @@ __device__ __forceinline__ void herm6_rows(const double2* __restrict__ C, int V,
 // takes the two hops of direction t and three rows of one chiral block of the
 // clover term, and finishes spin t.  An SM's scheduler starts an FP64
 // instruction of a warp every 64 cycles, so one thread per site and column
-// (about 1000 of them) needs 33 us however few there are (4^4, 12 columns: 46
-// us a launch, 18 in this form); a quarter of that each, on four times the
-// warps, is faster while they do not fill the chip's
-// 608 schedulers about twice (see dslash_col_impl).
+// takes 40 us however few there are; a quarter of that each, on four times the
+// warps, is faster while they do not fill the chip (see split_over_warps).
 __global__ void __launch_bounds__(128) k_dslash_col4(const __grid_constant__ DColArgs<BK_FP64> a) {
     __shared__ double hs[4][24][32], ys[4][6][32];
     const int t = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -741,6 +739,15 @@ bk_status dslash_pair_impl(const DslashOp& op, cudaStream_t st) {
     return BK_OK;
 }
 
+// Which FP64 form: n rounds of one 32-item block per SM take the split form 11 us
+// each; the other form is as slow as the fullest scheduler, which steps after 4,
+// 6 and 8 warps an SM.  Measured (us, split / one thread each): n = 1 14 / 40, 2
+// 24 / 40, 3 35 / 42, 4 46 / 42, 5 57 / 63, 6 67 / 63, 7 79 / 80.
+bool split_over_warps(long long items) {
+    const long long n = ((items + 31) / 32 + 151) / 152;
+    return n <= 3 || n == 5 || n == 7;
+}
+
 // Threads per block of the one-column-per-thread kernels.  Their FP64 pipe
 // works at full rate with few warps, so what matters is that every scheduler
 // has the same number: single-warp blocks up to 16 warps a scheduler, two-warp
@@ -765,7 +772,7 @@ bk_status dslash_col_impl(const DslashOp& op, cudaStream_t st) {
         for (int j = 0; j < n; ++j) a.kappa[j] = op.kappa[c0 + j];
         const long long items = (long long)op.V * n;
         if constexpr (P == BK_FP64) {
-            if (items <= 608LL * 2 * 32 && op.x.np == op.y.np && (!op.residual || op.b.np == op.x.np)) {
+            if (split_over_warps(items) && op.x.np == op.y.np && (!op.residual || op.b.np == op.x.np)) {
                 k_dslash_col4<<<(unsigned)((items + 31) / 32), 128, 0, st>>>(a);
                 BK_CUDA_TRY(cudaGetLastError());
                 continue;

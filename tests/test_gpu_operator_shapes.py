@@ -101,3 +101,15 @@ def test_schur_block_sizes(prec, dims, L):
     for j in (0, L - 1):
         assert np.all(Y[j][odd] == 0)
         assert _rel(Y[j:j + 1], evenodd.schur_apply(U, X[j:j + 1], kap[j], 1.0)) < SCHUR_TOL[prec]
+
+
+# 32 columns of one site to a block: 456 blocks fill 152 SMs three times; the split over four warps and the form with
+# one thread each take turns above that
+@pytest.mark.parametrize("L", [57, 58, 77, 96, 128, 140])
+def test_fp64_operator_forms(L):
+    dims = (4, 4, 4, 4)
+    lat, U = _lat(dims, 51 + L)
+    X = synth.gaussian_sources(dims, L, 9)
+    kap = np.linspace(0.10, 0.13, L)
+    Y = lat.dslash(torch.from_numpy(X).cuda(), list(kap), "fp64").cpu().numpy()
+    assert _rel(Y, dirac.apply_dirac(U, X, kap, 1.0)) < 1e-13
