@@ -791,13 +791,18 @@ bk_status dslash_col_impl(const DslashOp& op, cudaStream_t st) {
 // dcol[j] (dcol == nullptr: dbase + j), through a shared-memory tile of CT_S
 // sites x CT_C columns: a canonical column is contiguous along (site,
 // component), a device row along the columns, so one side of a direct copy
-// touches a separate line per lane (12 columns, 16^3x32, FP64: 103 us in and
-// 118 out, of 88 at the memory rate; operator with both conversions 3428 us,
-// now 3330).
+// touches a separate line per lane.  Loads issued one by one and half of the
+// device-side lanes idle made this slower than the direct copy where L2 holds
+// the blocks (8^3x16, 64 columns, FP32: direct 34 us, tile then 42, tile now
+// 26; 12^3x24, 24 columns 60, 76, 50; 4^4, 16 columns 3.1, 4.6, 3.2).
 constexpr int CT_S = 8, CT_C = 16, CT_R = CT_S * 12;
 
 __device__ __forceinline__ int dev_col(const int* dcol, int dbase, int j) { return dcol ? __ldg(dcol + j) : dbase + j; }
 
+// A thread issues its loads before their first use.  On the device side 16 bytes
+// of a pair of the layout are a lane's access (FP32: the pair; FP64: its real or
+// its imaginary parts), for the two neighbouring columns of the tile that the
+// lane owns, whichever of them the pair starts at.
 template <int P, bool PACK>
 __global__ void __launch_bounds__(256) k_convert(double2* __restrict__ canon, int ncan, const int* __restrict__ dcol,
                                                  int dbase, Field f) {
@@ -805,75 +810,92 @@ __global__ void __launch_bounds__(256) k_convert(double2* __restrict__ canon, in
     const int j0 = blockIdx.y * CT_C, nj = min(CT_C, ncan - j0);
     const int n0 = blockIdx.x * CT_S, nr = 12 * min(CT_S, f.V - n0);
     const int t = threadIdx.x;
-    auto canonical = [&]() {  // rows fastest
-        for (int e = t; e < nj * CT_R; e += 256) {
-            const int j = e / CT_R, r = e - j * CT_R;
-            if (r >= nr) continue;
+    // canonical side, rows fastest
+    constexpr int NU = CT_R * CT_C / 256;
+    auto canonical = [&](bool load) {
+        double2 v[NU];
+#pragma unroll
+        for (int u = 0; u < NU; ++u) {
+            if (256 * u >= nj * CT_R) break;
+            const int e = t + 256 * u, j = e / CT_R, r = e - j * CT_R;
             double2* q = canon + ((size_t)(j0 + j) * f.V + n0) * 12 + r;
-            if (PACK) tile[r][j] = *q;
-            else *q = tile[r][j];
-        }
-    };
-    auto device = [&]() {  // columns fastest
-        int cw = CT_C;  // columns side by side: a power of two that covers the tile's
-        while (cw / 2 >= nj) cw /= 2;
-        const int j = t & (cw - 1);
-        if (j >= nj) return;
-        const int c = dev_col(dcol, dbase, j0 + j), half = c & 1;
-        // both columns of a pair in the tile side by side: the even one's thread takes them
-        const bool both = !half && j + 1 < nj && dev_col(dcol, dbase, j0 + j + 1) == c + 1;
-        if (half && j > 0 && dev_col(dcol, dbase, j0 + j - 1) == c - 1) return;
-        for (int r = t / cw; r < nr; r += 256 / cw) {
-            const size_t e = ((size_t)n0 * 12 + r) * f.np + (c >> 1);
-            if constexpr (P == BK_FP64) {
-                double2* q = (double2*)f.data + 2 * e;
-                if (both) {
-                    if (PACK) {
-                        const double2 a = tile[r][j], b = tile[r][j + 1];
-                        q[0] = make_double2(a.x, b.x);
-                        q[1] = make_double2(a.y, b.y);
-                    } else {
-                        const double2 re = q[0], im = q[1];
-                        tile[r][j] = make_double2(re.x, im.x);
-                        tile[r][j + 1] = make_double2(re.y, im.y);
-                    }
-                } else {
-                    double* s = (double*)q + half;
-                    if (PACK) {
-                        s[0] = tile[r][j].x;
-                        s[2] = tile[r][j].y;
-                    } else {
-                        tile[r][j] = make_double2(s[0], s[2]);
-                    }
-                }
-            } else {
-                float4* q = (float4*)f.data + e;
-                if (both) {
-                    if (PACK) {
-                        const double2 a = tile[r][j], b = tile[r][j + 1];
-                        *q = make_float4(d2f(a.x), d2f(b.x), d2f(a.y), d2f(b.y));
-                    } else {
-                        const float4 v = *q;
-                        tile[r][j] = make_double2(f2d(v.x), f2d(v.z));
-                        tile[r][j + 1] = make_double2(f2d(v.y), f2d(v.w));
-                    }
-                } else {
-                    float* s = (float*)q + half;
-                    if (PACK) {
-                        s[0] = d2f(tile[r][j].x);
-                        s[2] = d2f(tile[r][j].y);
-                    } else {
-                        tile[r][j] = make_double2(f2d(s[0]), f2d(s[2]));
-                    }
-                }
+            if (j < nj && r < nr) {
+                if (load) v[u] = *q;
+                else *q = tile[r][j];
             }
         }
+        if (load)
+#pragma unroll
+            for (int u = 0; u < NU; ++u) {
+                if (256 * u >= nj * CT_R) break;
+                const int e = t + 256 * u, j = e / CT_R, r = e - j * CT_R;
+                if (j < nj && r < nr) tile[r][j] = v[u];
+            }
     };
-    if (PACK) canonical();
-    else device();
-    __syncthreads();
-    if (PACK) device();
-    else canonical();
+    if (PACK) canonical(true);
+    // device side, columns fastest: a power of two of column pairs side by side
+    constexpr int LP = P == BK_FP64 ? 2 : 1;  // lanes a pair
+    using R = typename Prec<P>::real;
+    int sw = CT_C / 2;
+    while (sw > 1 && sw >= nj) sw /= 2;
+    const int js = 2 * ((t & (sw * LP - 1)) / LP), part = t & (LP - 1), r0 = t / (sw * LP), rstep = 256 / (sw * LP);
+    int col[2], act[2];  // device column; 0: nothing to do here, 1: the column alone, 2: with the next one
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int j = js + h;
+        col[h] = act[h] = 0;
+        if (j >= nj) continue;
+        col[h] = dev_col(dcol, dbase, j0 + j);
+        if (col[h] & 1) act[h] = j > 0 && dev_col(dcol, dbase, j0 + j - 1) == col[h] - 1 ? 0 : 1;
+        else act[h] = j + 1 < nj && dev_col(dcol, dbase, j0 + j + 1) == col[h] + 1 ? 2 : 1;
+    }
+    if (PACK) __syncthreads();
+    constexpr int NR = CT_R / (256 / (CT_C / 2 * LP));  // passes over the rows, at most
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        if (!act[h]) continue;
+        const int j = js + h, half = col[h] & 1;
+        const bool both = act[h] == 2;
+        R* base = (R*)f.data + 4 * ((size_t)n0 * 12 * f.np + (col[h] >> 1)) + 2 * part;
+        R v[NR][4 / LP];
+        if (!PACK)
+#pragma unroll
+            for (int u = 0; u < NR; ++u) {
+                const int r = r0 + u * rstep;
+                const R* q = base + 4 * (size_t)r * f.np;
+                if (r >= nr) break;
+                if constexpr (LP == 2) {
+                    if (both) *(double2*)v[u] = *(const double2*)q;
+                    else v[u][0] = q[half];
+                } else {
+                    if (both) *(float4*)v[u] = *(const float4*)q;
+                    else v[u][0] = q[half], v[u][2] = q[2 + half];
+                }
+            }
+#pragma unroll
+        for (int u = 0; u < NR; ++u) {
+            const int r = r0 + u * rstep;
+            if (r >= nr) break;
+            R* q = base + 4 * (size_t)r * f.np;
+            double2 *a = &tile[r][j], *b = both ? a + 1 : a;
+            if constexpr (LP == 2) {  // part 0: real parts, 1: imaginary parts
+                double *x = (double*)a + part, *y = (double*)b + part;
+                if (PACK && both) *(double2*)q = make_double2(*x, *y);
+                else if (PACK) q[half] = *x;
+                else *x = v[u][0];
+                if (!PACK && both) *y = v[u][1];
+            } else {
+                if (PACK && both) *(float4*)q = make_float4(d2f(a->x), d2f(b->x), d2f(a->y), d2f(b->y));
+                else if (PACK) q[half] = d2f(a->x), q[2 + half] = d2f(a->y);
+                else *a = make_double2(f2d(v[u][0]), f2d(v[u][2]));
+                if (!PACK && both) *b = make_double2(f2d(v[u][1]), f2d(v[u][3]));
+            }
+        }
+    }
+    if (!PACK) {
+        __syncthreads();
+        canonical(false);
+    }
 }
 
 // FP16: the same with one thread per (canonical column, site), which forms or

@@ -113,3 +113,21 @@ def test_fp64_operator_forms(L):
     kap = np.linspace(0.10, 0.13, L)
     Y = lat.dslash(torch.from_numpy(X).cuda(), list(kap), "fp64").cpu().numpy()
     assert _rel(Y, dirac.apply_dirac(U, X, kap, 1.0)) < 1e-13
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("L", [1, 2, 3, 4, 8, 9, 15, 16, 17, 18, 31, 33])
+def test_layout_conversions(prec, L):
+    """Canonical to device layout and back: tiles of 8 sites and 16 columns, 90 sites, every column exact."""
+    import paper_0903_4936_gb300 as bk
+    dims, V = (3, 5, 2, 3), 90
+    lat = bk.Lattice(dims)
+    X = synth.gaussian_sources(dims, L, 10)
+    X = X.astype(np.complex64).astype(np.complex128) if prec == "fp32" else X
+    F = lat.pack(torch.from_numpy(X).cuda(), prec)
+    v = F.cpu().numpy().view(np.float64 if prec == "fp64" else np.float32)  # (its size is rounded up)
+    v = v[:V * 12 * ((L + 1) // 2) * 4].reshape(V * 12, (L + 1) // 2, 2, 2)
+    x = X.reshape(L, V * 12)
+    for j in range(L):
+        assert np.array_equal(v[:, j // 2, 0, j % 2], x[j].real) and np.array_equal(v[:, j // 2, 1, j % 2], x[j].imag)
+    assert np.array_equal(lat.unpack(F, L, prec).cpu().numpy(), X)
