@@ -235,28 +235,36 @@ WideWork wide_work(const SysPart& p, int T) {
     return w;
 }
 
-// threads a block: the count that leaves the fewest idle over the systems, of
-// those whose blocks fit the work list (fewer threads a block need more
-// blocks: one system of 1000 columns 245 with 256 threads, 326 with 192)
+// Threads a block: the count, of those whose blocks fit the work list, that
+// leaves the fewest threads idle over the launch; then the one with the fewest
+// blocks a row chunk, since each of them stages the system's rows for itself.
+// A block with few tiles has its rows shared out over slices and ends early.  Up
+// to 8 blocks a chunk all blocks are resident at once, so the longest one is the
+// launch's time (64 columns: 192 threads take 192 tiles and 64 in three slices,
+// 256 take all in one block).
 int wide_threads(const SysPart& p) {
-    int best = 256;
+    int best = 256, fewest = 1 << 30;
     double most = 0.0;
     for (int T = 192; T <= 320; T += 32) {
-        if (wide_work(p, T).n < 0) continue;
-        double use = 0.0, all = 0.0;
+        const int n = wide_work(p, T).n;
+        if (n <= 0) continue;
+        double use = 0.0, sum = 0.0, longest = 0.0;
         for (int s = 0; s < p.nsys; ++s) {
             if (!((p.active >> s) & 1ull)) continue;
             const int nps = (p.L[s] + 1) / 2, side = (nps + 1) / 2;
             for (int t0 = 0; t0 < side * side; t0 += T) {
                 const int nt = std::min(T, side * side - t0);
+                const double time = 1.0 / (T / nt);  // slices share it
                 use += (double)nt / T;               // work in units of full blocks
-                all += (double)nt / (nt * (T / nt));  // blocks' time: slices share it
+                sum += time;
+                longest = std::max(longest, time);
             }
         }
-        const double u = all > 0.0 ? use / all : 0.0;
-        if (u > most + 1e-9) {
-            most = u;
+        const double u = use / (n <= 8 ? n * longest : sum);
+        if (u > most + 1e-9 || (u > most - 1e-9 && n < fewest)) {
+            most = std::max(most, u);
             best = T;
+            fewest = n;
         }
     }
     return best;
