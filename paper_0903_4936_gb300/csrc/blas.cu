@@ -423,16 +423,17 @@ __global__ void __launch_bounds__(256) k_genop(const __grid_constant__ GenOp g, 
 // its system's other lanes by shuffles and combines them with its two columns
 // of M (registers), then adds the elementwise terms and writes its pair of Y
 // and X.  Every operand has the layout's pair count np, so one element offset
-// serves them all.
-template <int MAXL>
+// serves them all.  NMI, NE and HX fix the operand counts of the solvers'
+// updates at compile time.
+template <int MAXL, int NMI, int NE, int HX>
 __global__ void __launch_bounds__(GW_WARPS * 32) k_genop_w(const __grid_constant__ GenOp g, PTiles wt, int V,
                                                           int nchunk, int ncols, int np) {
     constexpr int P = BK_FP16, XP = BK_FP32;
     using R = float;
     using R2 = float2;
-    constexpr int MMI = GENOP_MAXMI, ME = GENOP_MAXE;
-    const int nmi = g.nmi, ne = g.ne;
-    const bool hx = g.hasX != 0;
+    constexpr int MMI = NMI >= 0 ? NMI : GENOP_MAXMI, ME = NE >= 0 ? NE : GENOP_MAXE;
+    const int nmi = NMI >= 0 ? NMI : g.nmi, ne = NE >= 0 ? NE : g.ne;
+    const bool hx = HX >= 0 ? HX != 0 : g.hasX != 0;
     __shared__ double2 ynred[GW_WARPS][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int chunk = blockIdx.y;
@@ -440,7 +441,7 @@ __global__ void __launch_bounds__(GW_WARPS * 32) k_genop_w(const __grid_constant
     const bool act = L.live && !(g.skip && g.skip[L.s]);
     const int s = L.s;
     const bool mat = nmi > 0 && g.M != nullptr && ((g.hasY && g.ym != 0.0) || (hx && g.xm != 0.0));
-    cx<R> ea[ME], ma[MMI], xa = mk(R(0), R(0));
+    cx<R> ea[ME > 0 ? ME : 1], ma[MMI > 0 ? MMI : 1], xa = mk(R(0), R(0));
 #pragma unroll
     for (int e = 0; e < ME; ++e) ea[e] = e < ne ? coef<P>(g.ea[e], g.ea_mult[e], 0, s) : mk(R(0), R(0));
 #pragma unroll
@@ -471,7 +472,7 @@ __global__ void __launch_bounds__(GW_WARPS * 32) k_genop_w(const __grid_constant
     for (int it = 0; it < iters; ++it) {
         const int n = (it * nchunk + chunk) * GW_WARPS + w;
         if (n >= V) break;  // the same for the whole warp
-        R2 msc[MMI], esc[ME], xsc = pzero<R2>();
+        R2 msc[MMI > 0 ? MMI : 1], esc[ME > 0 ? ME : 1], xsc = pzero<R2>();
 #pragma unroll
         for (int u = 0; u < MMI; ++u) msc[u] = act && u < nmi ? pair_scale<P>(g.Mi[u], n, L.q) : pzero<R2>();
 #pragma unroll
@@ -484,7 +485,7 @@ __global__ void __launch_bounds__(GW_WARPS * 32) k_genop_w(const __grid_constant
 #pragma unroll
         for (int k = 0; k < 12; ++k) {
             const size_t e = e0 + (size_t)k * np;
-            CxPair<R2> vm[MMI], ve[ME], vx = cp_zero<R2>(), x = cp_zero<R2>();
+            CxPair<R2> vm[MMI > 0 ? MMI : 1], ve[ME > 0 ? ME : 1], vx = cp_zero<R2>(), x = cp_zero<R2>();
 #pragma unroll
             for (int u = 0; u < MMI; ++u)
                 vm[u] = act && mat && u < nmi ? ldg_at<P>(g.Mi[u], e, msc[u]) : cp_zero<R2>();
@@ -1097,8 +1098,24 @@ bk_status launch_genop(int prec, const GenOp& g, int V, cudaStream_t st, bool* y
     } else if (maxL <= ROWS_MAXL) {
         const PTiles wt = make_ptiles(g.p, WT_PAIRS);
         const dim3 grid(wt.n, nchunk);
-        if (maxL <= 6) k_genop_w<6><<<grid, GW_WARPS * 32, 0, st>>>(g, wt, V, nchunk, ncols, np);
-        else k_genop_w<12><<<grid, GW_WARPS * 32, 0, st>>>(g, wt, V, nchunk, ncols, np);
+        const bool h = g.hasX != 0;
+#define BK_GW(ML, NM, NE, HX) k_genop_w<ML, NM, NE, HX><<<grid, GW_WARPS * 32, 0, st>>>(g, wt, V, nchunk, ncols, np)
+        // the updates of the two methods, then any other combination
+#define BK_GWS(ML)                                                \
+    if (g.nmi == 1 && g.ne == 0 && !h) BK_GW(ML, 1, 0, 0);        \
+    else if (g.nmi == 1 && g.ne == 1 && !h) BK_GW(ML, 1, 1, 0);   \
+    else if (g.nmi == 1 && g.ne == 2 && h) BK_GW(ML, 1, 2, 1);    \
+    else if (g.nmi == 2 && g.ne == 1 && !h) BK_GW(ML, 2, 1, 0);   \
+    else if (g.nmi == 2 && g.ne == 0 && h) BK_GW(ML, 2, 0, 1);    \
+    else if (g.nmi == 0 && g.ne == 3 && !h) BK_GW(ML, 0, 3, 0);   \
+    else BK_GW(ML, -1, -1, -1);
+        if (maxL <= 6) {
+            BK_GWS(6)
+        } else {
+            BK_GWS(12)
+        }
+#undef BK_GWS
+#undef BK_GW
     } else {
         const PTiles tl = make_ptiles(g.p, TILE_MAXP);
         constexpr int SR = 4;
