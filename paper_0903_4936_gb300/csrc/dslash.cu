@@ -15,15 +15,16 @@
 // x - kappa C x needs x(n) only once); each of the eight hops then adds -kappa
 // times its term directly.
 //
-// What bounds it: the rows' eight-fold fetches from L2, 10 TB/s of L2-to-SM
-// traffic (16^3x32, 30 columns: 3.0 GB in 280 us).  Before, links and clover
+// What bounds it (16^3x32, 30 columns, 281 us): the load pipe of L1, 79 % busy,
+// with the 15 warps an SM that registers allow waiting for it 57 % of their
+// time; L2 is 46 % busy (2.8 GB to the SMs, the rows about seven times), DRAM 37
+// %, issue 34 %.  A row element takes four passes of that pipe per warp and load,
+// a link or clover entry one per site in the warp.  Before, links and clover
 // were stored as the duplicated pairs (224 and 816 bytes) and took 216 loads a
-// thread, which with staging copies through shared memory kept the load/store
-// pipe 74 % busy: 404 us there (24^3x48, 96 columns 5080 us, now 4060; FP16
-// 12x10x14x18, 13 columns 51, now 34).  A form with the rows staged by bulk
-// copies (cp.async.bulk, a producer warp, 2x2x2 site tiles sharing their rows,
-// 5 fetches a site instead of 8) took 306 us: its producer and 128-register
-// workers, not L2, were the limit.
+// thread: 404 us there (24^3x48, 96 columns 5080 us, now 4060; FP16 12x10x14x18,
+// 13 columns 51, now 34).  A form with the rows staged by bulk copies
+// (cp.async.bulk, a producer warp, 2x2x2 site tiles sharing their rows, 5
+// fetches a site instead of 8) took 306 us.
 //
 // FP64 / double-float (k_dslash_col): one thread per site and column, FP64
 // links and clover in [element][site] order (the FP64 pipe, not memory,

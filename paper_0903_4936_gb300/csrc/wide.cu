@@ -9,7 +9,7 @@
 // matrix, or 4 rows x 4 columns of an update, and needs 4 (8) 16-byte reads
 // for 32 (64) packed multiply-adds.
 //
-// 16^3x32, 48 columns, FP32: Gram 938 us and update 863 us; 1930 and 16100
+// 16^3x32, 48 columns, FP32: Gram 887 us and update 845 us; 1930 and 16100
 // before, when the update read M and the partner columns through L1 for every
 // product (at the FP32 rate each is 370 us).
 #include <cstring>
