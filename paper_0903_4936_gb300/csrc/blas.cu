@@ -900,9 +900,12 @@ __global__ void __launch_bounds__(256) k_chol_inv(const double2* __restrict__ S,
     for (int k = 0; k < n; ++k) {
         if (tid == 0) {
             double d = A[k * n + k].r;
-            const double low = floor * n * S[off + k * n + k].x;
-            if (low > 0.0 && d <= low && fabs(d) > CHOL_EXACT / (floor * n) * low) d = low;
-            if (!(d > (floor > 0.0 ? 0.0 : 1e-14 * dmax)) || !isfinite(d)) bad = 1;
+            const double low = floor > 0.0 ? floor * n * S[off + k * n + k].x : 1e-14 * dmax;
+            if (!(d > low)) {  // with a floor: that, unless the pivot is zero to FP64 rounding
+                if (floor > 0.0 && low > 0.0 && fabs(d) > CHOL_EXACT / (floor * n) * low) d = low;
+                else bad = 1;
+            }
+            if (!isfinite(d)) bad = 1;
             else A[k * n + k] = mk(sqrt(d), 0.0);
         }
         __syncthreads();

@@ -450,3 +450,16 @@ def test_fp32_blocks_keep_the_fp64_iteration_count(c1, source, anchor):
         total += info["iterations"]
         want += 1.5 * ref["iterations"] + 5
     assert total <= want
+
+
+@pytest.mark.parametrize("L", [5, 14])
+def test_fp32_equal_sources_break_down(c1, L):
+    """Equal right-hand sides give P^H P a pivot of FP64 rounding: the basis is left alone, small (up to 12 columns)
+    and general Cholesky alike, and the singular L x L system is reported."""
+    dims, lat, U, B, Xd, A = c1
+    Bd = synth.gaussian_sources(dims, L, 43)
+    Bd[L - 1] = Bd[1]
+    X, info = lat.block_solve(torch.from_numpy(Bd).cuda(), 0.12, method="bicgstab", prec="fp32", tol=1e-10,
+                              maxiter=300, raise_on_fail=False)
+    assert info["status"] == "BK_ERR_BREAKDOWN" and info["breakdown"] == 1
+    assert np.all(np.isfinite(X.cpu().numpy()))
