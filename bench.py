@@ -528,7 +528,7 @@ def gb300_arm(args, wl, rank, world, local_rank):
         # the plain FP64 block BiCGGR at the same split: precision alone.  One
         # batched solve per case (all cases at once would need seven FP64
         # blocks of every column beside the benchmark's buffers); a short
-        # untimed solve first tunes the FP64 operator's launch shape.
+        # untimed solve first allocates the workspace.
         tot, its, first = 0.0, [], None
         for ci, c in enumerate(cases):
             idx = [si for si in range(len(L_s)) if owner[si] == ci]

@@ -55,7 +55,7 @@ def main(argv=None) -> None:
         sp = "fp64" if p == "df64" else p
         fields[p] = (lat.pack(X, sp), lat.empty_field(L, sp))
     del X
-    for p, (F, Y) in fields.items():  # warm-up (and launch-shape tuning)
+    for p, (F, Y) in fields.items():  # warm-up
         for _ in range(3):
             lat.dslash_dev(F, L, args.kappa, p, out=Y)
     torch.cuda.synchronize()
